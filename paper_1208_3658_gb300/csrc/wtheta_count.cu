@@ -172,6 +172,10 @@ __device__ __forceinline__ float4 sentinel32(int tag, long long k) {
     return make_float4(sign * kSentinel * (float)(k + 1), kSentinel * (float)tag, 0.f, 0.f);
 }
 
+__device__ __forceinline__ bool is_sentinel(const float4& q) {
+    return q.x * q.x + q.y * q.y + q.z * q.z > 4.f;
+}
+
 // RA/Dec degrees -> FP64 unit vectors (SoA with stride xyz_stride).
 __global__ void k_radec_to_xyz(const double* __restrict__ rd, long long n,
                                double* __restrict__ xyz, long long xyz_stride) {
@@ -404,14 +408,84 @@ __global__ void __launch_bounds__(64) k_joint_keys(const double* __restrict__ a,
     }
 }
 
+// One chunk of 32 consecutive positions of the spatial order, one point per
+// lane (q its FP32 copy, (px, py, pz) its FP64 one): the chunk's bounding
+// sphere and the points' coordinates relative to the sphere's centre c.
+//   - Sphere: centre = the FP32 mean of the chunk's points, radius = the
+//     largest FP32 distance of a point from it, enlarged by a relative 1e-6
+//     for the few roundings of that arithmetic.
+//   - Local coordinates b' = fl32(b - c), from the FP64 points: the rounding is
+//     relative to |b'|, so a chunk's own geometry is kept to 2^-24 of its size.
+//   - For the pair kernel's local form (two_slot_step) the chunk keeps
+//     kappa = |b|^2 - |c|^2 (for unit vectors the same for every point of the
+//     chunk; the middle of its range here) and half the slack that the form
+//     adds to an edge's guard band for this chunk: the deviation of kappa from
+//     that middle, and u (10 r + 55 r^2 + 5 |kappa|) for the roundings that
+//     grow with the chunk's radius r (u = 2^-24; derived at local_guard in the
+//     host sources), times 1.05.
+// A chunk holding a padding sentinel gets radius -1 and one wider than 0.5 gets
+// radius 3, so that their pairs are never settled per chunk; both keep the
+// origin as their centre (b' = the FP32 copy).
+struct LocalChunks {
+    float* xyz;       // planar local coordinates, stride apart
+    long long stride;
+    float4* caps;     // per chunk: centre, radius
+    float2* kap;      // per chunk: kappa, half the slack
+};
+__device__ __forceinline__ void write_chunk(long long i, const float4& q, double px, double py,
+                                            double pz, const LocalChunks& L) {
+    const int lane = threadIdx.x & 31;
+    float sx = q.x, sy = q.y, sz = q.z;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sx += __shfl_xor_sync(0xffffffffu, sx, o);
+        sy += __shfl_xor_sync(0xffffffffu, sy, o);
+        sz += __shfl_xor_sync(0xffffffffu, sz, o);
+    }
+    float cx = sx * (1.f / 32), cy = sy * (1.f / 32), cz = sz * (1.f / 32);
+    const float dx = q.x - cx, dy = q.y - cy, dz = q.z - cz;
+    float m = dx * dx + dy * dy + dz * dz;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    // (a NaN coordinate leaves the sum NaN and the centre with it)
+    const bool pad = __any_sync(0xffffffffu, is_sentinel(q));
+    float r = sqrtf(m) * (1.f + 1e-6f);
+    const bool wide = !(r <= 0.5f && cx * cx + cy * cy + cz * cz <= 4.f);
+    if (pad || wide) cx = cy = cz = 0.f;
+    const double ex = px - (double)cx, ey = py - (double)cy, ez = pz - (double)cz;
+    const double kb = ex * (px + (double)cx) + ey * (py + (double)cy) + ez * (pz + (double)cz);
+    double k0 = kb, k1 = kb;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        k0 = fmin(k0, __shfl_xor_sync(0xffffffffu, k0, o));
+        k1 = fmax(k1, __shfl_xor_sync(0xffffffffu, k1, o));
+    }
+    L.xyz[i] = pad ? q.x : (float)ex;
+    L.xyz[L.stride + i] = pad ? q.y : (float)ey;
+    L.xyz[2 * L.stride + i] = pad ? q.z : (float)ez;
+    if (lane == 0) {
+        const float kappa = (float)(0.5 * (k0 + k1));
+        const float dev = (float)fmax(k1 - (double)kappa, (double)kappa - k0);
+        const float rr = r + 2.4e-7f;
+        const float slack = 1.05f * (dev + 5.9604645e-8f * (10.f * rr + 55.f * rr * rr +
+                                                            5.f * fabsf(kappa)));
+        L.caps[i / 32] = make_float4(cx, cy, cz, pad ? -1.f : wide ? 3.f : r);
+        L.kap[i / 32] = make_float2(kappa, 0.5f * slack);
+    }
+}
+
 // FP32 and FP64 copies of both catalogues in the joint order (order: the
-// sorted positions of x, a's points first): a's at [0, na) with sentinels up
-// to pa, b's at [pa, pa + nb) with sentinels up to pa + pb (tags tag0 and
-// tag0 + 1); the FP64 copy has stride pa + pb, and each FP32 point keeps in w
-// its index within its own catalogue.
-__global__ void k_gather_joint(const double* __restrict__ x, long long na, long long pa,
-                               long long nb, long long pb, const unsigned* __restrict__ order,
-                               int tag0, float4* __restrict__ p32, double* __restrict__ s64) {
+// sorted positions of x, a's points first): FP32 with a's points at [0, na)
+// and sentinels up to pa, b's at [pa, pa + nb) and sentinels up to pa + pb
+// (tags tag0 and tag0 + 1), each point keeping in w its index within its own
+// catalogue, and the chunks' spheres and local coordinates; FP64 without
+// padding (stride na + nb, b's points from na on).  One warp per chunk (pa and
+// pb are multiples of 32).  L.xyz may lie where the sort kept its keys.
+__global__ void __launch_bounds__(256) k_gather_joint(const double* __restrict__ x, long long na,
+                                                      long long pa, long long nb, long long pb,
+                                                      const unsigned* __restrict__ order, int tag0,
+                                                      float4* __restrict__ p32,
+                                                      double* __restrict__ s64, LocalChunks L) {
     const long long N = na + nb, P = pa + pb;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P;
          i += (long long)gridDim.x * blockDim.x) {
@@ -420,11 +494,15 @@ __global__ void k_gather_joint(const double* __restrict__ x, long long na, long 
         double px, py, pz;
         float4 q;
         if (j < n) {
-            const long long k = order[(in_b ? na : 0) + j];
+            const long long o = (in_b ? na : 0) + j;
+            const long long k = order[o];
             px = x[k];
             py = x[N + k];
             pz = x[2 * N + k];
             q = point32(px, py, pz, in_b ? k - na : k);
+            s64[o] = px;
+            s64[N + o] = py;
+            s64[2 * N + o] = pz;
         } else {
             q = sentinel32(tag0 + (in_b ? 1 : 0), j - n);
             px = q.x;
@@ -432,37 +510,7 @@ __global__ void k_gather_joint(const double* __restrict__ x, long long na, long 
             pz = q.z;
         }
         p32[i] = q;
-        s64[i] = px;
-        s64[P + i] = py;
-        s64[2 * P + i] = pz;
-    }
-}
-
-// FP32 copies in sorted order (w = original index); slots n..n_pad-1 get
-// sentinels.
-__global__ void k_gather_points(const double* __restrict__ xyz, long long stride, long long n,
-                                long long n_pad, const unsigned* __restrict__ order,
-                                float4* __restrict__ p32, double* __restrict__ s64, int tag) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_pad;
-         i += (long long)gridDim.x * blockDim.x) {
-        double x, y, z;
-        float4 q;
-        if (i < n) {
-            const long long j = order[i];
-            x = xyz[j];
-            y = xyz[stride + j];
-            z = xyz[2 * stride + j];
-            q = point32(x, y, z, j);
-        } else {
-            q = sentinel32(tag, i - n);
-            x = q.x;
-            y = q.y;
-            z = q.z;
-        }
-        p32[i] = q;
-        s64[i] = x;
-        s64[n_pad + i] = y;
-        s64[2 * n_pad + i] = z;
+        write_chunk(i, q, px, py, pz, L);
     }
 }
 
@@ -497,16 +545,19 @@ __global__ void k_count_labels(const unsigned* __restrict__ lab, long long n, in
 
 // FP32 copies with every region starting on a tile boundary: region r's
 // points (sorted positions src[r] .. src[r+1]-1) go to dst[r] .., the rest of
-// its last tile holds sentinels.  dst[R] = n_pad.  A sentinel is numbered
+// its last tile holds sentinels; with the chunks' spheres and local
+// coordinates, one warp per chunk.  dst[R] = n_pad, a multiple of 32.  A sentinel is numbered
 // within its region (below the tile size) and tagged by its region and
 // array, so that no two sentinels a count can pair coincide in FP32 (numbered
 // by their position in a long array, sentinels more than 2^24 points in would
 // round onto one another).
-__global__ void k_gather_regions(const double* __restrict__ xyz, long long stride,
-                                 const unsigned* __restrict__ order,
-                                 const long long* __restrict__ src,
-                                 const long long* __restrict__ dst, int R, long long n_pad,
-                                 float4* __restrict__ p32, int tag) {
+__global__ void __launch_bounds__(256) k_gather_regions(const double* __restrict__ xyz,
+                                                        long long stride,
+                                                        const unsigned* __restrict__ order,
+                                                        const long long* __restrict__ src,
+                                                        const long long* __restrict__ dst, int R,
+                                                        long long n_pad, float4* __restrict__ p32,
+                                                        int tag, LocalChunks L) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_pad;
          i += (long long)gridDim.x * blockDim.x) {
         int lo = 0, hi = R - 1;  // last region with dst <= i
@@ -515,12 +566,22 @@ __global__ void k_gather_regions(const double* __restrict__ xyz, long long strid
             if (dst[mid] <= i) lo = mid; else hi = mid - 1;
         }
         const long long j = i - dst[lo], n_lo = src[lo + 1] - src[lo];
+        double px, py, pz;
+        float4 q;
         if (j < n_lo) {
             const long long k = order[src[lo] + j];
-            p32[i] = point32(xyz[k], xyz[stride + k], xyz[2 * stride + k], k);
+            px = xyz[k];
+            py = xyz[stride + k];
+            pz = xyz[2 * stride + k];
+            q = point32(px, py, pz, k);
         } else {
-            p32[i] = sentinel32(2 * lo + tag, j - n_lo);
+            q = sentinel32(2 * lo + tag, j - n_lo);
+            px = q.x;
+            py = q.y;
+            pz = q.z;
         }
+        p32[i] = q;
+        write_chunk(i, q, px, py, pz, L);
     }
 }
 
@@ -607,10 +668,6 @@ __device__ __forceinline__ void item_to_tiles(long long t, long long T_a, long l
 // centre = normalised FP64 sum, radius = the largest angle from the centre,
 // plus 1e-6 rad for the FP32 rounding of the points (a point moves by at most
 // ~1.1e-7 rad from its FP64 position).
-__device__ __forceinline__ bool is_sentinel(const float4& q) {
-    return q.x * q.x + q.y * q.y + q.z * q.z > 4.f;
-}
-
 __global__ void __launch_bounds__(128) k_tile_caps(const float4* __restrict__ p32, long long n,
                                                    int T, TileCap* __restrict__ caps) {
     __shared__ double red[4][4];
@@ -663,38 +720,6 @@ __global__ void __launch_bounds__(128) k_tile_caps(const float4* __restrict__ p3
         cap.rho = empty ? -1.0
                         : (spread ? 4.0 : 2.0 * asin(fmin(1.0, 0.5 * sqrt(m))) + 1e-6);
         caps[blockIdx.x] = cap;
-    }
-}
-
-// Bounding sphere of every chunk of 32 consecutive spatially ordered FP32
-// points: centre = the FP32 mean of the chunk's points, radius = the largest
-// FP32 distance of a point from it, enlarged by a relative 1e-6 for the few
-// roundings of that arithmetic.  A chunk holding a padding sentinel gets
-// radius -1, so that its pairs are never settled per chunk.  One warp per
-// chunk.
-__global__ void k_chunk_caps(const float4* __restrict__ p32, long long n, long long n_pad,
-                             float4* __restrict__ caps) {
-    const int lane = threadIdx.x & 31;
-    const long long n_chunks = n_pad / 32;
-    const long long wpb = blockDim.x / 32;
-    for (long long c = blockIdx.x * wpb + (threadIdx.x >> 5); c < n_chunks;
-         c += (long long)gridDim.x * wpb) {
-        const long long i = c * 32 + lane;
-        const float4 q = p32[i];
-        float sx = q.x, sy = q.y, sz = q.z;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sx += __shfl_xor_sync(0xffffffffu, sx, o);
-            sy += __shfl_xor_sync(0xffffffffu, sy, o);
-            sz += __shfl_xor_sync(0xffffffffu, sz, o);
-        }
-        const float cx = sx * (1.f / 32), cy = sy * (1.f / 32), cz = sz * (1.f / 32);
-        const float dx = q.x - cx, dy = q.y - cy, dz = q.z - cz;
-        float m = dx * dx + dy * dy + dz * dz;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        const bool pad = __any_sync(0xffffffffu, i >= n || is_sentinel(q));
-        if (lane == 0) caps[c] = make_float4(cx, cy, cz, pad ? -1.f : sqrtf(m) * (1.f + 1e-6f));
     }
 }
 
@@ -876,7 +901,7 @@ struct PairKernel {
         b += (size_t)TB / 32 * 16;              // bounding spheres of its 32-point chunks
         b += (size_t)n_lut * 16;                // screening table
         b += (size_t)(K + 2) * 8;               // FP64 edges (+ pad)
-        b += (size_t)(K + 2) * 8;               // guard band of every edge
+        b += (size_t)(K + 2) * 8;               // middle and half slack of every edge
         b += (size_t)(K + 2) * ROWB;            // histograms, row K+1 a trash row
         return b;
     }
@@ -1051,12 +1076,13 @@ __device__ __forceinline__ void exact_steps(int j0, int j1, unsigned bxy, unsign
     }
 }
 
-// Bounding sphere of the thread's R A points (FP32): centre = their mean,
-// radius = the largest distance from it, enlarged by a relative 1e-6 for the
-// roundings of that arithmetic.  Padding sentinels give a radius far above 2.
+// Bounding sphere of the thread's R A points (FP32), given relative to their
+// chunk's centre c: centre = c + their mean, radius = the largest distance
+// from the mean, enlarged by a relative 1e-6 for the roundings of that
+// arithmetic.  Padding sentinels give a radius far above 2.
 template <int R>
 __device__ __forceinline__ float4 group_cap(const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
-                                            const f2_t (&az)[R / 2]) {
+                                            const f2_t (&az)[R / 2], const float4& c) {
     float x[R], y[R], z[R];
 #pragma unroll
     for (int q = 0; q < R / 2; ++q) {
@@ -1074,7 +1100,7 @@ __device__ __forceinline__ float4 group_cap(const f2_t (&ax)[R / 2], const f2_t 
         const float dx = x[r] - cx, dy = y[r] - cy, dz = z[r] - cz;
         m = fmaxf(m, dx * dx + dy * dy + dz * dz);
     }
-    return make_float4(cx, cy, cz, sqrtf(m) * (1.f + 1e-6f));
+    return make_float4(c.x + cx, c.y + cy, c.z + cz, sqrtf(m) * (1.f + 1e-6f));
 }
 
 // How the pairs of a group of A points (sphere ga) with a chunk of B points
@@ -1119,13 +1145,51 @@ __device__ __forceinline__ int span_class(float4 ga, float4 gb, unsigned lut, in
     return 2;
 }
 
-// One step of a three-slot chunk: as two_slot_step, against two edges (the
-// middles of their guard bands mid1 < mid2), with one accumulator each.
+// The local form of a pair's squared chord: with the chunk's centre c, b = c +
+// b', and a' = a - c,
+//     s = |a'|^2 + kappa - 2 a.b',   kappa = |b|^2 - |c|^2,
+// where kappa is one number for the whole chunk when b is a unit vector.  So
+// per pair d = (s - mid) / 2 is three fused multiply-adds from
+// A0 = (|a'|^2 + (kappa - mid)) / 2, which each A point has once per job, and
+// the three subtractions of |a - b|^2 fall away.  The products are small (|b'|
+// is at most the chunk's radius), so the roundings stay below those of the
+// difference form; |d| > G, G the edge's half slack plus the chunk's
+// (local_guard, write_chunk), settles the side of the FP64 squared chord.
+//
+// Survey, 1M + 1M points: the two-slot loop is 12 packed fmas per B point and
+// 8 A points instead of 24 packed operations.
+//
+// One step: JU B points (staged negated) and the thread's R A points.  neg[q]
+// counts the values with d < 0 and mb[q] keeps the smallest |d|, one
+// accumulator per A pair q so that the steps' dependency chains interleave.
+template <int R, int JU>
+__device__ __forceinline__ void two_slot_step(unsigned bxy_base, unsigned bz_base,
+                                              const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
+                                              const f2_t (&az)[R / 2], const f2_t (&a0)[R / 2],
+                                              int j, unsigned (&neg)[R / 2], float (&mb)[R / 2]) {
+#pragma unroll
+    for (int h = 0; h < JU; ++h) {
+        f2_t bx, by;
+        lds_f2x2(bxy_base + 16u * (unsigned)(j + h), bx, by);
+        const f2_t bz = lds_f2(bz_base + 8u * (unsigned)(j + h));
+#pragma unroll
+        for (int q = 0; q < R / 2; ++q) {
+            float d0, d1;
+            unpack2(fma2(ax[q], bx, fma2(ay[q], by, fma2(az[q], bz, a0[q]))), d0, d1);
+            mb[q] = min3f(mb[q], fabsf(d0), fabsf(d1));
+            neg[q] += (__float_as_uint(d0) >> 31) + (__float_as_uint(d1) >> 31);
+        }
+    }
+}
+
+// One step of a three-slot chunk: the same against two edges, the second's
+// value from the first's by one more subtraction of half their distance
+// (ndel = -(mid2 - mid1) / 2).
 template <int R, int JU>
 __device__ __forceinline__ void three_slot_step(unsigned bxy_base, unsigned bz_base,
                                                 const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
-                                                const f2_t (&az)[R / 2], int j, f2_t nmid1,
-                                                f2_t nmid2, unsigned& neg1, unsigned& neg2,
+                                                const f2_t (&az)[R / 2], const f2_t (&a0)[R / 2],
+                                                int j, f2_t ndel, unsigned& neg1, unsigned& neg2,
                                                 float& mb1, float& mb2) {
 #pragma unroll
     for (int h = 0; h < JU; ++h) {
@@ -1134,50 +1198,14 @@ __device__ __forceinline__ void three_slot_step(unsigned bxy_base, unsigned bz_b
         const f2_t bz = lds_f2(bz_base + 8u * (unsigned)(j + h));
 #pragma unroll
         for (int q = 0; q < R / 2; ++q) {
-            const f2_t dx = add2(ax[q], bx);
-            const f2_t dy = add2(ay[q], by);
-            const f2_t dz = add2(az[q], bz);
-            const f2_t t = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+            const f2_t t = fma2(ax[q], bx, fma2(ay[q], by, fma2(az[q], bz, a0[q])));
             float d0, d1, e0, e1;
-            unpack2(add2(t, nmid1), d0, d1);
-            unpack2(add2(t, nmid2), e0, e1);
+            unpack2(t, d0, d1);
+            unpack2(add2(t, ndel), e0, e1);
             mb1 = min3f(mb1, fabsf(d0), fabsf(d1));
             mb2 = min3f(mb2, fabsf(e0), fabsf(e1));
             neg1 += (__float_as_uint(d0) >> 31) + (__float_as_uint(d1) >> 31);
             neg2 += (__float_as_uint(e0) >> 31) + (__float_as_uint(e1) >> 31);
-        }
-    }
-}
-
-// One step of a two-slot chunk: for JU B points and the thread's R A points,
-// d = s - mid evaluated as fma(dz, dz, fma(dy, dy, fma(dx, dx, -mid))) from the
-// same FP32 differences as chords().  Each fma rounds once, on a magnitude of
-// at most max(s, mid), so for s <= 2c + 1e-12 (the only values near the edge)
-// |d - (s - mid)| stays within the three roundings the guard band already
-// allows for s (gamma_3 (s + E1), evaluated at 2c + 1e-12), and |d| > G
-// settles the side of the FP64 squared chord exactly as the band does; far
-// above the edge d is large and positive.  neg[q] counts the values with
-// d < 0 and mb[q] keeps the smallest |d|, one accumulator per A pair q so that
-// the steps' dependency chains interleave.
-template <int R, int JU>
-__device__ __forceinline__ void two_slot_step(unsigned bxy_base, unsigned bz_base,
-                                              const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
-                                              const f2_t (&az)[R / 2], int j, f2_t nmid,
-                                              unsigned (&neg)[R / 2], float (&mb)[R / 2]) {
-#pragma unroll
-    for (int h = 0; h < JU; ++h) {
-        f2_t bx, by;
-        lds_f2x2(bxy_base + 16u * (unsigned)(j + h), bx, by);
-        const f2_t bz = lds_f2(bz_base + 8u * (unsigned)(j + h));
-#pragma unroll
-        for (int q = 0; q < R / 2; ++q) {
-            const f2_t dx = add2(ax[q], bx);
-            const f2_t dy = add2(ay[q], by);
-            const f2_t dz = add2(az[q], bz);
-            float d0, d1;
-            unpack2(fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, nmid))), d0, d1);
-            mb[q] = min3f(mb[q], fabsf(d0), fabsf(d1));
-            neg[q] += (__float_as_uint(d0) >> 31) + (__float_as_uint(d1) >> 31);
         }
     }
 }
@@ -1286,6 +1314,56 @@ __device__ __forceinline__ void load_group(const float4* __restrict__ gA, f2_t (
     }
 }
 
+// The R consecutive points from position pos on (R | pos) of the planar local
+// coordinates p, packed two by two: relative to the centre of their own chunk.
+// A warp that reads 32 groups of one sub-tile touches 8 lines per load (lanes
+// 32 B apart) where float4 points, 128 B apart, touch 32: the reads of the
+// jobs' A points had been over half of the L1 data pipe's wavefronts, which
+// bounded the kernel (69% of their peak rate, FMA and ALU pipes at 40%).
+template <int R>
+__device__ __forceinline__ void load_local(const float* __restrict__ p, long long stride,
+                                           long long pos, f2_t (&ax)[R / 2], f2_t (&ay)[R / 2],
+                                           f2_t (&az)[R / 2]) {
+#pragma unroll
+    for (int q = 0; q < R / 4; ++q) {
+        const float4 x = *reinterpret_cast<const float4*>(p + pos + 4 * q);
+        const float4 y = *reinterpret_cast<const float4*>(p + stride + pos + 4 * q);
+        const float4 z = *reinterpret_cast<const float4*>(p + 2 * stride + pos + 4 * q);
+        ax[2 * q] = pack2(x.x, x.y);
+        ax[2 * q + 1] = pack2(x.z, x.w);
+        ay[2 * q] = pack2(y.x, y.y);
+        ay[2 * q + 1] = pack2(y.z, y.w);
+        az[2 * q] = pack2(z.x, z.y);
+        az[2 * q + 1] = pack2(z.z, z.w);
+    }
+}
+
+// The group's points, given relative to centre a, relative to centre b (b = 0:
+// the points themselves).  b - a is rounded relative to itself and the sum
+// relative to itself, so a coordinate difference against a point b' of b's
+// chunk errs by about 2 u |a - b| + u (ra + rb) instead of the 2 u of
+// differences of the FP32 copies: inside every guard band derived for those.
+template <int R>
+__device__ __forceinline__ void recentre(const float4& a, const float4& b, const f2_t (&ax)[R / 2],
+                                         const f2_t (&ay)[R / 2], const f2_t (&az)[R / 2],
+                                         f2_t (&lx)[R / 2], f2_t (&ly)[R / 2], f2_t (&lz)[R / 2]) {
+    const float x = a.x - b.x, y = a.y - b.y, z = a.z - b.z;
+    const f2_t dx = pack2(x, x), dy = pack2(y, y), dz = pack2(z, z);
+#pragma unroll
+    for (int q = 0; q < R / 2; ++q) {
+        lx[q] = add2(ax[q], dx);
+        ly[q] = add2(ay[q], dy);
+        lz[q] = add2(az[q], dz);
+    }
+}
+
+// Sphere of chunk c of the staged tile (caps: shared address).
+__device__ __forceinline__ float4 chunk_sphere(unsigned caps, int c) {
+    const uint4 g = lds_u4(caps + 16u * (unsigned)c);
+    return make_float4(__uint_as_float(g.x), __uint_as_float(g.y), __uint_as_float(g.z),
+                       __uint_as_float(g.w));
+}
+
 // ---------------------------------------------------------------------------
 // Span jobs.  A (group, chunk) pair whose span needs its pairs computed (two
 // slots, three slots, or pair by pair) is a job: the lane whose R A points
@@ -1351,59 +1429,72 @@ __device__ __forceinline__ void exact_chunk(int c0, int rot, int t0, int ts, int
     }
 }
 
-// A job's R A points (the owner lane's group) from the FP32 copy.
+// A job's R A points (the owner lane's group), relative to the centre ca of
+// their own chunk.
 template <int NT, int R, int JU, int HM>
-__device__ __forceinline__ int job_points(unsigned job, unsigned sIJ, const Segment& S,
+__device__ __forceinline__ int job_points(unsigned job, unsigned sIJ, const Segment& S, float4& ca,
                                           f2_t (&ax)[R / 2], f2_t (&ay)[R / 2],
                                           f2_t (&az)[R / 2]) {
     constexpr int TA = PairKernel<NT, R, JU, HM, 0>::TA, SA = 32 * R;
     const int a_first = (int)((job >> 5) & 7u) * SA + (int)(job & 31u) * R;
-    load_group<R>(S.a32 + lds_s64(sIJ) * TA + a_first, ax, ay, az);
+    const long long pos = lds_s64(sIJ) * TA + a_first;
+    ca = __ldg(S.a_caps + pos / kChunk);
+    load_local<R>(S.al, S.al_stride, pos, ax, ay, az);
     return a_first;
 }
 
 // A job of the pair-by-pair kind (the chunk's points t0, t0 + ts, ...).
 template <int NT, int R, int JU, int HM>
 __device__ __forceinline__ void exact_job(unsigned job, int t0, int ts, unsigned sIJ,
-                                          unsigned bxy, unsigned bz, unsigned lut, unsigned sC,
-                                          unsigned col, const PairParams& p, const Segment& S,
-                                          unsigned& n_recheck) {
+                                          unsigned bxy, unsigned bz, unsigned lut, unsigned caps,
+                                          unsigned sC, unsigned col, const PairParams& p,
+                                          const Segment& S, unsigned& n_recheck) {
     f2_t ax[R / 2], ay[R / 2], az[R / 2];
-    const int a_first = job_points<NT, R, JU, HM>(job, sIJ, S, ax, ay, az);
+    float4 ca;
+    const int a_first = job_points<NT, R, JU, HM>(job, sIJ, S, ca, ax, ay, az);
     const int c = (int)((job >> 8) & 255u);
+    recentre<R>(ca, chunk_sphere(caps, c), ax, ay, az, ax, ay, az);
     exact_chunk<NT, R, JU, HM>(c * kChunk, (JU * c) & (kChunk - 1), t0, ts, a_first, sIJ, bxy,
                                bz, lut, sC, col, ax, ay, az, p, S, n_recheck);
 }
 
-// The middle of the guard band of edge k (band table at shared address band)
-// and the band's half-width.
+// The middle of edge k (edge table at shared address band) and half its slack
+// for the local form.
 __device__ __forceinline__ float edge_mid(unsigned band, unsigned k, float& G) {
-    unsigned lo, hi;
-    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(lo), "=r"(hi) : "r"(band + 8u * k));
-    const float lo_f = __uint_as_float(lo), hi_f = __uint_as_float(hi);
-    const float mid = 0.5f * (lo_f + hi_f);
-    G = fmaxf(mid - lo_f, hi_f - mid);
+    float mid;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(mid), "=f"(G) : "r"(band + 8u * k));
     return mid;
 }
 
 // A job of kind T (two or three slots) over the chunk's steps t0, t0 + ts,
-// ... (JU points each).  Two slots: d = s - mid per pair, mid the middle of
-// the edge's guard band; three slots: the same against two edges.  neg1 and
-// neg2 count the values with d < 0 for the first and second edge (neg2 = 0
-// for two slots), mb1 and mb2 keep the smallest |d|.
+// ... (JU points each).  neg1 and neg2 count the values below the first and
+// second edge (neg2 = 0 for two slots), mb1 and mb2 return the smallest |d|
+// less the slack: at most zero if some value may be on either side.
 template <int NT, int R, int JU, int HM>
 __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, unsigned sIJ,
-                                          unsigned bxy, unsigned bz, unsigned band,
+                                          unsigned bxy, unsigned bz, unsigned caps, unsigned band,
                                           const Segment& S, unsigned& neg1, unsigned& neg2,
                                           float& mb1, float& mb2) {
-    f2_t ax[R / 2], ay[R / 2], az[R / 2];
-    job_points<NT, R, JU, HM>(job, sIJ, S, ax, ay, az);
+    constexpr int CPT = PairKernel<NT, R, JU, HM, 0>::TB / kChunk;
     const int c = (int)((job >> 8) & 255u);
+    const float2 kap = __ldg(S.b_kap + lds_s64(sIJ + 8u) * CPT + c);
+    f2_t ax[R / 2], ay[R / 2], az[R / 2], a0[R / 2];
+    float4 ca;
+    job_points<NT, R, JU, HM>(job, sIJ, S, ca, ax, ay, az);
     const int c0 = c * kChunk, rot = (JU * c) & (kChunk - 1);
     const unsigned slot = (job >> 16) & 0x3FFFu;
-    float G;
+    float G, G2 = 0.f;
     const float mid = edge_mid(band, slot, G);
-    const f2_t nmid = pack2(-mid, -mid);
+    {
+        f2_t lx[R / 2], ly[R / 2], lz[R / 2];
+        recentre<R>(ca, chunk_sphere(caps, c), ax, ay, az, lx, ly, lz);
+        recentre<R>(ca, make_float4(0.f, 0.f, 0.f, 0.f), ax, ay, az, ax, ay, az);
+        const float km = kap.x - mid;
+        const f2_t km2 = pack2(km, km), half = pack2(0.5f, 0.5f);
+#pragma unroll
+        for (int q = 0; q < R / 2; ++q)
+            a0[q] = mul2(half, fma2(lx[q], lx[q], fma2(ly[q], ly[q], fma2(lz[q], lz[q], km2))));
+    }
     neg1 = neg2 = 0;
     mb1 = mb2 = __int_as_float(0x7f800000);
     if (T == kJobTwo) {
@@ -1416,44 +1507,42 @@ __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, u
         }
 #pragma unroll 1
         for (int t = t0; t < kChunk; t += ts)
-            two_slot_step<R, JU>(bxy, bz, ax, ay, az, chunk_point<JU>(c0, t, rot), nmid, negq,
-                                 mbq);
+            two_slot_step<R, JU>(bxy, bz, ax, ay, az, a0, chunk_point<JU>(c0, t, rot), negq, mbq);
 #pragma unroll
         for (int q = 0; q < R / 2; ++q) {
             neg1 += negq[q];
             mb1 = fminf(mb1, mbq[q]);
         }
-        return;
-    }
-    const float mid2 = edge_mid(band, slot + 1u, G);
+    } else {
+        const float mid2 = edge_mid(band, slot + 1u, G2);
+        const float ndel = 0.5f * (mid - mid2);
 #pragma unroll 1
-    for (int t = t0; t < kChunk; t += ts)
-        three_slot_step<R, JU>(bxy, bz, ax, ay, az, chunk_point<JU>(c0, t, rot), nmid,
-                               pack2(-mid2, -mid2), neg1, neg2, mb1, mb2);
+        for (int t = t0; t < kChunk; t += ts)
+            three_slot_step<R, JU>(bxy, bz, ax, ay, az, a0, chunk_point<JU>(c0, t, rot),
+                                   pack2(ndel, ndel), neg1, neg2, mb1, mb2);
+        mb2 -= G2 + kap.y;
+    }
+    mb1 -= G + kap.y;
 }
 
 // Settles a two- or three-slot job from its counts (summed over the lanes
-// that shared it): |d| > G for every value puts each value outside its
-// edge's guard band, and then d < 0 means below the edge.  Returns false if
-// some value had |d| <= G (rare): nothing is counted, and the chunk has to go
-// pair by pair.
+// that shared it): with every |d| beyond the slack (mb1, mb2 > 0), d < 0 means
+// below the edge.  Returns false otherwise (rare): nothing is counted, and the
+// chunk has to go pair by pair.
 template <int NT, int R, int JU, int HM>
-__device__ __forceinline__ bool span_settle(int T, unsigned job, unsigned band, unsigned col,
-                                            unsigned neg1, unsigned neg2, float mb1, float mb2) {
+__device__ __forceinline__ bool span_settle(int T, unsigned job, unsigned col, unsigned neg1,
+                                            unsigned neg2, float mb1, float mb2) {
     constexpr unsigned NP = (unsigned)(R * kChunk);
     constexpr unsigned row_bytes = PairKernel<NT, R, JU, HM, 0>::ROWB;
     const unsigned slot = (job >> 16) & 0x3FFFu;
     const unsigned rlo = slot * row_bytes;
-    float G, G2 = 0.f;
-    edge_mid(band, slot, G);
-    if (mb1 <= G) return false;
+    if (!(mb1 > 0.f)) return false;
     if (T == kJobTwo) {
         hist_add<HM>(col + rlo, neg1);
         hist_add<HM>(col + rlo + row_bytes, NP - neg1);
         return true;
     }
-    edge_mid(band, slot + 1u, G2);
-    if (mb2 <= G2) return false;
+    if (!(mb2 > 0.f)) return false;
     hist_add<HM>(col + rlo, neg1);
     hist_add<HM>(col + rlo + row_bytes, neg2 - neg1);
     hist_add<HM>(col + rlo + 2u * row_bytes, NP - neg2);
@@ -1478,21 +1567,22 @@ __device__ __forceinline__ void warp_stat(unsigned a, bool flag, unsigned w) {
 template <int NT, int R, int JU, int HM, bool ST>
 __device__ __forceinline__ unsigned job_round(int T, unsigned run, bool active, int t0, int ts,
                                               unsigned sIJ, unsigned bxy, unsigned bz,
-                                              unsigned lut, unsigned band, unsigned sC,
-                                              unsigned col, const PairParams& p,
+                                              unsigned lut, unsigned caps, unsigned band,
+                                              unsigned sC, unsigned col, const PairParams& p,
                                               const Segment& S, bool stats, unsigned stat) {
     constexpr unsigned NP = (unsigned)(R * kChunk);
     const int lane = threadIdx.x & 31;
     unsigned n_recheck = 0, fb = 0;
     bool settled = false;
     if (T == kJobExact) {
-        if (active) exact_job<NT, R, JU, HM>(run, t0, ts, sIJ, bxy, bz, lut, sC, col, p, S, n_recheck);
+        if (active)
+            exact_job<NT, R, JU, HM>(run, t0, ts, sIJ, bxy, bz, lut, caps, sC, col, p, S, n_recheck);
     } else {
         unsigned neg1 = 0, neg2 = 0;
         float mb1 = __int_as_float(0x7f800000), mb2 = mb1;
         if (active)
-            span_part<NT, R, JU, HM>(T, run, t0 * JU, ts * JU, sIJ, bxy, bz, band, S, neg1, neg2,
-                                     mb1, mb2);
+            span_part<NT, R, JU, HM>(T, run, t0 * JU, ts * JU, sIJ, bxy, bz, caps, band, S, neg1,
+                                     neg2, mb1, mb2);
 #pragma unroll 1
         for (int o = ts >> 1; o > 0; o >>= 1) {
             neg1 += __shfl_xor_sync(0xffffffffu, neg1, o);
@@ -1501,7 +1591,7 @@ __device__ __forceinline__ unsigned job_round(int T, unsigned run, bool active, 
             mb2 = fminf(mb2, __shfl_xor_sync(0xffffffffu, mb2, o));
         }
         if (active && t0 == 0) {
-            settled = span_settle<NT, R, JU, HM>(T, run, band, col, neg1, neg2, mb1, mb2);
+            settled = span_settle<NT, R, JU, HM>(T, run, col, neg1, neg2, mb1, mb2);
             if (!settled) fb = run | (1u << 30);
         }
     }
@@ -1590,8 +1680,9 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
             }
             if (sub != cap_sub) {
                 f2_t ax[R / 2], ay[R / 2], az[R / 2];
-                load_group<R>(S.a32 + lds_s64(sIJ) * TA + sub * SA + lane * R, ax, ay, az);
-                ga = group_cap<R>(ax, ay, az);
+                const long long pos = lds_s64(sIJ) * TA + sub * SA + lane * R;
+                load_local<R>(S.al, S.al_stride, pos, ax, ay, az);
+                ga = group_cap<R>(ax, ay, az, __ldg(S.a_caps + pos / kChunk));
                 cap_sub = sub;
             }
             cn = ub / kChunk;
@@ -1605,9 +1696,7 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
         if (!done) {
             const int c = cn;
             cn = (c + 1) % CPU == 0 ? -1 : c + 1;
-            const uint4 gbu = lds_u4(caps + 16u * (unsigned)c);
-            const float4 gb = make_float4(__uint_as_float(gbu.x), __uint_as_float(gbu.y),
-                                          __uint_as_float(gbu.z), __uint_as_float(gbu.w));
+            const float4 gb = chunk_sphere(caps, c);
             unsigned rlo = 0;
             const unsigned trash = (unsigned)(p.tab.K + 1) * row_bytes;
             const int mode = span_class(ga, gb, lut, p.tab.shift, p.tab.base, p.tab.n_lut - 1,
@@ -1683,7 +1772,7 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
             if (push && pos >= 32) sts_u32(rt + 4u * (unsigned)(pos - 32), job);
             fills = (fills & ~(255u << (8 * T))) | ((unsigned)max(total - 32, 0) << (8 * T));
             fb = job_round<NT, R, JU, HM, ST>(T, run, jl < total, lane % ts, ts, sIJ, bxy, bz, lut,
-                                              band, sC, col, p, S, stats, stat);
+                                              caps, band, sC, col, p, S, stats, stat);
         }
         if (done) break;
     }
@@ -1722,8 +1811,8 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
             const unsigned run =
                 lds_u32(rings + RING_BYTES * (unsigned)q + 128u * (unsigned)T + 4u * (unsigned)i);
             const unsigned fb = job_round<NT, R, JU, HM, ST>(T, run, jl < m, lane % ts, ts, sIJ,
-                                                             bxy, bz, lut, band, sC, col, p, S,
-                                                             stats, stat);
+                                                             bxy, bz, lut, caps, band, sC, col,
+                                                             p, S, stats, stat);
             if (T == kJobTwo) fb0 = fb;
             if (T == kJobThree) fb1 = fb;
         }
@@ -1744,7 +1833,7 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
             const unsigned run = lds_u32(rt + 4u * (unsigned)min(jl, n - 1));
             __syncwarp();
             job_round<NT, R, JU, HM, ST>(kJobExact, run, jl < n, lane % ts, ts, sIJ, bxy, bz, lut,
-                                         band, sC, col, p, S, stats, stat);
+                                         caps, band, sC, col, p, S, stats, stat);
         }
     }
     // the diagonal units taken: pair by pair, i < j
@@ -1755,10 +1844,16 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
         const int sub = b / UPS, ub = (b % UPS) * UB, a_first = sub * SA + lane * R;
         const long long I = lds_s64(sIJ), J = lds_s64(sIJ + 8u);
         f2_t ax[R / 2], ay[R / 2], az[R / 2];
-        load_group<R>(S.a32 + I * TA + a_first, ax, ay, az);
+        load_local<R>(S.al, S.al_stride, I * TA + a_first, ax, ay, az);
+        const float4 ca = __ldg(S.a_caps + (I * TA + a_first) / kChunk);
         unsigned long long nr = 0;
-        tile_pass<NT, R, JU, HM, 0, true>(bxy, bz, lut, sC, hist, ax, ay, az, p, S, I, J, a_first,
-                                          ub, ub + UB, nr);
+#pragma unroll 1
+        for (int c = ub / kChunk; c < (ub + UB) / kChunk; ++c) {
+            f2_t lx[R / 2], ly[R / 2], lz[R / 2];
+            recentre<R>(ca, chunk_sphere(caps, c), ax, ay, az, lx, ly, lz);
+            tile_pass<NT, R, JU, HM, 0, true>(bxy, bz, lut, sC, hist, lx, ly, lz, p, S, I, J,
+                                              a_first, c * kChunk, (c + 1) * kChunk, nr);
+        }
         if (stats) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
@@ -1787,7 +1882,7 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
     float4* sCap = reinterpret_cast<float4*>(sBz + TB);
     uint4* sLut = reinterpret_cast<uint4*>(sCap + TB / 32);
     double* sC = reinterpret_cast<double*>(sLut + p.tab.n_lut);
-    uint2* sBand = reinterpret_cast<uint2*>(sC + (K + 2));
+    float2* sBand = reinterpret_cast<float2*>(sC + (K + 2));
     unsigned* hist = reinterpret_cast<unsigned*>(sBand + (K + 2));
     // the item and its tile pair (I, J), in two buffers by the parity of the
     // block's item count: thread 0 writes the next item's pair while other
@@ -1802,7 +1897,7 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
                              p.tab.lut[q][3] * row_bytes);
     for (int q = tid; q <= K; q += NT) {
         sC[q] = p.tab.c64[q];
-        sBand[q] = make_uint2(p.tab.band[q][0], p.tab.band[q][1]);
+        sBand[q] = make_float2(p.tab.edge[q][0], p.tab.edge[q][1]);
     }
     for (int q = tid; q < (K + 2) * HSTRIDE; q += NT) hist[q] = 0u;
     if (tid < 3) s_stat[tid] = 0ull;
@@ -1859,15 +1954,30 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
         }
         const Segment& S = sSeg;
         const long long I = s_IJ[n_items & 1][0], J = s_IJ[n_items & 1][1];
-        const float4* gB = S.b32 + J * TB;
+        // with span binning the tile holds local coordinates (relative to each
+        // chunk's centre), otherwise the FP32 copies
+        bool spans = false;
+        if constexpr (!DEF && HM != kHistWarp) spans = p.span && S.b_caps;
+        if (spans) {
+            const float* gL = S.bl + J * TB;
+            const long long ls = S.bl_stride;
 #pragma unroll 4
-        for (int q = 0; q < R; ++q) {
-            const float4 b = gB[q * NT + tid];
-            sBxy[q * NT + tid] = make_ulonglong2(pack2(-b.x, -b.x), pack2(-b.y, -b.y));
-            sBz[q * NT + tid] = pack2(-b.z, -b.z);
-        }
-        if (S.b_caps)
+            for (int q = 0; q < R; ++q) {
+                const int i = q * NT + tid;
+                const float x = -gL[i], y = -gL[ls + i], z = -gL[2 * ls + i];
+                sBxy[i] = make_ulonglong2(pack2(x, x), pack2(y, y));
+                sBz[i] = pack2(z, z);
+            }
             for (int q = tid; q < TB / 32; q += NT) sCap[q] = S.b_caps[J * (TB / 32) + q];
+        } else {
+            const float4* gB = S.b32 + J * TB;
+#pragma unroll 4
+            for (int q = 0; q < R; ++q) {
+                const float4 b = gB[q * NT + tid];
+                sBxy[q * NT + tid] = make_ulonglong2(pack2(-b.x, -b.x), pack2(-b.y, -b.y));
+                sBz[q * NT + tid] = pack2(-b.z, -b.z);
+            }
+        }
         if (tid < NW) s_units[tid] = 0;
         __syncthreads();  // B tile staged, unit counters reset
         const unsigned a_bxy = smem_addr(sBxy), a_bz = smem_addr(sBz), a_lut = smem_addr(sLut),
@@ -1880,8 +1990,6 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
         // whatever the mix of cheap and costly units.
         const int lane = tid & 31, warp = tid >> 5;
         const bool diag = S.is_auto && I == J;
-        bool spans = false;
-        if constexpr (!DEF && HM != kHistWarp) spans = p.span && S.b_caps;
         if constexpr (!DEF && HM != kHistWarp) {
             if (spans)
                 span_item<NT, R, JU, HM, ST>(smem_addr(s_units), smem_addr(s_ring),
@@ -2154,10 +2262,10 @@ static SortBufs sort_bufs(unsigned char* scratch, long long n, int with_labels) 
     SortBufs B;
     B.G = sort_blocks(n);
     B.rounds = sort_rounds(n);
-    B.key[0] = (unsigned*)scratch;
-    B.key[1] = (unsigned*)(scratch + a4);
-    B.idx[0] = (unsigned*)(scratch + 2 * a4);
-    B.idx[1] = (unsigned*)(scratch + 3 * a4);
+    B.idx[0] = (unsigned*)scratch;  // first: what follows it is free once it is sorted
+    B.idx[1] = (unsigned*)(scratch + a4);
+    B.key[0] = (unsigned*)(scratch + 2 * a4);
+    B.key[1] = (unsigned*)(scratch + 3 * a4);
     B.lab = (unsigned*)(scratch + 4 * a4);
     B.hist = (unsigned*)(scratch + (4 + (with_labels ? 1 : 0)) * a4);
     B.tot = B.hist + ((size_t)B.G * 256 + 63) / 64 * 64;
@@ -2212,58 +2320,21 @@ int spatial_order(const double* x64, long long stride, long long n, int check,
     return check_cuda(cudaGetLastError());
 }
 
-size_t prepare_bytes(long long n, long long n_pad, int is_xyz) {
-    size_t b = (size_t)n_pad * 16 + 256;               // FP32 points
-    b += ((size_t)n_pad / 32 * 16 + 255) / 256 * 256;  // chunk bounding spheres
-    b += order_bytes(n, 0);                            // the sort
-    if (!is_xyz) b += ((size_t)n * 24 + 255) / 256 * 256;  // FP64 SoA
-    b += (size_t)n_pad * 24 + 256;                     // the same, in the spatial order
-    return b;
-}
-
-int prepare(const double* coords, long long n, long long n_pad, int is_xyz, int tag,
-                   unsigned char* scratch, int sm_count, cudaStream_t st, Prepared* out) {
-    TraceRange trace("prepare");
-    unsigned char* sp = scratch;
-    float4* p32 = (float4*)sp;
-    sp += ((size_t)n_pad * 16 + 255) / 256 * 256;
-    float4* c32 = (float4*)sp;
-    sp += ((size_t)n_pad / 32 * 16 + 255) / 256 * 256;
-    unsigned char* sort_scratch = sp;
-    sp += order_bytes(n, 0);
-    const double* x64 = coords;
-    long long stride = n;
-    if (!is_xyz && n > 0) {
-        double* x = (double*)sp;
-        k_radec_to_xyz<<<launch_grid(n, sm_count), 256, 0, st>>>(coords, n, x, n);
-        count_launch();
-        x64 = x;
-    }
-    if (!is_xyz) sp += ((size_t)n * 24 + 255) / 256 * 256;
-    double* s64 = (double*)sp;  // FP64 SoA in the spatial order (stride n_pad)
-    const unsigned* order = nullptr;
-    int rc = spatial_order(x64, stride, n, is_xyz, nullptr, 0, sort_scratch, sm_count, st, &order,
-                           nullptr);
-    if (rc) return rc;
-    k_gather_points<<<launch_grid(n_pad, sm_count), 256, 0, st>>>(x64, stride, n, n_pad, order,
-                                                                  p32, s64, tag);
-    k_chunk_caps<<<launch_grid(n_pad, sm_count), 256, 0, st>>>(p32, n, n_pad, c32);
-    count_launch(2);
-    out->p32 = p32;
-    out->c32 = c32;
-    out->x64 = s64;
-    out->stride = n_pad;
-    out->sorted = 1;
-    return check_cuda(cudaGetLastError());
-}
+// The FP32 part of a prepared set of P padded positions: points, then chunk
+// spheres; and the part that may lie where the sort kept its buffers: local
+// coordinates and the chunks' kappa and slack.
+static size_t a256(size_t b) { return (b + 255) / 256 * 256; }
+static size_t local_bytes(long long P) { return a256((size_t)P * 12) + (size_t)P / 32 * 8; }
 
 size_t prepare_joint_bytes(long long na, long long pa, long long nb, long long pb) {
     const long long N = na + nb, P = pa + pb;
-    size_t b = ((size_t)P * 16 + 255) / 256 * 256;       // FP32 points
-    b += ((size_t)P / 32 * 16 + 255) / 256 * 256;        // chunk bounding spheres
-    b += ((size_t)P * 24 + 255) / 256 * 256;             // FP64, spatial order
-    b += ((size_t)N * 24 + 255) / 256 * 256;             // FP64, input order
-    b += order_bytes(N, 0);                              // the sort
+    size_t b = a256((size_t)P * 16);              // FP32 points
+    b += a256((size_t)P / 32 * 16);               // chunk bounding spheres
+    b += a256((size_t)N * 24);                    // FP64, spatial order
+    b += a256((size_t)N * 24);                    // FP64, input order
+    // the sort; once the order is known its other buffers become the local
+    // coordinates
+    b += std::max(order_bytes(N, 0), a256((size_t)N * 4) + local_bytes(P));
     return b;
 }
 
@@ -2275,14 +2346,20 @@ int prepare_joint(const double* a, long long na, long long pa, const double* b, 
     if (N >= (1LL << 32) - 1) return WTHETA_EINVAL;  // 32-bit positions in the sort
     unsigned char* sp = scratch;
     float4* p32 = (float4*)sp;
-    sp += ((size_t)P * 16 + 255) / 256 * 256;
+    sp += a256((size_t)P * 16);
     float4* c32 = (float4*)sp;
-    sp += ((size_t)P / 32 * 16 + 255) / 256 * 256;
+    sp += a256((size_t)P / 32 * 16);
     double* s64 = (double*)sp;
-    sp += ((size_t)P * 24 + 255) / 256 * 256;
+    sp += a256((size_t)N * 24);
     double* x = (double*)sp;
-    sp += ((size_t)N * 24 + 255) / 256 * 256;
+    sp += a256((size_t)N * 24);
     const SortBufs S = sort_bufs(sp, N, 0);
+    sp += a256((size_t)N * 4);                    // S.idx[0], the order
+    LocalChunks L;
+    L.xyz = (float*)sp;
+    L.stride = P;
+    L.caps = c32;
+    L.kap = (float2*)(sp + a256((size_t)P * 12));
     if (N > 0) {
         const long long g = std::min<long long>((N + 63) / 64, (long long)sm_count * 32);
         k_joint_keys<<<(unsigned)g, 64, 0, st>>>(a, na, b, nb, is_xyz, x, S.key[0], S.idx[0]);
@@ -2291,19 +2368,24 @@ int prepare_joint(const double* a, long long na, long long pa, const double* b, 
     }
     if (P > 0) {
         k_gather_joint<<<launch_grid(P, sm_count), 256, 0, st>>>(x, na, pa, nb, pb, S.idx[0], tag0,
-                                                                 p32, s64);
-        k_chunk_caps<<<launch_grid(P, sm_count), 256, 0, st>>>(p32, P, P, c32);
-        count_launch(2);
+                                                                 p32, s64, L);
+        count_launch();
     }
     A->p32 = p32;
     A->c32 = c32;
+    A->kap = L.kap;
+    A->l32 = L.xyz;
+    A->l_stride = P;
     A->x64 = s64;
-    A->stride = P;
+    A->stride = N;
     A->sorted = 1;
     B->p32 = p32 + pa;
     B->c32 = c32 + pa / 32;
-    B->x64 = s64 + pa;
-    B->stride = P;
+    B->kap = L.kap + pa / 32;
+    B->l32 = L.xyz + pa;
+    B->l_stride = P;
+    B->x64 = s64 + na;
+    B->stride = N;
     B->sorted = 1;
     return check_cuda(cudaGetLastError());
 }
@@ -2326,20 +2408,42 @@ int launch_count_labels(const unsigned* lab, long long n, int n_labels,
 
 int launch_gather_regions(const double* x64, long long stride, const unsigned* order,
                           const long long* src, const long long* dst, int R, long long n_pad,
-                          float4* p32, int tag, int sm_count, cudaStream_t st) {
+                          int tag, int sm_count, cudaStream_t st, const Prepared& out) {
     if (n_pad <= 0) return WTHETA_OK;
-    k_gather_regions<<<launch_grid(n_pad, sm_count), 256, 0, st>>>(x64, stride, order, src, dst,
-                                                                   R, n_pad, p32, tag);
+    LocalChunks L;
+    L.xyz = (float*)out.l32;
+    L.stride = out.l_stride;
+    L.caps = (float4*)out.c32;
+    L.kap = (float2*)out.kap;
+    k_gather_regions<<<launch_grid(n_pad, sm_count), 256, 0, st>>>(
+        x64, stride, order, src, dst, R, n_pad, (float4*)out.p32, tag, L);
     count_launch();
     return check_cuda(cudaGetLastError());
 }
 
-int launch_chunk_caps(const float4* p32, long long n_pad, float4* c32, int sm_count,
-                      cudaStream_t st) {
-    if (n_pad <= 0) return WTHETA_OK;
-    k_chunk_caps<<<launch_grid(n_pad, sm_count), 256, 0, st>>>(p32, n_pad, n_pad, c32);
-    count_launch();
-    return check_cuda(cudaGetLastError());
+size_t regions_bytes(long long n_pad) {
+    return a256((size_t)n_pad * 16) + a256((size_t)n_pad / 32 * 16) + a256(local_bytes(n_pad));
+}
+
+Prepared regions_layout(unsigned char* p, long long n_pad) {
+    Prepared q;
+    q.p32 = (const float4*)p;
+    p += a256((size_t)n_pad * 16);
+    q.c32 = (const float4*)p;
+    p += a256((size_t)n_pad / 32 * 16);
+    q.l32 = (const float*)p;
+    q.l_stride = n_pad;
+    q.kap = (const float2*)(p + a256((size_t)n_pad * 12));
+    return q;
+}
+
+Prepared tile_view(const Prepared& A, long long pos) {
+    Prepared q = A;
+    q.p32 += pos;
+    q.c32 += pos / 32;
+    q.kap += pos / 32;
+    q.l32 += pos;
+    return q;
 }
 
 int launch_cull_batch(const CullSeg* cs, int n_segs, long long total, double theta_top,
@@ -2375,7 +2479,13 @@ Segment make_segment(const Prepared& A, const Prepared& B, long long ta, long lo
     Segment g;
     std::memset(&g, 0, sizeof(g));
     g.a32 = A.p32; g.b32 = B.p32; g.a64 = A.x64; g.b64 = B.x64;
+    g.a_caps = A.c32;
+    g.al = A.l32;
+    g.al_stride = A.l_stride;
     g.b_caps = B.c32;
+    g.b_kap = B.kap;
+    g.bl = B.l32;
+    g.bl_stride = B.l_stride;
     g.a64_stride = A.stride; g.b64_stride = B.stride;
     g.sorted64 = (A.sorted ? 1 : 0) | (B.sorted ? 2 : 0);
     g.tiles_a = ta; g.tiles_b = tb;
@@ -2940,8 +3050,7 @@ struct wtheta_plan {
     double* x_all = nullptr;
     int* lab_all = nullptr;
     unsigned char* sort_scratch = nullptr;
-    float4* p32_all = nullptr;
-    float4* c32_all = nullptr;
+    wtheta::Prepared all;                   // the copies of every catalogue
     wtheta::TileCap* caps_all = nullptr;
     wtheta::Segment* d_segs = nullptr;
     int n_segs = 0;
@@ -3008,10 +3117,9 @@ static int batch_prepare(wtheta_plan* P, int T, cudaStream_t st) {
                            P->sort_scratch, P->sm_count, st, &order, nullptr);
     if (!rc)
         rc = launch_gather_regions(P->x_all, P->n_all, order, P->d_src_off, P->d_src_off + nc2 + 1,
-                                   nc2, P->n_all_pad, P->p32_all, 0, P->sm_count, st);
-    if (!rc) rc = launch_chunk_caps(P->p32_all, P->n_all_pad, P->c32_all, P->sm_count, st);
+                                   nc2, P->n_all_pad, 0, P->sm_count, st, P->all);
     if (!rc && P->cull)
-        rc = launch_tile_caps(P->p32_all, P->n_all_pad, T, P->n_all_pad / T, P->caps_all, st);
+        rc = launch_tile_caps(P->all.p32, P->n_all_pad, T, P->n_all_pad / T, P->caps_all, st);
     return rc;
 }
 
@@ -3036,9 +3144,9 @@ static int plan_layout(wtheta_plan* P, const Variant* v, int sm_count, cudaStrea
     P->n_all = P->src_off[nc2];
     P->n_all_pad = P->dst_off[nc2];
     const long long N = P->n_all, NP = P->n_all_pad;
-    auto a256 = [](size_t b) { return (b + 255) / 256 * 256; };
     // scratch: the cursor head, the catalogue table and offsets, the FP64
-    // array and labels, the sort, the FP32 copies and chunk spheres
+    // array and labels, the sort, the FP32 copies, chunk spheres and local
+    // coordinates
     size_t bytes = 256;
     const size_t off_cats = bytes;
     bytes += a256((size_t)nc2 * sizeof(BatchCat));
@@ -3050,10 +3158,8 @@ static int plan_layout(wtheta_plan* P, const Variant* v, int sm_count, cudaStrea
     bytes += a256((size_t)N * 4);
     const size_t off_sort = bytes;
     bytes += a256(order_bytes(N, 1));
-    const size_t off_p32 = bytes;
-    bytes += a256((size_t)NP * 16);
-    const size_t off_c32 = bytes;
-    bytes += a256((size_t)NP / 32 * 16);
+    const size_t off_all = bytes;
+    bytes += regions_bytes(NP);
     if (P->scratch) cudaFree(P->scratch);
     P->scratch = nullptr;
     int rc = dev_malloc(&P->scratch, bytes);
@@ -3065,8 +3171,9 @@ static int plan_layout(wtheta_plan* P, const Variant* v, int sm_count, cudaStrea
     P->x_all = (double*)(base + off_x);
     P->lab_all = (int*)(base + off_lab);
     P->sort_scratch = base + off_sort;
-    P->p32_all = (float4*)(base + off_p32);
-    P->c32_all = (float4*)(base + off_c32);
+    P->all = regions_layout(base + off_all, NP);
+    P->all.x64 = P->x_all;
+    P->all.stride = N;
     std::vector<long long> offs(P->src_off);
     offs.insert(offs.end(), P->dst_off.begin(), P->dst_off.end());
     rc = check_cuda(cudaMemcpyAsync(P->d_cats, hc.data(), sizeof(BatchCat) * nc2,
@@ -3077,14 +3184,7 @@ static int plan_layout(wtheta_plan* P, const Variant* v, int sm_count, cudaStrea
     // every catalogue's view of the shared copies (FP64 in the caller's order:
     // the FP32 copies carry each point's position in the FP64 array)
     P->prep.assign(nc2, Prepared());
-    for (int c = 0; c < nc2; ++c) {
-        Prepared& q = P->prep[c];
-        q.p32 = P->p32_all + P->dst_off[c];
-        q.c32 = P->c32_all + P->dst_off[c] / 32;
-        q.x64 = P->x_all;
-        q.stride = N;
-        q.sorted = 0;
-    }
+    for (int c = 0; c < nc2; ++c) P->prep[c] = tile_view(P->all, P->dst_off[c]);
     // the work table: DD, DR, RR of every pair, biggest count first
     std::vector<Segment> segs;
     std::vector<int> seg_cat_a, seg_cat_b;  // prepared catalogue of each side

@@ -64,6 +64,33 @@ double guard_half_width(double c) {
     return 2.0 * (e32 + e64 + edge + tiny);
 }
 
+// Slack of the local form's s - mid around an edge c (the part that does not
+// depend on the chunk; see two_slot_step and write_chunk).
+//
+// With a the FP64 point, c0 the chunk's centre (an FP32 vector, exact), r its
+// radius, q = |a32 - c0| <= sqrt(s) + r + u and mid = fl32(c), the kernel's
+// value differs from s - c by at most, with u = 2^-24 and first order in u,
+//   2 u q + 2 u r        a32 = fl32(a) in |a - c0|^2 and in 2 a.b'
+//   2 u q^2              a' = fl32(a32 - c0), rounded relative to itself
+//   u |kappa - mid| + u c  kappa - mid and mid rounded
+//   3 u (max(c, q^2) + |kappa|)  the three roundings of |a'|^2 + (kappa - mid)
+//   4 u r + 3 u |s - c|  the three fmas: every partial sum is the result plus
+//                        products that add up to at most 2 r
+//   2 u r                b' rounded relative to itself
+// and the chunk's deviation of kappa.  q^2 <= 1.1 c + 11 r^2 near the edge, so
+// the sum is u (2 sqrt(c) + 7.5 c + 10 r + 55 r^2 + 5 |kappa|) + deviation:
+// the first two terms here, the others per chunk.  The second edge of a
+// three-slot job adds 5 u c for its subtraction.  The terms 3 u |s - c| and
+// the growth of the bound with s are less than |s - c| itself by a factor 10
+// for c >= 1e-10 and lie within the 5% margin; smaller edges are never settled
+// in this form (infinite slack).  The FP64 predicate's own error (8 u64 s) and
+// the second-order terms are inside 1e-13 + the margin.
+double local_guard(double c) {
+    const double u = 5.9604644775390625e-08;  // 2^-24
+    if (!(c >= 1e-10)) return std::numeric_limits<double>::infinity();
+    return 1.05 * u * (2.0 * std::sqrt(c) + 12.5 * c) + 1e-13;
+}
+
 static float round_down_f(double x) {
     float f = (float)x;
     if ((double)f > x) f = std::nextafter(f, -INFINITY);
@@ -103,14 +130,13 @@ int build_table(const double* edges_deg, int K, BinTable* t) {
     Band bands[kMaxBins + 1];
     size_t n_bands = 0;
     for (int k = 0; k <= K; ++k) {
-        t->band[k][0] = t->band[k][1] = 0xFFFFFFFFu;
+        t->edge[k][0] = (float)t->c64[k];
+        t->edge[k][1] = round_up_f(0.5 * local_guard(t->c64[k]));
         if (t->c64[k] == 0.0) continue;
         Band b;
         guard_bounds(t->c64[k], &b.lo, &b.hi, nullptr);
         b.k = k;
         bands[n_bands++] = b;
-        t->band[k][0] = b.lo;
-        t->band[k][1] = b.hi;
     }
     // K >= 1 and the edges increase, so c_K > 0 and there is at least one band.
     t->h_top = bands[n_bands - 1].hi;

@@ -35,7 +35,7 @@ struct BinTable {
     int32_t n_lut;         // entries used
     int32_t n_complex;     // buckets holding more than one guard band
     double c64[kMaxBins + 1];            // FP64 squared-chord edges
-    uint32_t band[kMaxBins + 1][2];      // {lo_bits, hi_bits}: guard band of edge k (c_k > 0)
+    float edge[kMaxBins + 1][2];         // {fl32(c_k), half slack of the local form} (local_guard)
     uint32_t lut[kMaxLut][4];            // {lo_bits, hi_bits, slot_below, slot_above}
 };
 
@@ -63,6 +63,12 @@ struct Segment {
     long long item_offset;   // item of the count that global item item_begin is
     const unsigned* item_list;   // if set: the count's kept items (tile pairs not skipped)
     const float4* b_caps;    // bounding spheres of B's chunks of 32 sorted points, or null
+    const float4* a_caps;    // the same of A's chunks
+    const float* al;         // A's local coordinates (planar, al_stride apart)
+    long long al_stride;
+    const float2* b_kap;     // per chunk of B: kappa and half the slack (with b_caps)
+    const float* bl;         // B's local coordinates (planar, bl_stride apart; with b_caps)
+    long long bl_stride;
     int is_auto;
     int sorted64;            // bit 0 (a64), bit 1 (b64): in the spatial order, else original
 };
@@ -119,6 +125,9 @@ struct DeviceInfo {
 struct Prepared {
     const float4* p32 = nullptr;
     const float4* c32 = nullptr;   // bounding sphere of each chunk of 32 sorted points
+    const float2* kap = nullptr;   // kappa and half the slack of each chunk
+    const float* l32 = nullptr;    // coordinates relative to the chunk's centre (planar, l_stride)
+    long long l_stride = 0;
     const double* x64 = nullptr;   // FP64 SoA (stride), in the spatial order if sorted
     long long stride = 0;
     int sorted = 0;
@@ -135,17 +144,14 @@ int grid_for(const Variant* v, size_t smem, long long n_items, int sm_count, int
              int* grid);
 long long round_up(long long x, long long m);
 int check_cuda(cudaError_t e);
-size_t prepare_bytes(long long n, long long n_pad, int is_xyz);
-int prepare(const double* coords, long long n, long long n_pad, int is_xyz, int tag,
-            unsigned char* scratch, int sm_count, cudaStream_t st, Prepared* out);
 // The one or two catalogues of a count prepared together (b absent: nb = pb
 // = 0): one conversion and key launch, one sort of the na + nb points, one
-// gather into FP32 and FP64 copies with a's points at [0, pa) and b's at
-// [pa, pa + pb) (each catalogue tile-padded with sentinels of tags tag0 and
-// tag0 + 1: catalogues that a count may pair need different tags), one
-// launch for the chunk spheres of both.  scratch: prepare_joint_bytes(na, pa,
-// nb, pb); a and b may lie in its first 16 (na + nb) bytes (the FP32 copies,
-// written after both are read).
+// gather into FP32 and FP64 copies, chunk spheres and local coordinates with
+// a's points at [0, pa) and b's at [pa, pa + pb) (each catalogue tile-padded
+// with sentinels of tags tag0 and tag0 + 1: catalogues that a count may pair
+// need different tags).  scratch: prepare_joint_bytes(na, pa, nb, pb); a and b
+// may lie in its first 16 (na + nb) bytes (the FP32 copies, written after both
+// are read).
 size_t prepare_joint_bytes(long long na, long long pa, long long nb, long long pb);
 int prepare_joint(const double* a, long long na, long long pa, const double* b, long long nb,
                   long long pb, int is_xyz, int tag0, unsigned char* scratch, int sm_count,
@@ -172,14 +178,18 @@ int launch_radec_to_xyz(const double* coords, long long n, double* xyz, int sm_c
 // sizes[l] += points with label l (sizes zeroed by the caller).
 int launch_count_labels(const unsigned* lab, long long n, int n_labels,
                         unsigned long long* sizes, int sm_count, cudaStream_t st);
-// FP32 copies with region r's sorted points (positions src[r]..src[r+1]-1 of
-// order) from dst[r] on, sentinels up to dst[r+1]; dst[R] = n_pad.
+// FP32 copies, chunk spheres and local coordinates (out, laid out by
+// regions_layout) with region r's sorted points (positions
+// src[r]..src[r+1]-1 of order) from dst[r] on, sentinels up to dst[r+1];
+// dst[R] = n_pad.
 int launch_gather_regions(const double* x64, long long stride, const unsigned* order,
                           const long long* src, const long long* dst, int R, long long n_pad,
-                          float4* p32, int tag, int sm_count, cudaStream_t st);
-// Bounding sphere of every chunk of 32 positions (sentinels mark padding).
-int launch_chunk_caps(const float4* p32, long long n_pad, float4* c32, int sm_count,
-                      cudaStream_t st);
+                          int tag, int sm_count, cudaStream_t st, const Prepared& out);
+// The memory those copies take and their layout in it; the copies from
+// position pos (a multiple of the tile) on.
+size_t regions_bytes(long long n_pad);
+Prepared regions_layout(unsigned char* p, long long n_pad);
+Prepared tile_view(const Prepared& A, long long pos);
 // Skipping over a table of counts: kept items per count, then each count's
 // kept range and list written into segs, their number into *n_kept.
 int launch_cull_batch(const CullSeg* cs, int n_segs, long long total, double theta_top,
@@ -214,6 +224,7 @@ struct TraceRange {
 int validate_edges(const double* edges_deg, int K);
 void chord2_edges(const double* edges_deg, int K, double* c);
 double guard_half_width(double c);
+double local_guard(double c);
 void guard_bounds(double c, uint32_t* lo_bits, uint32_t* hi_bits, double* g);
 int build_table(const double* edges_deg, int K, BinTable* t);
 

@@ -147,13 +147,11 @@ int count_regions_impl(const double* cd, long long nd, const int* ld, const doub
     b2 += ((size_t)std::max(n_segs, 1) * 8 + 255) / 256 * 256;
     const size_t off_off = b2;
     b2 += ((size_t)4 * (R + 1) * 8 + 255) / 256 * 256;
-    size_t off_p32[2], off_c32[2], off_tc[2];
+    size_t off_copies[2], off_tc[2];
     for (int c = 0; c < 2; ++c) {
         const long long np = L[c].dst[R];
-        off_p32[c] = b2;
-        b2 += ((size_t)np * 16 + 255) / 256 * 256;
-        off_c32[c] = b2;
-        b2 += ((size_t)np / 32 * 16 + 255) / 256 * 256;
+        off_copies[c] = b2;
+        b2 += regions_bytes(np);
         off_tc[c] = b2;
         b2 += ((size_t)(np / T) * sizeof(TileCap) + 255) / 256 * 256;
     }
@@ -181,18 +179,14 @@ int count_regions_impl(const double* cd, long long nd, const int* ld, const doub
     TileCap* tcaps[2];
     for (int c = 0; c < 2 && !rc; ++c) {
         const long long np = L[c].dst[R];
-        float4* p32 = (float4*)(m2 + off_p32[c]);
-        float4* c32 = (float4*)(m2 + off_c32[c]);
-        tcaps[c] = (TileCap*)(m2 + off_tc[c]);
-        rc = launch_gather_regions(x64[c], n_of[c], order[c], d_off + (size_t)c * 2 * (R + 1),
-                                   d_off + (size_t)c * 2 * (R + 1) + (R + 1), R, np, p32, c,
-                                   di.sm_count, st);
-        if (!rc) rc = launch_chunk_caps(p32, np, c32, di.sm_count, st);
-        if (!rc && cull) rc = launch_tile_caps(p32, np, (int)T, np / T, tcaps[c], st);
-        P[c].p32 = p32;
-        P[c].c32 = c32;
+        P[c] = regions_layout(m2 + off_copies[c], np);
         P[c].x64 = x64[c];
         P[c].stride = n_of[c];
+        tcaps[c] = (TileCap*)(m2 + off_tc[c]);
+        rc = launch_gather_regions(x64[c], n_of[c], order[c], d_off + (size_t)c * 2 * (R + 1),
+                                   d_off + (size_t)c * 2 * (R + 1) + (R + 1), R, np, c,
+                                   di.sm_count, st, P[c]);
+        if (!rc && cull) rc = launch_tile_caps(P[c].p32, np, (int)T, np / T, tcaps[c], st);
     }
     std::vector<Segment> segs;
     std::vector<CullSeg> cs;
@@ -203,11 +197,7 @@ int count_regions_impl(const double* cd, long long nd, const int* ld, const doub
         const long long ta = (L[ca].dst[q.a + 1] - L[ca].dst[q.a]) / T;
         const long long tb = (L[cb].dst[q.b + 1] - L[cb].dst[q.b]) / T;
         const bool aut = q.kind != 1 && q.a == q.b;
-        Prepared A = P[ca], B = P[cb];
-        A.p32 += ta0 * T;
-        A.c32 += ta0 * T / 32;
-        B.p32 += tb0 * T;
-        B.c32 += tb0 * T / 32;
+        const Prepared A = tile_view(P[ca], ta0 * T), B = tile_view(P[cb], tb0 * T);
         const unsigned long long na = (unsigned long long)L[ca].n[q.a];
         const unsigned long long nb = (unsigned long long)L[cb].n[q.b];
         unsigned long long* c = counts + (((size_t)q.kind * R + q.a) * R + q.b) * K2;
