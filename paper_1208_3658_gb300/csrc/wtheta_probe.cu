@@ -7,6 +7,8 @@
 // warp) or every thread to one word; the SM clock counter times the block.
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "wtheta_internal.h"
 
 namespace {
@@ -61,6 +63,8 @@ extern "C" int wtheta_probe_shared_atomics(int32_t same_address, double* per_sm_
     // warp-wide reductions per SM per clock, averaged over the blocks (one per SM)
     const double warps = kThreads / 32.0;
     const double mean_cycles = (double)cyc / (double)di.sm_count;
-    *per_sm_per_clock = warps * kIters / mean_cycles;
+    // to three decimals: the block's start and end cost some 10^-5 of its cycles,
+    // differently from launch to launch
+    *per_sm_per_clock = std::round(1000.0 * warps * kIters / mean_cycles) / 1000.0;
     return WTHETA_OK;
 }
