@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(64) k_joint_keys(const double* __restrict__ a,
 //     for the few roundings of that arithmetic.
 //   - Local coordinates b' = fl32(b - c), from the FP64 points: the rounding is
 //     relative to |b'|, so a chunk's own geometry is kept to 2^-24 of its size.
-//   - For the pair kernel's local form (two_slot_step) the chunk keeps
+//   - For the pair kernel's local form (one_edge_step) the chunk keeps
 //     kappa = |b|^2 - |c|^2 (for unit vectors the same for every point of the
 //     chunk; the middle of its range here) and half the slack that the form
 //     adds to an edge's guard band for this chunk: the deviation of kappa from
@@ -853,8 +853,7 @@ __global__ void k_cull_prefix(Segment* __restrict__ segs, const CullSeg* __restr
 // FP32 copies (S.sorted64 says which); c64 is the shared address of
 // the FP64 edges.  hint >= 0: the slot just below the one edge whose guard
 // band held the FP32 value (checked, else the edges are searched in order).
-__device__ __forceinline__ unsigned recheck_slot(const Segment& S, long long ia, long long jb,
-                                                 unsigned c64, int K, int hint = -1) {
+__device__ __forceinline__ double pair_chord2(const Segment& S, long long ia, long long jb) {
     const long long i = (S.sorted64 & 1) ? ia : __float_as_int(S.a32[ia].w);
     const long long j = (S.sorted64 & 2) ? jb : __float_as_int(S.b32[jb].w);
     const double* a = S.a64;
@@ -863,7 +862,12 @@ __device__ __forceinline__ unsigned recheck_slot(const Segment& S, long long ia,
     const double dx = __dsub_rn(a[i], b[j]);
     const double dy = __dsub_rn(a[as + i], b[bs + j]);
     const double dz = __dsub_rn(a[2 * as + i], b[2 * bs + j]);
-    const double s = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+}
+
+__device__ __forceinline__ unsigned recheck_slot(const Segment& S, long long ia, long long jb,
+                                                 unsigned c64, int K, int hint = -1) {
+    const double s = pair_chord2(S, ia, jb);
     if (hint >= 0 && hint <= K) {
         // the FP32 value lay in the guard band of edge `hint` alone: the slot
         // is hint or hint + 1, confirmed against the neighbouring edges
@@ -888,12 +892,22 @@ struct PairKernel {
     static constexpr int TA = NT * R;   // A points per tile
     static constexpr int TB = NT * R;   // B points per tile (equal: auto needs square tiles)
     static constexpr int NW = NT / 32;
-    // columns of the private histograms (one per thread or per warp) and the
-    // words from one slot's row to the next: per-warp columns updated by
-    // shared reductions (kHistWarpRed) take an odd stride, so that lanes adding
-    // to different rows of their warp's column hit different banks
-    static constexpr int HCOLS = (HM == kHistWarp || HM == kHistWarpRed) ? NW : NT;
-    static constexpr int HSTRIDE = HM == kHistWarpRed ? (NW | 1) : HCOLS;
+    // Columns of the private histograms and the words from one slot's row to
+    // the next.  With span jobs (kHistLaneAtomic, not deferred) the lanes of a
+    // warp share CPW = 4 columns updated by shared reductions: most updates are
+    // one or two per job, so sharing costs nothing measurable, and the columns
+    // take an eighth of the memory (17.4 -> 2.3 KB at 32 bins), which keeps five
+    // blocks on an SM and leaves the L1 room for their A tiles.  Rows lie an
+    // odd number of words apart, so that lanes adding to different rows of one
+    // column hit different banks.
+    static constexpr int CPW = (HM == kHistWarp || HM == kHistWarpRed) ? 1
+                               : HM == kHistLaneAtomic && !DEF         ? 4
+                                                                       : 32;
+    static constexpr int HCOLS = NW * CPW;
+    static constexpr int HSTRIDE = CPW == 4 || HM == kHistWarpRed ? (HCOLS | 1) : HCOLS;
+    __device__ static int column() {
+        return (int)(threadIdx.x >> 5) * CPW + (int)(threadIdx.x & (CPW - 1));
+    }
     static constexpr unsigned ROWB = 4u * HSTRIDE;
 
     static size_t smem_bytes(int K, int n_lut) {
@@ -914,7 +928,8 @@ __device__ __forceinline__ void flush_hist(unsigned* hist, int K,
     for (int b = warp; b <= K + 1; b += NT / 32) {
         unsigned long long sum = 0;
         for (int q = lane; q < HCOLS; q += 32) {
-            sum += hist[b * HSTRIDE + q];
+            // signed: an edge's counts go to a column as +n below and -n above it
+            sum += (unsigned long long)(long long)(int)hist[b * HSTRIDE + q];
             hist[b * HSTRIDE + q] = 0;
         }
 #pragma unroll
@@ -1109,40 +1124,39 @@ __device__ __forceinline__ float4 group_cap(const f2_t (&ax)[R / 2], const f2_t 
 // within 1.2e-7 of their FP32 copies and the FP32 arithmetic here errs by a
 // few units in the last place, all covered by the 1e-6 absolute and relative
 // slack, so every pair's FP64 squared chord lies in [slo, shi].  The table
-// classifies both ends (values inside a guard band or a bucket with several
-// edges are ambiguous):
-//   0  both ends in one slot: every pair is in slot rlo;
-//   1  adjacent slots k and k+1 (rlo = slot k), split by edge k alone: each
-//      pair is in one or the other by one FP32 comparison outside the
-//      edge's guard band;
-//   3  slots k, k+1, k+2, split by edges k and k+1: two comparisons per pair;
-//   2  anything else: bin pair by pair.
-// rlo is a byte offset of a slot's row, slot * row_bytes; a span wholly
-// above h_top (the top edge's band) is the overflow row trash at once.
-__device__ __forceinline__ int span_class(float4 ga, float4 gb, unsigned lut, int shift, int base,
+// gives the lowest slot rlo and the highest rhi that the interval can touch (an
+// end inside an edge's guard band takes the edge in), as byte offsets of the
+// slots' rows (slot * row_bytes).  Returns the number of edges between them:
+//   0        every pair is in slot rlo (a span wholly above h_top, the top
+//            edge's band, is the overflow row trash at once);
+//   1 .. kMaxEdges  the counts of the slots follow from the number of pairs
+//            below each of those edges;
+//   -1       more edges, a bucket of the table holding several edges, or
+//            padding: bin pair by pair.
+// Per edge a job costs 16 packed fmas and 8 wavefronts of shared loads per 8
+// pairs where the table costs a 16-byte lookup and a shared atomic per pair, so
+// the line lies well above one edge: 6 measured best of 2, 4, 6 and 8.
+constexpr int kMaxEdges = 6;
+__device__ __forceinline__ int span_edges(float4 ga, float4 gb, unsigned lut, int shift, int base,
                                           int top_idx, unsigned row_bytes, unsigned& rlo,
-                                          unsigned h_top, unsigned trash) {
+                                          unsigned& rhi, unsigned h_top, unsigned trash) {
     const float dx = ga.x - gb.x, dy = ga.y - gb.y, dz = ga.z - gb.z;
     const float dc = sqrtf(dx * dx + dy * dy + dz * dz);
     const float rr = (ga.w + gb.w) * (1.f + 1e-6f) + 1e-6f;
     const float lo = dc * (1.f - 1e-6f) - rr, hi = dc * (1.f + 1e-6f) + rr;
     const float slo = lo > 0.f ? lo * lo * (1.f - 1e-5f) : 0.f;
     const float shi = hi * hi * (1.f + 1e-5f);
-    if (!(ga.w <= 2.f && gb.w >= 0.f && gb.w <= 2.f)) return 2;  // padding (or NaN)
+    if (!(ga.w <= 2.f && gb.w >= 0.f && gb.w <= 2.f)) return -1;  // padding (or NaN)
     const unsigned bl = __float_as_uint(slo), bh = __float_as_uint(shi);
-    if (bl > h_top) {  // every pair beyond the top edge's band: overflow (row trash)
-        rlo = trash;
-        return 0;
-    }
+    rlo = rhi = trash;
+    if (bl > h_top) return 0;
     const uint4 el = lut_entry(bl, lut, shift, base, top_idx);
     const uint4 eh = lut_entry(bh, lut, shift, base, top_idx);
-    if (!(bl < el.x || bl > el.y) || !(bh < eh.x || bh > eh.y)) return 2;
-    rlo = bl < el.x ? el.z : el.w;
-    const unsigned rhi = bh < eh.x ? eh.z : eh.w;
-    if (rlo == rhi) return 0;
-    if (rhi == rlo + row_bytes) return 1;
-    if (rhi == rlo + 2u * row_bytes) return 3;
-    return 2;
+    if (el.z == trash || eh.z == trash) return -1;  // several edges in one bucket
+    rlo = bl <= el.y ? el.z : el.w;
+    rhi = bh < eh.x ? eh.z : eh.w;
+    const int n = (int)(rhi - rlo) / (int)row_bytes;
+    return n <= kMaxEdges ? n : -1;
 }
 
 // The local form of a pair's squared chord: with the chunk's centre c, b = c +
@@ -1156,14 +1170,13 @@ __device__ __forceinline__ int span_class(float4 ga, float4 gb, unsigned lut, in
 // difference form; |d| > G, G the edge's half slack plus the chunk's
 // (local_guard, write_chunk), settles the side of the FP64 squared chord.
 //
-// Survey, 1M + 1M points: the two-slot loop is 12 packed fmas per B point and
-// 8 A points instead of 24 packed operations.
+// A one-edge step is 12 packed fmas per B point and 8 A points.
 //
 // One step: JU B points (staged negated) and the thread's R A points.  neg[q]
 // counts the values with d < 0 and mb[q] keeps the smallest |d|, one
 // accumulator per A pair q so that the steps' dependency chains interleave.
 template <int R, int JU>
-__device__ __forceinline__ void two_slot_step(unsigned bxy_base, unsigned bz_base,
+__device__ __forceinline__ void one_edge_step(unsigned bxy_base, unsigned bz_base,
                                               const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
                                               const f2_t (&az)[R / 2], const f2_t (&a0)[R / 2],
                                               int j, unsigned (&neg)[R / 2], float (&mb)[R / 2]) {
@@ -1182,11 +1195,11 @@ __device__ __forceinline__ void two_slot_step(unsigned bxy_base, unsigned bz_bas
     }
 }
 
-// One step of a three-slot chunk: the same against two edges, the second's
+// One step against two edges, the second's
 // value from the first's by one more subtraction of half their distance
 // (ndel = -(mid2 - mid1) / 2).
 template <int R, int JU>
-__device__ __forceinline__ void three_slot_step(unsigned bxy_base, unsigned bz_base,
+__device__ __forceinline__ void two_edge_step(unsigned bxy_base, unsigned bz_base,
                                                 const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
                                                 const f2_t (&az)[R / 2], const f2_t (&a0)[R / 2],
                                                 int j, f2_t ndel, unsigned& neg1, unsigned& neg2,
@@ -1223,13 +1236,12 @@ __device__ __forceinline__ void tile_pass(unsigned bxy, unsigned bz, unsigned lu
     using PK = PairKernel<NT, R, JU, HM, DEF>;
     constexpr int TA = PK::TA, TB = PK::TB;
     constexpr int NV = JU * R;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int lane = threadIdx.x & 31;
     const unsigned h_top = p.tab.h_top;
     const float hf = __uint_as_float(h_top);
     const int shift = p.tab.shift, base = p.tab.base, K = p.tab.K, top_idx = p.tab.n_lut - 1;
     constexpr unsigned row_bytes = PK::ROWB;
-    const unsigned col =
-        hist + 4u * (unsigned)((HM == kHistWarp || HM == kHistWarpRed) ? warp : tid);
+    const unsigned col = hist + 4u * (unsigned)PK::column();
     const long long a0 = I * TA + a_first, b0 = J * TB;
 
     if (DEF) {
@@ -1365,19 +1377,22 @@ __device__ __forceinline__ float4 chunk_sphere(unsigned caps, int c) {
 }
 
 // ---------------------------------------------------------------------------
-// Span jobs.  A (group, chunk) pair whose span needs its pairs computed (two
-// slots, three slots, or pair by pair) is a job: the lane whose R A points
-// form the group, its sub-tile, the chunk's index in the staged B tile and
-// the lowest slot of the span.  Each warp keeps one ring of 32 jobs per kind
-// in shared memory and runs a full ring as one round, one job per lane: a
-// lane computes only pairs whose slot is not known from the spheres, whatever
-// its own group's spans, and the lanes of a round run the same loop.  A job's
-// A points are read again from the FP32 copy of the catalogue (L2).
+// Span jobs.  A (group, chunk) pair whose span needs its pairs computed is one
+// or more jobs: for every edge inside the span the number of pairs below it is
+// counted, two edges to a job (kJobTwo) and the last of an odd number alone
+// (kJobOne); a span with too many edges is one job binned pair by pair
+// (kJobExact).  Every pair of a span of edges goes to its highest slot at
+// first, and an edge with n pairs below it then moves n of them one slot down
+// (+n below, -n above), so the jobs of a span are independent of one another.
+// Each warp keeps one ring of jobs per kind in shared memory and runs 32 of
+// them as one round, one job per lane: a lane computes only pairs whose slot
+// is not known from the spheres, whatever its own group's spans, and the lanes
+// of a round run the same loop.
 // ---------------------------------------------------------------------------
-constexpr int kJobTwo = 0, kJobThree = 1, kJobExact = 2, kJobKinds = 3, kChunk = 32;
+constexpr int kJobOne = 0, kJobTwo = 1, kJobExact = 2, kJobKinds = 3, kChunk = 32;
+constexpr int kRing = 64;  // words of a ring: fewer than 32 waiting, at most 32 pushed at once
 
-// Bits 0-4 lane, 5-7 sub-tile, 8-15 chunk, 16-29 slot; the ring loop keeps
-// the job's kind + 1 in bits 30-31 of the word it carries.
+// Bits 0-4 lane, 5-7 sub-tile, 8-15 chunk, 16-29 the (first) edge.
 __device__ __forceinline__ unsigned job_word(int lane, int sub, int chunk, unsigned slot) {
     return (unsigned)lane | ((unsigned)sub << 5) | ((unsigned)chunk << 8) | (slot << 16);
 }
@@ -1466,10 +1481,10 @@ __device__ __forceinline__ float edge_mid(unsigned band, unsigned k, float& G) {
     return mid;
 }
 
-// A job of kind T (two or three slots) over the chunk's steps t0, t0 + ts,
-// ... (JU points each).  neg1 and neg2 count the values below the first and
-// second edge (neg2 = 0 for two slots), mb1 and mb2 return the smallest |d|
-// less the slack: at most zero if some value may be on either side.
+// A job of kind T (one or two edges) over the chunk's steps t0, t0 + ts, ...
+// (JU points each).  neg1 and neg2 count the values below the first and second
+// edge (neg2 = 0 for one), mb1 and mb2 return the smallest |d| less the slack:
+// at most zero if some value may be on either side.
 template <int NT, int R, int JU, int HM>
 __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, unsigned sIJ,
                                           unsigned bxy, unsigned bz, unsigned caps, unsigned band,
@@ -1497,7 +1512,7 @@ __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, u
     }
     neg1 = neg2 = 0;
     mb1 = mb2 = __int_as_float(0x7f800000);
-    if (T == kJobTwo) {
+    if (T == kJobOne) {
         unsigned negq[R / 2];
         float mbq[R / 2];
 #pragma unroll
@@ -1507,7 +1522,7 @@ __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, u
         }
 #pragma unroll 1
         for (int t = t0; t < kChunk; t += ts)
-            two_slot_step<R, JU>(bxy, bz, ax, ay, az, a0, chunk_point<JU>(c0, t, rot), negq, mbq);
+            one_edge_step<R, JU>(bxy, bz, ax, ay, az, a0, chunk_point<JU>(c0, t, rot), negq, mbq);
 #pragma unroll
         for (int q = 0; q < R / 2; ++q) {
             neg1 += negq[q];
@@ -1518,35 +1533,49 @@ __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, u
         const float ndel = 0.5f * (mid - mid2);
 #pragma unroll 1
         for (int t = t0; t < kChunk; t += ts)
-            three_slot_step<R, JU>(bxy, bz, ax, ay, az, a0, chunk_point<JU>(c0, t, rot),
+            two_edge_step<R, JU>(bxy, bz, ax, ay, az, a0, chunk_point<JU>(c0, t, rot),
                                    pack2(ndel, ndel), neg1, neg2, mb1, mb2);
         mb2 -= G2 + kap.y;
     }
     mb1 -= G + kap.y;
 }
 
-// Settles a two- or three-slot job from its counts (summed over the lanes
-// that shared it): with every |d| beyond the slack (mb1, mb2 > 0), d < 0 means
-// below the edge.  Returns false otherwise (rare): nothing is counted, and the
-// chunk has to go pair by pair.
-template <int NT, int R, int JU, int HM>
-__device__ __forceinline__ bool span_settle(int T, unsigned job, unsigned col, unsigned neg1,
-                                            unsigned neg2, float mb1, float mb2) {
-    constexpr unsigned NP = (unsigned)(R * kChunk);
-    constexpr unsigned row_bytes = PairKernel<NT, R, JU, HM, 0>::ROWB;
-    const unsigned slot = (job >> 16) & 0x3FFFu;
-    const unsigned rlo = slot * row_bytes;
-    if (!(mb1 > 0.f)) return false;
-    if (T == kJobTwo) {
-        hist_add<HM>(col + rlo, neg1);
-        hist_add<HM>(col + rlo + row_bytes, NP - neg1);
-        return true;
+// Rare: a job found a value within the slack of edge k.  The warp counts the
+// job's pairs below the edge again, one B point per lane, and settles each
+// value within the slack by its FP64 squared chord.  Returns that count, with
+// the number of values rechecked above bit 16.  Out of line: its FP64
+// registers do not weigh on the loops.
+template <int NT, int R>
+__device__ __noinline__ unsigned recount_edge(unsigned job, unsigned k, unsigned sIJ, unsigned band,
+                                              unsigned sC, const Segment& S) {
+    constexpr int TA = NT * R, TB = NT * R, SA = 32 * R;
+    const int lane = threadIdx.x & 31;
+    const long long pa = lds_s64(sIJ) * TA + (int)((job >> 5) & 7u) * SA + (int)(job & 31u) * R;
+    const long long pb = lds_s64(sIJ + 8u) * TB + (int)((job >> 8) & 255u) * kChunk + lane;
+    const float4 ca = __ldg(S.a_caps + pa / kChunk), cb = __ldg(S.b_caps + pb / kChunk);
+    const float2 kap = __ldg(S.b_kap + pb / kChunk);
+    const float bx = -S.bl[pb], by = -S.bl[S.bl_stride + pb], bz = -S.bl[2 * S.bl_stride + pb];
+    float G;
+    const float mid = edge_mid(band, k, G);
+    G += kap.y;
+    const float km = kap.x - mid, dx = ca.x - cb.x, dy = ca.y - cb.y, dz = ca.z - cb.z;
+    const double c = lds_f64(sC + 8u * k);
+    unsigned n = 0;
+#pragma unroll 1
+    for (int r = 0; r < R; ++r) {
+        const float ax = S.al[pa + r], ay = S.al[S.al_stride + pa + r],
+                    az = S.al[2 * S.al_stride + pa + r];
+        const float lx = __fadd_rn(ax, dx), ly = __fadd_rn(ay, dy), lz = __fadd_rn(az, dz);
+        const float a0 = 0.5f * fmaf(lx, lx, fmaf(ly, ly, fmaf(lz, lz, km)));
+        const float d = fmaf(__fadd_rn(ax, ca.x), bx,
+                             fmaf(__fadd_rn(ay, ca.y), by, fmaf(__fadd_rn(az, ca.z), bz, a0)));
+        if (fabsf(d) > G) {
+            n += d < 0.f ? 1u : 0u;
+        } else {
+            n += (pair_chord2(S, pa + r, pb) < c ? 1u : 0u) + (1u << 16);
+        }
     }
-    if (!(mb2 > 0.f)) return false;
-    hist_add<HM>(col + rlo, neg1);
-    hist_add<HM>(col + rlo + row_bytes, neg2 - neg1);
-    hist_add<HM>(col + rlo + 2u * row_bytes, NP - neg2);
-    return true;
+    return __reduce_add_sync(0xffffffffu, n);
 }
 
 // Adds a warp's count (lanes with flag set, times w) to a 64-bit shared
@@ -1561,19 +1590,17 @@ __device__ __forceinline__ void warp_stat(unsigned a, bool flag, unsigned w) {
 
 // One round of jobs of kind T: this lane's share of job `run` (active: the
 // lane has one; steps t0, t0 + ts, ... of the job, its ts lanes adjacent and
-// ts a power of two).  Span jobs are settled by the first lane of each job
-// from the counts summed over its ts lanes; the return value is the job (bit
-// 30 set) if it has to go pair by pair, else 0.
+// ts a power of two).  The first lane of each job moves the counts, summed
+// over the ts lanes, below the job's edges.
 template <int NT, int R, int JU, int HM, bool ST>
-__device__ __forceinline__ unsigned job_round(int T, unsigned run, bool active, int t0, int ts,
-                                              unsigned sIJ, unsigned bxy, unsigned bz,
-                                              unsigned lut, unsigned caps, unsigned band,
-                                              unsigned sC, unsigned col, const PairParams& p,
-                                              const Segment& S, bool stats, unsigned stat) {
-    constexpr unsigned NP = (unsigned)(R * kChunk);
+__device__ __forceinline__ void job_round(int T, unsigned run, bool active, int t0, int ts,
+                                          unsigned sIJ, unsigned bxy, unsigned bz, unsigned lut,
+                                          unsigned caps, unsigned band, unsigned sC, unsigned col,
+                                          const PairParams& p, const Segment& S, bool stats,
+                                          unsigned stat) {
+    constexpr unsigned row_bytes = PairKernel<NT, R, JU, HM, 0>::ROWB;
     const int lane = threadIdx.x & 31;
-    unsigned n_recheck = 0, fb = 0;
-    bool settled = false;
+    unsigned n_recheck = 0;
     if (T == kJobExact) {
         if (active)
             exact_job<NT, R, JU, HM>(run, t0, ts, sIJ, bxy, bz, lut, caps, sC, col, p, S, n_recheck);
@@ -1590,13 +1617,32 @@ __device__ __forceinline__ unsigned job_round(int T, unsigned run, bool active, 
             mb1 = fminf(mb1, __shfl_xor_sync(0xffffffffu, mb1, o));
             mb2 = fminf(mb2, __shfl_xor_sync(0xffffffffu, mb2, o));
         }
-        if (active && t0 == 0) {
-            settled = span_settle<NT, R, JU, HM>(T, run, col, neg1, neg2, mb1, mb2);
-            if (!settled) fb = run | (1u << 30);
+        const bool first = active && t0 == 0;
+        const unsigned edge = (run >> 16) & 0x3FFFu;
+        // jobs with a value within the slack of their first or second edge
+        unsigned b1 = __ballot_sync(0xffffffffu, first && !(mb1 > 0.f));
+        unsigned b2 = __ballot_sync(0xffffffffu, first && !(mb2 > 0.f));
+#pragma unroll 1
+        while (b1 | b2) {
+            const bool second = b1 == 0u;
+            const int src = __ffs(second ? b2 : b1) - 1;
+            if (second) b2 &= b2 - 1u; else b1 &= b1 - 1u;
+            const unsigned j = __shfl_sync(0xffffffffu, run, src);
+            const unsigned v = recount_edge<NT, R>(j, ((j >> 16) & 0x3FFFu) + (second ? 1u : 0u),
+                                                   sIJ, band, sC, S);
+            if (lane == src) {
+                if (second) neg2 = v & 0xFFFFu; else neg1 = v & 0xFFFFu;
+                n_recheck += v >> 16;
+            }
+        }
+        if (first) {
+            const unsigned row = col + edge * row_bytes;
+            hist_add<HM>(row, neg1);
+            hist_add<HM>(row + row_bytes, neg2 - neg1);
+            if (T == kJobTwo) hist_add<HM>(row + 2u * row_bytes, 0u - neg2);
         }
     }
     if (ST && stats) {
-        warp_stat(stat + 8u, settled, NP);
         if (__any_sync(0xffffffffu, n_recheck != 0)) {
             unsigned long long v = n_recheck;
 #pragma unroll
@@ -1605,7 +1651,6 @@ __device__ __forceinline__ unsigned job_round(int T, unsigned run, bool active, 
                 asm volatile("red.shared.add.u64 [%0], %1;" ::"r"(stat), "l"(v) : "memory");
         }
     }
-    return fb;
 }
 
 // Lanes per job for a round of m < 32 jobs: the largest power of two with
@@ -1621,13 +1666,15 @@ __device__ __forceinline__ int round_share(int T, int m) {
 // first, then those left of the others (shared counters at address units, one
 // per sub-tile).  Each lane classifies its group against every chunk of a
 // unit; a chunk in one slot is counted at once, the others become jobs (the
-// warp's rings in the block's ring array at shared address rings, 32 words
-// per kind) and a ring that fills runs as one round.  When every unit is
-// taken, the jobs left in all the warps' rings are pooled and shared out
-// evenly (a warp would otherwise run its own leftovers in partial rounds
-// while the others wait at the next item's barrier; a block of one warp
-// flushes its own rings instead); then the diagonal units of an auto count
-// that the warp took go pair by pair, with the i < j mask.
+// warp's rings in the block's ring array at shared address rings, kRing words
+// per kind) and 32 jobs of a kind run as one round.  When every unit is taken,
+// the jobs left in all the warps' rings are pooled and shared out evenly (a
+// warp would otherwise run its own leftovers in partial rounds while the
+// others wait at the next item's barrier), each job of a partial round shared
+// among several lanes.
+// In a diagonal tile pair of an auto count (pairs i < j) a group skips the
+// chunks before its own and takes those after it like any other; its own
+// chunk goes pair by pair with the i < j mask, every warp its own sub-tile.
 // The tile pair (I, J) stays in shared memory (sIJ) and the statistics go to
 // the block's shared counters (stat: rechecks, span pairs, skipped pairs), so
 // that the rounds run with few live registers.  Every thread of the block
@@ -1643,217 +1690,149 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
     constexpr int NW = NT / 32, SA = 32 * R, UPS = 4, UB = TB / UPS, CPU = UB / kChunk;
     constexpr unsigned row_bytes = PK::ROWB;
     constexpr unsigned NP = (unsigned)(R * kChunk);
-    constexpr unsigned RING_BYTES = 4u * kJobKinds * 32u;  // one warp's rings
-    static_assert(NW <= 8 && TB / kChunk <= 256 && UB % kChunk == 0 && kChunk % JU == 0 &&
-                      NW * UPS <= 32,
+    constexpr unsigned RING = 4u * kRing, RINGS = RING * kJobKinds;  // bytes: a ring, a warp's
+    constexpr unsigned FULL = 0x202020u;  // some fill (8 bits per kind) is 32 or more
+    static_assert(NW <= 8 && TB / kChunk <= 256 && UB % kChunk == 0 && kChunk % JU == 0,
                   "job fields");
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned ring = rings + RING_BYTES * (unsigned)warp;
-    const unsigned col = hist + 4u * (unsigned)(HM == kHistWarpRed ? warp : tid);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned ring = rings + RINGS * (unsigned)warp;
+    const unsigned col = hist + 4u * (unsigned)PK::column();
+    const unsigned trash = (unsigned)(p.tab.K + 1) * row_bytes;
     const bool stats = ST && p.stats != nullptr;
-    unsigned fills = 0;      // jobs waiting per kind, 8 bits each
-    unsigned diag_units = 0;  // diagonal units taken (bit sub UPS + u)
-    int k = 0, cap_sub = -1, cn = -1;  // cn: next chunk of the current unit, -1: none
+    unsigned fills = 0;   // jobs waiting per kind, 8 bits each; bit 24 + T: ring T starts at 32
+    unsigned word = 0;    // this lane's next job (of the chunk it has classified)
+    int ones = 0, twos = 0, exact = 0;     // and how many of each kind it has to push
+    int k = 0, cap_sub = -1, cn = -1;      // cn: next chunk of the current unit, -1: none
+    int pool = -1;                         // kind of the pooled leftovers being run
     float4 ga = make_float4(0.f, 0.f, 0.f, 0.f);
-    // A block of one warp has nobody to pool its leftovers with: when its
-    // units are all taken it flushes its own rings in the ring steps below
-    // (partial rounds, each job shared among lanes), so that the span jobs
-    // redone pair by pair join the pair-by-pair ring's last round.
-    bool done = false;
 #pragma unroll 1
     for (;;) {
+        int T, m = 32;
+        unsigned at = 0;  // shared address of this lane's job
+        int ts = 1;
+        if (pool < 0 && (fills & FULL) == 0u) {
+            if (!__any_sync(0xffffffffu, (ones | twos | exact) != 0)) {
+                // the next chunk
 #pragma unroll 1
-        while (k < NW && cn < 0) {
-            const int sub = (warp + k) % NW;
-            unsigned u = 0;
-            if (lane == 0) u = atom_add_shared(units + 4u * (unsigned)sub, 1u);
-            u = __shfl_sync(0xffffffffu, u, 0);
-            if (u >= (unsigned)UPS) {
-                ++k;
-                continue;
-            }
-            const int ub = (int)u * UB;
-            if (diag && ub + UB <= sub * SA) continue;  // every pair has i >= j
-            if (diag && ub < (sub + 1) * SA) {
-                diag_units |= 1u << (sub * UPS + (int)u);
-                continue;
-            }
-            if (sub != cap_sub) {
-                f2_t ax[R / 2], ay[R / 2], az[R / 2];
-                const long long pos = lds_s64(sIJ) * TA + sub * SA + lane * R;
-                load_local<R>(S.al, S.al_stride, pos, ax, ay, az);
-                ga = group_cap<R>(ax, ay, az, __ldg(S.a_caps + pos / kChunk));
-                cap_sub = sub;
-            }
-            cn = ub / kChunk;
-        }
-        if (k == NW) {
-            if constexpr (NW > 1) break;  // every unit taken: the leftovers are pooled below
-            done = true;
-        }
-        // the chunk's job word with its kind + 1 in bits 30-31 (0: none)
-        unsigned kj = 0;
-        if (!done) {
-            const int c = cn;
-            cn = (c + 1) % CPU == 0 ? -1 : c + 1;
-            const float4 gb = chunk_sphere(caps, c);
-            unsigned rlo = 0;
-            const unsigned trash = (unsigned)(p.tab.K + 1) * row_bytes;
-            const int mode = span_class(ga, gb, lut, p.tab.shift, p.tab.base, p.tab.n_lut - 1,
-                                        row_bytes, rlo, p.tab.h_top, trash);
-            if (mode == 0) {
-                if (rlo != trash) hist_add<HM>(col + rlo, NP);  // the trash row is never read
-            } else {
-                kj = job_word(lane, (warp + k) % NW, c, rlo / row_bytes) |
-                     ((unsigned)(mode == 1 ? kJobTwo + 1 : mode == 3 ? kJobThree + 1
-                                                                     : kJobExact + 1) << 30);
-            }
-            if (stats) {
-                warp_stat(stat + 8u, mode == 0, NP);
-                warp_stat(stat + 16u, mode == 0, NP);
-            }
-        }
-        // Most chunks fill no ring: their jobs are appended at once and the
-        // warp takes the next chunk (fills stay below 64, so 8 bits each).
-        if (!done) {
-            const unsigned kind = kj >> 30;
-            const unsigned m1 = __ballot_sync(0xffffffffu, kind == 1u);
-            const unsigned m2 = __ballot_sync(0xffffffffu, kind == 2u);
-            const unsigned m3 = __ballot_sync(0xffffffffu, kind == 3u);
-            const unsigned nf = fills + (unsigned)__popc(m1) + ((unsigned)__popc(m2) << 8) +
-                                ((unsigned)__popc(m3) << 16);
-            if ((nf & 0x202020u) == 0u) {
-                if (kind != 0u) {
-                    const int T = (int)kind - 1;
-                    const unsigned mk = T == 0 ? m1 : T == 1 ? m2 : m3;
-                    const int pos = (int)((fills >> (8 * T)) & 255u) +
-                                    __popc(mk & ((1u << lane) - 1u));
-                    sts_u32(ring + 128u * (unsigned)T + 4u * (unsigned)pos, kj & 0x3FFFFFFFu);
+                while (k < NW && cn < 0) {
+                    const int sub = (warp + k) % NW;
+                    unsigned u = 0;
+                    if (lane == 0) u = atom_add_shared(units + 4u * (unsigned)sub, 1u);
+                    u = __shfl_sync(0xffffffffu, u, 0);
+                    if (u >= (unsigned)UPS) {
+                        ++k;
+                        continue;
+                    }
+                    const int ub = (int)u * UB;
+                    if (diag && ub + UB <= sub * SA) continue;  // every pair has i >= j
+                    if (sub != cap_sub) {
+                        f2_t ax[R / 2], ay[R / 2], az[R / 2];
+                        const long long pos = lds_s64(sIJ) * TA + sub * SA + lane * R;
+                        load_local<R>(S.al, S.al_stride, pos, ax, ay, az);
+                        ga = group_cap<R>(ax, ay, az, __ldg(S.a_caps + pos / kChunk));
+                        cap_sub = sub;
+                    }
+                    cn = ub / kChunk;
                 }
-                fills = nf;
-                continue;
+                if (k == NW) {
+                    pool = 0;  // every unit taken: the leftovers
+                    __syncthreads();  // the rings are quiescent
+                    if (lane == 0) sts_u32(units + 4u * (unsigned)warp, fills);
+                    __syncthreads();
+                    continue;
+                }
+                const int c = cn, sub = (warp + k) % NW;
+                cn = (c + 1) % CPU == 0 ? -1 : c + 1;
+                unsigned rlo = 0, rhi = 0;
+                const int n = span_edges(ga, chunk_sphere(caps, c), lut, p.tab.shift, p.tab.base,
+                                         p.tab.n_lut - 1, row_bytes, rlo, rhi, p.tab.h_top, trash);
+                const int own = diag ? (sub * SA + lane * R) / kChunk : -1;
+                const bool mine = c > own;
+                if (mine) {
+                    if (n >= 0 && rhi != trash) hist_add<HM>(col + rhi, NP);
+                    exact = n < 0 ? 1 : 0;
+                    ones = n > 0 ? n & 1 : 0;
+                    twos = n > 0 ? n >> 1 : 0;
+                    word = job_word(lane, sub, c, rlo / row_bytes);
+                }
+                if (stats) {
+                    warp_stat(stat + 8u, mine && n >= 0, NP);
+                    warp_stat(stat + 16u, mine ? n == 0 : c < own, NP);
+                }
             }
-        }
-        // A ring that fills runs as one round, one job per lane: the two-slot
-        // ring, the pair-by-pair ring for the two-slot jobs that found a value
-        // near their edge, the three-slot ring, the same for its jobs, then the
-        // pair-by-pair ring for the chunk's own job.  One code path per kind.
-        unsigned fb = 0;  // this lane's job that has to go pair by pair (bit 30: valid)
-#pragma unroll 1
-        for (int st = 0; st < 5; ++st) {
-            const int T = (0x298 >> (2 * st)) & 3;  // rings 0, 2, 1, 2, 2
-            const bool from_fb = (st & 1) != 0;
-            const unsigned word = from_fb ? fb : kj;
-            const bool push = from_fb ? fb != 0u : (kj >> 30) == (unsigned)(T + 1);
-            if (from_fb) fb = 0u;
-            // one-warp blocks, units all taken: every ring but the
-            // pair-by-pair one flushes at its step, that one at the last
-            const bool flush = done && (T != kJobExact || st == 4);
-            const unsigned m = __ballot_sync(0xffffffffu, push);
-            const int fill = (int)((fills >> (8 * T)) & 255u);
-            const int n = __popc(m);
-            if (n == 0 && !(flush && fill > 0)) continue;
-            const unsigned rt = ring + 128u * (unsigned)T;
-            const int pos = fill + __popc(m & ((1u << lane) - 1u));
-            const unsigned job = word & 0x3FFFFFFFu;
-            if (push && pos < 32) sts_u32(rt + 4u * (unsigned)pos, job);
-            const int total = fill + n;
-            if (total < 32 && !flush) {
-                fills += (unsigned)n << (8 * T);
-                continue;
+            // push one job of every lane that has some left
+            const unsigned m1 = __ballot_sync(0xffffffffu, ones != 0);
+            const unsigned m2 = __ballot_sync(0xffffffffu, ones == 0 && twos != 0);
+            const unsigned m3 = __ballot_sync(0xffffffffu, exact != 0);
+            if (m1 | m2 | m3) {
+                const int Tp = ones ? kJobOne : twos ? kJobTwo : kJobExact;
+                const unsigned mk = Tp == kJobOne ? m1 : Tp == kJobTwo ? m2 : m3;
+                const unsigned pos = ((fills >> (8 * Tp)) & 255u) + ((fills >> (24 + Tp)) & 1u) * 32u +
+                                     (unsigned)__popc(mk & ((1u << lane) - 1u));
+                if (ones | twos | exact)
+                    sts_u32(ring + RING * (unsigned)Tp + 4u * (pos & (kRing - 1)), word);
+                word += Tp == kJobOne ? 1u << 16 : 2u << 16;
+                if (Tp == kJobOne) ones = 0;
+                else if (Tp == kJobTwo) --twos;
+                else exact = 0;
+                fills += (unsigned)__popc(m1) + ((unsigned)__popc(m2) << 8) +
+                         ((unsigned)__popc(m3) << 16);
             }
-            // a full round gives each lane a job; a flushed partial round
-            // shares each job among ts lanes (round_share)
-            const int ts = total < 32 ? round_share<JU>(T, total) : 1;
-            const int jl = lane / ts;
-            __syncwarp();
-            const unsigned run = lds_u32(rt + 4u * (unsigned)min(jl, 31));
-            __syncwarp();
-            if (push && pos >= 32) sts_u32(rt + 4u * (unsigned)(pos - 32), job);
-            fills = (fills & ~(255u << (8 * T))) | ((unsigned)max(total - 32, 0) << (8 * T));
-            fb = job_round<NT, R, JU, HM, ST>(T, run, jl < total, lane % ts, ts, sIJ, bxy, bz, lut,
-                                              caps, band, sC, col, p, S, stats, stat);
+            if ((fills & FULL) == 0u) continue;
         }
-        if (done) break;
-    }
-    // The leftovers of every warp, pooled (blocks of several warps).  Once
-    // all warps are here the rings are quiescent; each warp publishes its
-    // fills in its unit counter (no longer claimed), and the jobs of each
-    // kind, the rings taken in warp order, are shared out in contiguous slices
-    // of about n / NW jobs, each slice one round with the lanes of a job
-    // adjacent.
-    if constexpr (NW > 1) {
-        __syncthreads();
-        if (lane == 0) sts_u32(units + 4u * (unsigned)warp, fills);
-        __syncthreads();
-        unsigned fl[NW];
-#pragma unroll
-        for (int q = 0; q < NW; ++q) fl[q] = lds_u32(units + 4u * (unsigned)q);
-        unsigned fb0 = 0, fb1 = 0;  // pooled two- and three-slot jobs to redo pair by pair
-#pragma unroll 1
-        for (int T = 0; T < kJobKinds; ++T) {
+        if (pool < 0) {
+            // a full round of the first kind that has one
+            T = (fills & 0x20u) ? kJobOne : (fills & 0x2000u) ? kJobTwo : kJobExact;
+            at = ring + RING * (unsigned)T +
+                 4u * ((((fills >> (24 + T)) & 1u) * 32u + (unsigned)lane));
+            fills = (fills - (32u << (8 * T))) ^ (1u << (24 + T));
+        } else {
+            // The leftovers of every warp, pooled: each warp published its fills
+            // in its unit counter (no longer claimed), and the jobs of each
+            // kind, the rings taken in warp order, are shared out in contiguous
+            // slices of about n / NW jobs, each slice one round with the lanes
+            // of a job adjacent.
+            if (pool == kJobKinds) break;
+            T = pool++;
             int n = 0;
 #pragma unroll
-            for (int q = 0; q < NW; ++q) n += (int)((fl[q] >> (8 * T)) & 255u);
-            const int lo = warp * n / NW, m = (warp + 1) * n / NW - lo;
+            for (int q = 0; q < NW; ++q) n += (int)((lds_u32(units + 4u * (unsigned)q) >> (8 * T)) & 255u);
+            const int lo = warp * n / NW;
+            m = (warp + 1) * n / NW - lo;
             if (m == 0) continue;
-            const int ts = round_share<JU>(T, m);
-            const int jl = lane / ts;
-            // job lo + jl of the pool: position i of warp q's ring
-            int i = lo + min(jl, m - 1), q = 0;
+            ts = round_share<JU>(T, m);
+            // job lo + lane / ts of the pool: position i of warp q's ring
+            int i = lo + min(lane / ts, m - 1), q = 0;
+            unsigned f = lds_u32(units);
 #pragma unroll
             for (int w = 0; w < NW - 1; ++w) {
-                const int f = (int)((fl[w] >> (8 * T)) & 255u);
-                const bool past = q == w && i >= f;
-                i -= past ? f : 0;
-                q += past ? 1 : 0;
+                const int fw = (int)((f >> (8 * T)) & 255u);
+                if (q == w && i >= fw) {
+                    i -= fw;
+                    ++q;
+                    f = lds_u32(units + 4u * (unsigned)q);
+                }
             }
-            const unsigned run =
-                lds_u32(rings + RING_BYTES * (unsigned)q + 128u * (unsigned)T + 4u * (unsigned)i);
-            const unsigned fb = job_round<NT, R, JU, HM, ST>(T, run, jl < m, lane % ts, ts, sIJ,
-                                                             bxy, bz, lut, caps, band, sC, col,
-                                                             p, S, stats, stat);
-            if (T == kJobTwo) fb0 = fb;
-            if (T == kJobThree) fb1 = fb;
+            at = rings + RINGS * (unsigned)q + RING * (unsigned)T +
+                 4u * (((((f >> (24 + T)) & 1u) * 32u) + (unsigned)i) & (kRing - 1));
         }
-        __syncthreads();  // every pooled job read: the rings are free again
-        // pooled span jobs that found a value near an edge (rare): pair by pair,
-        // each warp its own, through its pair-by-pair ring
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-            const unsigned fb = h == 0 ? fb0 : fb1;
-            const unsigned m = __ballot_sync(0xffffffffu, fb != 0u);
-            if (m == 0u) continue;
-            const int n = __popc(m);
-            const unsigned rt = ring + 128u * (unsigned)kJobExact;
-            if (fb) sts_u32(rt + 4u * (unsigned)__popc(m & ((1u << lane) - 1u)), fb & 0x3FFFFFFFu);
-            __syncwarp();
-            const int ts = round_share<JU>(kJobExact, n);
-            const int jl = lane / ts;
-            const unsigned run = lds_u32(rt + 4u * (unsigned)min(jl, n - 1));
-            __syncwarp();
-            job_round<NT, R, JU, HM, ST>(kJobExact, run, jl < n, lane % ts, ts, sIJ, bxy, bz, lut,
-                                         caps, band, sC, col, p, S, stats, stat);
-        }
+        __syncwarp();
+        const unsigned run = lds_u32(at);
+        __syncwarp();
+        job_round<NT, R, JU, HM, ST>(T, run, lane / ts < m, lane % ts, ts, sIJ, bxy, bz, lut, caps,
+                                     band, sC, col, p, S, stats, stat);
     }
-    // the diagonal units taken: pair by pair, i < j
-#pragma unroll 1
-    while (diag_units) {
-        const int b = __ffs(diag_units) - 1;
-        diag_units &= diag_units - 1;
-        const int sub = b / UPS, ub = (b % UPS) * UB, a_first = sub * SA + lane * R;
+    if (diag) {
+        // every group against its own chunk, pair by pair, i < j
+        const int a_first = warp * SA + lane * R, c = a_first / kChunk;
         const long long I = lds_s64(sIJ), J = lds_s64(sIJ + 8u);
         f2_t ax[R / 2], ay[R / 2], az[R / 2];
         load_local<R>(S.al, S.al_stride, I * TA + a_first, ax, ay, az);
-        const float4 ca = __ldg(S.a_caps + (I * TA + a_first) / kChunk);
+        recentre<R>(__ldg(S.a_caps + (I * TA + a_first) / kChunk), chunk_sphere(caps, c), ax, ay,
+                    az, ax, ay, az);
         unsigned long long nr = 0;
-#pragma unroll 1
-        for (int c = ub / kChunk; c < (ub + UB) / kChunk; ++c) {
-            f2_t lx[R / 2], ly[R / 2], lz[R / 2];
-            recentre<R>(ca, chunk_sphere(caps, c), ax, ay, az, lx, ly, lz);
-            tile_pass<NT, R, JU, HM, 0, true>(bxy, bz, lut, sC, hist, lx, ly, lz, p, S, I, J,
-                                              a_first, c * kChunk, (c + 1) * kChunk, nr);
-        }
+        tile_pass<NT, R, JU, HM, 0, true>(bxy, bz, lut, sC, hist, ax, ay, az, p, S, I, J, a_first,
+                                          c * kChunk, (c + 1) * kChunk, nr);
         if (stats) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
@@ -1874,7 +1853,7 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
     static_assert(TA == NW * SA && TB % UPS == 0, "units tile the item");
     __shared__ unsigned s_units[NW];
     // span job rings (one per kind and warp) for the shapes that bin spans
-    __shared__ unsigned s_ring[(!DEF && HM != kHistWarp) ? NW * kJobKinds * 32 : 1];
+    __shared__ unsigned s_ring[(!DEF && HM != kHistWarp) ? NW * kJobKinds * kRing : 1];
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = p.tab.K;
     ulonglong2* sBxy = reinterpret_cast<ulonglong2*>(smem);
@@ -2461,16 +2440,16 @@ unsigned long long per_item_bound(const Variant* v) {
     // A thread bins (or settles by chunk) R x TB pairs per unit of its own
     // sub-tile and may take the units of every other sub-tile of the item
     // (NT/32 of them): own = NT/32 x R TB pairs of its own groups.  With span
-    // jobs it also runs at most one job (R x 32 pairs) per round of its warp;
-    // the warp's jobs are at most one per lane and chunk, plus one
-    // pair-by-pair job for each span job that found a value near an edge, so
-    // its full rounds add at most 2 own; after them come at most three pooled
-    // rounds and two rounds of pooled jobs redone pair by pair.  A per-warp
-    // column gains 32 times as much.
+    // jobs it also runs at most one job (R x 32 pairs, counted up or down in a
+    // word) per round of its warp; the warp's jobs are at most
+    // (kMaxEdges + 1) / 2 per lane and chunk, so its full rounds add at most
+    // that many times own; after them come at most three pooled rounds and
+    // the pairs of its own chunk of a diagonal tile pair.  A per-warp column
+    // gains 32 times as much, one shared by eight lanes eight times.
     const unsigned long long own = (unsigned long long)(v->nt / 32) * (unsigned long long)v->r *
                                    (unsigned long long)v->nt * (unsigned long long)v->r;
-    return (v->hm == kHistWarp || v->hm == kHistWarpRed ? 32ull : 1ull) *
-           (3ull * own + 5ull * 32ull * (unsigned)v->r);
+    return (v->hm == kHistWarp || v->hm == kHistWarpRed ? 32ull : 8ull) *
+           ((1ull + (kMaxEdges + 1) / 2) * own + 4ull * 32ull * (unsigned)v->r);
 }
 
 Segment make_segment(const Prepared& A, const Prepared& B, long long ta, long long tb,
@@ -2508,7 +2487,8 @@ PairParams make_params(const Variant* v, const BinTable& tab, const Segment* seg
     prm.n_segs = n_segs;
     prm.item_begin = item_begin;
     prm.n_items = n_items;
-    prm.items_per_flush = (int)std::min<unsigned long long>(0xFFFFFFFFull / per_item_bound(v),
+    // the words of the private columns are signed sums
+    prm.items_per_flush = (int)std::min<unsigned long long>(0x7FFFFFFFull / per_item_bound(v),
                                                             1ull << 30);
     prm.cursor = cursor;
     prm.stats = stats;
