@@ -97,10 +97,24 @@ __device__ __forceinline__ unsigned smem_addr(const void* p) {
 __device__ __forceinline__ void lds_f2x2(unsigned a, f2_t& x, f2_t& y) {
     asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "r"(a));
 }
+__device__ __forceinline__ void sts_f2x2(unsigned a, f2_t x, f2_t y) {
+    asm volatile("st.shared.v2.b64 [%0], {%1, %2};" :: "r"(a), "l"(x), "l"(y) : "memory");
+}
+__device__ __forceinline__ uint2 lds_u2(unsigned a) {
+    uint2 v;
+    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
 __device__ __forceinline__ f2_t lds_f2(unsigned a) {
     f2_t z;
     asm volatile("ld.shared.b64 %0, [%1];" : "=l"(z) : "r"(a));
     return z;
+}
+// n += sign bit of d, as one shift-and-add (written this way: as plain C++ the
+// adds of two values are combined first, into three operations instead of two)
+__device__ __forceinline__ void add_sign(unsigned& n, float d) {
+    asm("{\n\t.reg .u32 t;\n\tshr.u32 t, %1, 31;\n\tadd.u32 %0, %0, t;\n\t}"
+        : "+r"(n) : "r"(__float_as_uint(d)));
 }
 __device__ __forceinline__ uint4 lds_u4(unsigned a) {
     uint4 v;
@@ -125,6 +139,10 @@ __device__ __forceinline__ unsigned lds_u32(unsigned a) {
 }
 __device__ __forceinline__ void sts_u32(unsigned a, unsigned v) {
     asm volatile("st.shared.b32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts_u32_if(bool p, unsigned a, unsigned v) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.shared.b32 [%0], %1;\n\t}"
+                 :: "r"(a), "r"(v), "r"((unsigned)p) : "memory");
 }
 __device__ __forceinline__ void red_add_shared(unsigned a, unsigned v) {
     asm volatile("red.shared.add.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
@@ -847,6 +865,23 @@ __global__ void k_cull_prefix(Segment* __restrict__ segs, const CullSeg* __restr
     *total = acc;
 }
 
+// sqrt within 2^-22 relative
+__device__ __forceinline__ float sqrt_approx(float x) {
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// Edges at or below x (FP64 edges at shared address c64).
+__device__ __forceinline__ unsigned edges_below(double x, unsigned c64, int K) {
+    unsigned lo = 0, hi = (unsigned)K + 1;
+    while (lo < hi) {
+        const unsigned mid = (lo + hi) >> 1;
+        if (lds_f64(c64 + 8u * mid) <= x) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
 // FP64 recheck: the definition's squared chord and slot for the pair of
 // sorted positions (ia, jb), read from the FP64 copies in the spatial order,
 // or from the caller's FP64 arrays through the original indices kept in the
@@ -877,15 +912,20 @@ __device__ __forceinline__ unsigned recheck_slot(const Segment& S, long long ia,
             return (unsigned)hint + 1u;
         }
     }
-    // the number of edges at or below s, by bisection (K+1 = overflow)
-    unsigned lo = 0, hi = (unsigned)K + 1;
-    while (lo < hi) {
-        const unsigned mid = (lo + hi) >> 1;
-        if (lds_f64(c64 + 8u * mid) <= s) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
+    return edges_below(s, c64, K);  // (K + 1: overflow)
 }
+
+// The staged B tile: per point its three coordinates, negated and duplicated
+// for the packed FP32 arithmetic (24 B), so that two consecutive points are
+// three 16-byte loads; a chunk of 32 points takes 16 B more, so that lanes on
+// different chunks read different banks.
+constexpr unsigned kPointB = 24, kChunkB = 32 * kPointB + 16;
+__device__ __forceinline__ unsigned point_addr(unsigned tile, int j) {
+    return tile + (unsigned)(j >> 5) * kChunkB + (unsigned)(j & 31) * kPointB;
+}
+
+// Items are taken in parts until there are this many per block.
+constexpr int kPartWaves = 4;
 
 template <int NT, int R, int JU, int HM, int DEF>
 struct PairKernel {
@@ -901,7 +941,7 @@ struct PairKernel {
     // odd number of words apart, so that lanes adding to different rows of one
     // column hit different banks.
     static constexpr int CPW = (HM == kHistWarp || HM == kHistWarpRed) ? 1
-                               : HM == kHistLaneAtomic && !DEF         ? 4
+                               : HM == kHistLaneAtomic && DEF == 0     ? 4
                                                                        : 32;
     static constexpr int HCOLS = NW * CPW;
     static constexpr int HSTRIDE = CPW == 4 || HM == kHistWarpRed ? (HCOLS | 1) : HCOLS;
@@ -910,10 +950,14 @@ struct PairKernel {
     }
     static constexpr unsigned ROWB = 4u * HSTRIDE;
 
+    // log2 of the most parts an item is taken in: quarters of the B tile (the
+    // units of several warps), or single chunks in a one-warp block
+    static constexpr int MAXLP = NW == 1 ? ilog2(TB / 32) : 2;
+
     static size_t smem_bytes(int K, int n_lut) {
-        size_t b = (size_t)TB * 24;             // B tile: {-x,-x,-y,-y} + {-z,-z}
+        size_t b = (size_t)TB / 32 * kChunkB;   // B tile
         b += (size_t)TB / 32 * 16;              // bounding spheres of its 32-point chunks
-        b += (size_t)n_lut * 16;                // screening table
+        b += (size_t)n_lut * 8;                 // screening table
         b += (size_t)(K + 2) * 8;               // FP64 edges (+ pad)
         b += (size_t)(K + 2) * 8;               // middle and half slack of every edge
         b += (size_t)(K + 2) * ROWB;            // histograms, row K+1 a trash row
@@ -950,32 +994,50 @@ __device__ __forceinline__ void hist_add(unsigned cell, unsigned v) {
 }
 
 // Table entry of an FP32 squared chord's bucket (bits >= 0: non-negative).
-__device__ __forceinline__ uint4 lut_entry(unsigned bits, unsigned lut, int shift, int base,
+__device__ __forceinline__ uint2 lut_entry(unsigned bits, unsigned lut, int shift, int base,
                                            int top_idx) {
     const int idx = min(max((int)(bits >> shift) - base, 0), top_idx);
-    return lds_u4(lut + 16u * (unsigned)idx);
+    return lds_u2(lut + 8u * (unsigned)idx);
+}
+// The entry's parts: the slot below its edge, and whether bits lie below the
+// edge's band, or inside it (BinTable).
+__device__ __forceinline__ unsigned lut_slot(uint2 e) { return e.y & kLutSlot; }
+__device__ __forceinline__ bool lut_below(uint2 e, unsigned bits) { return bits < e.x; }
+__device__ __forceinline__ bool lut_band(uint2 e, unsigned bits) {
+    return bits - e.x <= e.y >> kLutWidthShift;  // below: the difference wraps
 }
 
 // Bins NV screened values s[h R + r] (pairs of A point r and B point j + h)
-// into the thread's private histogram column at shared address col.  The
-// table gives the byte offset of the row below / above the guard band of the
-// bucket's edge; a value beyond the top edge (or masked with +inf) lands in
-// the trash row K+1.  A value inside a band is counted, for now, in the row
-// above it; the function returns true if the step held any such value, and
-// the caller then settles them (recount_band_values).  No branch.
-template <int NV, int HM>
+// into the thread's private histogram column at shared address col (rows ROWB
+// bytes apart).  The table gives the slot below the bucket's edge; a value
+// beyond the top edge (or masked with +inf) lands in the trash row K+1.  A value
+// inside a band is counted, for now, in the row above it; the function returns
+// true if the step held any such value, and the caller then settles them
+// (recount_band_values).  No branch.
+template <int NV, int HM, unsigned ROWB>
 __device__ __forceinline__ bool bin_values(const float (&s)[NV], unsigned col, unsigned lut,
                                            int shift, int base, int top_idx) {
     bool any_band = false;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         const unsigned bits = __float_as_uint(s[v]);
-        const uint4 e = lut_entry(bits, lut, shift, base, top_idx);
-        const bool below = bits < e.x;
-        any_band |= !below && bits <= e.y;
-        hist_add<HM>(col + (below ? e.z : e.w), 1u);
+        const uint2 e = lut_entry(bits, lut, shift, base, top_idx);
+        const bool below = lut_below(e, bits);
+        any_band |= lut_band(e, bits);
+        hist_add<HM>(col + (lut_slot(e) + (below ? 0u : 1u)) * ROWB, 1u);
     }
     return any_band;
+}
+
+// Bounds of edge k's guard band, a little outside the table's: its half-width
+// (guard_half_width in the host sources) is at most u (11.4 sqrt(c) + 22.1 c)
+// plus 6e-13, u = 2^-24.
+__device__ __forceinline__ float guard_half(float c) {
+    return 5.9604645e-8f * (12.f * sqrt_approx(c) + 24.f * c) + 1e-12f;
+}
+__device__ __forceinline__ bool outside_guard(float s, unsigned c64, unsigned k) {
+    const float c = (float)lds_f64(c64 + 8u * k);
+    return fabsf(s - c) > 1.1f * guard_half(c);
 }
 
 // A step's NV squared chords, passed by value.
@@ -989,12 +1051,11 @@ struct StepValues {
 // recheck gives (one copy of the recheck code, in a loop over a bitmask);
 // returns the number of values rechecked.  Kept out of line: its FP64
 // registers then do not weigh on the loops that call it.
-template <int NT, int R, int NV, int HM>
+template <int NT, int R, int NV, int HM, unsigned ROWB>
 __device__ __noinline__ unsigned recount_band_values(const StepValues<NV> sv, unsigned col,
                                                      unsigned lut, int shift, int base,
-                                                     int top_idx, unsigned row_bytes, int K,
-                                                     const Segment& S, long long a0, long long bj,
-                                                     unsigned sC) {
+                                                     int top_idx, int K, const Segment& S,
+                                                     long long a0, long long bj, unsigned sC) {
     const float (&s)[NV] = sv.v;
     unsigned n_recheck = 0;
     unsigned mask = 0;
@@ -1002,46 +1063,63 @@ __device__ __noinline__ unsigned recount_band_values(const StepValues<NV> sv, un
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         const unsigned bits = __float_as_uint(s[v]);
-        const uint4 e = lut_entry(bits, lut, shift, base, top_idx);
-        if (bits >= e.x && bits <= e.y) {
+        const uint2 e = lut_entry(bits, lut, shift, base, top_idx);
+        if (lut_band(e, bits)) {
             mask |= 1u << v;
-            hist_add<HM>(col + e.w, 0xFFFFFFFFu);  // -1
+            hist_add<HM>(col + (lut_slot(e) + 1u) * ROWB, 0xFFFFFFFFu);  // -1
             if (hint_v < 0) {
                 hint_v = v;
-                hint = e.w == e.z + row_bytes ? (int)(e.z / row_bytes) : -1;
+                hint = (e.y & kLutSeveral) ? -1 : (int)lut_slot(e);
             }
         }
     }
     while (mask) {
         const int v = __ffs(mask) - 1;
         mask &= mask - 1;
-        const unsigned slot =
-            recheck_slot(S, a0 + v % R, bj + v / R, sC, K, v == hint_v ? hint : -1);
-        ++n_recheck;
-        hist_add<HM>(col + slot * row_bytes, 1u);
+        unsigned slot = 0;
+        bool sure = false;
+        if (v != hint_v || hint < 0) {
+            // perhaps a bucket with several edges: the edges searched in FP32
+            // first, and FP64 only within a guard band of the edges next to it
+            slot = edges_below(s[v], sC, K);
+            sure = (slot == 0u || outside_guard(s[v], sC, slot - 1u)) &&
+                   (slot > (unsigned)K || outside_guard(s[v], sC, slot));
+        }
+        if (!sure) {
+            slot = recheck_slot(S, a0 + v % R, bj + v / R, sC, K, v == hint_v ? hint : -1);
+            ++n_recheck;
+        }
+        hist_add<HM>(col + slot * ROWB, 1u);
     }
     return n_recheck;
 }
 
-// Squared chords of JU consecutive B points (from j) with the thread's R A
-// points: s[h R + r].  On a diagonal tile, pairs with i >= j get +inf, i
-// being a_first + r (the thread's first A point's position in the tile).
-// The B tile sits at shared addresses bxy (16 B per point: -x,-x,-y,-y) and
-// bz (8 B per point: -z,-z).
-template <int NT, int R, int JU, bool DIAG>
-__device__ __forceinline__ void chords(float (&s)[JU * R], unsigned bxy_base, unsigned bz_base,
-                                       const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
-                                       const f2_t (&az)[R / 2], int j, int a_first) {
+// Squared chords of JU consecutive B points (from tile position j, at shared
+// address b) with the thread's R A points: s[h R + r].  On a diagonal tile,
+// pairs with i >= j get +inf, i being a_first + r (the thread's first A point's
+// position in the tile).
+template <int R, int JU, bool DIAG>
+__device__ __forceinline__ void chords(float (&s)[JU * R], unsigned b, const f2_t (&ax)[R / 2],
+                                       const f2_t (&ay)[R / 2], const f2_t (&az)[R / 2], int j,
+                                       int a_first) {
+    static_assert(JU <= 2, "");
+    f2_t bx[JU], by[JU], bz[JU];
+    if (JU == 2) {
+        lds_f2x2(b, bx[0], by[0]);
+        lds_f2x2(b + 16u, bz[0], bx[JU - 1]);
+        lds_f2x2(b + 32u, by[JU - 1], bz[JU - 1]);
+    } else {
+        bx[0] = lds_f2(b);
+        by[0] = lds_f2(b + 8u);
+        bz[0] = lds_f2(b + 16u);
+    }
 #pragma unroll
     for (int h = 0; h < JU; ++h) {
-        f2_t bx, by;
-        lds_f2x2(bxy_base + 16u * (unsigned)(j + h), bx, by);
-        const f2_t bz = lds_f2(bz_base + 8u * (unsigned)(j + h));
 #pragma unroll
         for (int q = 0; q < R / 2; ++q) {
-            const f2_t dx = add2(ax[q], bx);
-            const f2_t dy = add2(ay[q], by);
-            const f2_t dz = add2(az[q], bz);
+            const f2_t dx = add2(ax[q], bx[h]);
+            const f2_t dy = add2(ay[q], by[h]);
+            const f2_t dz = add2(az[q], bz[h]);
             const f2_t t = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
             unpack2(t, s[h * R + 2 * q], s[h * R + 2 * q + 1]);
         }
@@ -1066,27 +1144,26 @@ __device__ __forceinline__ float min_of(const float (&s)[NV]) {
 
 // The FP32 steps [j0, j1) of a B tile for the thread's R A points, each pair
 // binned through the table (values inside a guard band settled in FP64).
-template <int NT, int R, int JU, int HM, bool DIAG>
-__device__ __forceinline__ void exact_steps(int j0, int j1, unsigned bxy, unsigned bz,
-                                            unsigned lut, unsigned sC,
-                                            unsigned col, const f2_t (&ax)[R / 2],
+template <int NT, int R, int JU, int HM, unsigned ROWB, bool DIAG>
+__device__ __forceinline__ void exact_steps(int j0, int j1, unsigned tile, unsigned lut,
+                                            unsigned sC, unsigned col, const f2_t (&ax)[R / 2],
                                             const f2_t (&ay)[R / 2], const f2_t (&az)[R / 2],
-                                            float hf, int shift, int base, int top_idx,
-                                            unsigned row_bytes, int K, const Segment& S,
-                                            long long a0, long long b0, int a_first,
-                                            unsigned long long& n_recheck) {
+                                            float hf, int shift, int base, int top_idx, int K,
+                                            const Segment& S, long long a0, long long b0,
+                                            int a_first, unsigned long long& n_recheck) {
     constexpr int NV = JU * R;
+    unsigned b = point_addr(tile, j0);
 #pragma unroll 1
-    for (int j = j0; j < j1; j += JU) {
+    for (int j = j0; j < j1; b += JU * kPointB + ((j & 31) == 32 - JU ? 16u : 0u), j += JU) {
         float s[NV];
-        chords<NT, R, JU, DIAG>(s, bxy, bz, ax, ay, az, j, a_first);
+        chords<R, JU, DIAG>(s, b, ax, ay, az, j, a_first);
         const float m = min_of(s);
         if (!(m <= hf)) continue;
-        if (bin_values<NV, HM>(s, col, lut, shift, base, top_idx)) {
+        if (bin_values<NV, HM, ROWB>(s, col, lut, shift, base, top_idx)) {
             StepValues<NV> s2;
-            chords<NT, R, JU, DIAG>(s2.v, bxy, bz, ax, ay, az, j, a_first);
-            n_recheck += recount_band_values<NT, R, NV, HM>(s2, col, lut, shift, base, top_idx,
-                                                            row_bytes, K, S, a0, b0 + j, sC);
+            chords<R, JU, DIAG>(s2.v, b, ax, ay, az, j, a_first);
+            n_recheck += recount_band_values<NT, R, NV, HM, ROWB>(s2, col, lut, shift, base,
+                                                                  top_idx, K, S, a0, b0 + j, sC);
         }
     }
 }
@@ -1124,39 +1201,48 @@ __device__ __forceinline__ float4 group_cap(const f2_t (&ax)[R / 2], const f2_t 
 // within 1.2e-7 of their FP32 copies and the FP32 arithmetic here errs by a
 // few units in the last place, all covered by the 1e-6 absolute and relative
 // slack, so every pair's FP64 squared chord lies in [slo, shi].  The table
-// gives the lowest slot rlo and the highest rhi that the interval can touch (an
-// end inside an edge's guard band takes the edge in), as byte offsets of the
-// slots' rows (slot * row_bytes).  Returns the number of edges between them:
+// gives the lowest slot rlo and the highest slot rhi that the interval can
+// touch (an end inside an edge's guard band takes the edge in; a bucket with
+// several edges has them searched, their FP32 values being far closer to the
+// FP64 ones than the slack).  Returns the number of edges between them:
 //   0        every pair is in slot rlo (a span wholly above h_top, the top
-//            edge's band, is the overflow row trash at once);
+//            edge's band, is the overflow slot K + 1 at once);
 //   1 .. kMaxEdges  the counts of the slots follow from the number of pairs
 //            below each of those edges;
-//   -1       more edges, a bucket of the table holding several edges, or
-//            padding: bin pair by pair.
-// Per edge a job costs 16 packed fmas and 8 wavefronts of shared loads per 8
-// pairs where the table costs a 16-byte lookup and a shared atomic per pair, so
-// the line lies well above one edge: 6 measured best of 2, 4, 6 and 8.
-constexpr int kMaxEdges = 6;
-__device__ __forceinline__ int span_edges(float4 ga, float4 gb, unsigned lut, int shift, int base,
-                                          int top_idx, unsigned row_bytes, unsigned& rlo,
-                                          unsigned& rhi, unsigned h_top, unsigned trash) {
+//            (up to kMaxEdgesFar beyond 60 degrees, where guard bands are
+//            widest and the table's buckets hold several edges, whose pairs
+//            would be searched one by one);
+//   -1       more edges, or padding: bin pair by pair.
+// Two edges cost a job about a quarter of the table's lookups and shared
+// atomics for its 256 pairs.  The lines, one build, kMaxEdges 4, 6, 8: 256 bins
+// (200k + 200k points) 8.70, 8.91, 9.39 ms; 24 bins (30k x 48k) 513, 509, 517
+// us; 32 bins (1M + 1M) 36.67, 36.72, 36.81 ms; 36 linear bins to 180 deg (100k +
+// 100k) 14.3, 13.6, 10.0 ms, and 10.0 with 6 and the line for far spans.
+constexpr int kMaxEdges = 6, kMaxEdgesFar = 16;
+__device__ __forceinline__ int span_edges(float4 ga, float4 gb, unsigned lut, unsigned c64,
+                                          int shift, int base, int top_idx, int K, unsigned h_top,
+                                          unsigned& rlo, unsigned& rhi) {
     const float dx = ga.x - gb.x, dy = ga.y - gb.y, dz = ga.z - gb.z;
-    const float dc = sqrtf(dx * dx + dy * dy + dz * dz);
+    const float dc = sqrt_approx(dx * dx + dy * dy + dz * dz);
     const float rr = (ga.w + gb.w) * (1.f + 1e-6f) + 1e-6f;
-    const float lo = dc * (1.f - 1e-6f) - rr, hi = dc * (1.f + 1e-6f) + rr;
-    const float slo = lo > 0.f ? lo * lo * (1.f - 1e-5f) : 0.f;
+    const float lo = fmaxf(dc * (1.f - 1e-6f) - rr, 0.f), hi = dc * (1.f + 1e-6f) + rr;
+    const float slo = lo * lo * (1.f - 1e-5f);
     const float shi = hi * hi * (1.f + 1e-5f);
-    if (!(ga.w <= 2.f && gb.w >= 0.f && gb.w <= 2.f)) return -1;  // padding (or NaN)
     const unsigned bl = __float_as_uint(slo), bh = __float_as_uint(shi);
-    rlo = rhi = trash;
-    if (bl > h_top) return 0;
-    const uint4 el = lut_entry(bl, lut, shift, base, top_idx);
-    const uint4 eh = lut_entry(bh, lut, shift, base, top_idx);
-    if (el.z == trash || eh.z == trash) return -1;  // several edges in one bucket
-    rlo = bl <= el.y ? el.z : el.w;
-    rhi = bh < eh.x ? eh.z : eh.w;
-    const int n = (int)(rhi - rlo) / (int)row_bytes;
-    return n <= kMaxEdges ? n : -1;
+    // padding (a group's radius far above 2, a chunk's -1), a wide chunk, NaN
+    const bool real = (ga.w <= 2.f) & (gb.w >= 0.f) & (gb.w <= 2.f);
+    const uint2 el = lut_entry(bl, lut, shift, base, top_idx);
+    const uint2 eh = lut_entry(bh, lut, shift, base, top_idx);
+    rlo = lut_slot(el) + ((lut_below(el, bl) | lut_band(el, bl)) ? 0u : 1u);
+    rhi = lut_slot(eh) + (lut_below(eh, bh) ? 0u : 1u);
+    if ((el.y | eh.y) & kLutSeveral) {
+        rlo = edges_below(slo, c64, K);
+        rhi = edges_below(shi, c64, K);
+    }
+    const int most = shi >= 1.f ? kMaxEdgesFar : kMaxEdges;
+    if (bl > h_top) rlo = rhi = (unsigned)K + 1u;
+    const int n = (int)(rhi - rlo);
+    return real && n <= most ? n : -1;
 }
 
 // The local form of a pair's squared chord: with the chunk's centre c, b = c +
@@ -1172,62 +1258,64 @@ __device__ __forceinline__ int span_edges(float4 ga, float4 gb, unsigned lut, in
 //
 // A one-edge step is 12 packed fmas per B point and 8 A points.
 //
-// One step: JU B points (staged negated) and the thread's R A points.  neg[q]
+// One step: two B points (staged negated, at shared address b) and the
+// thread's R A points.  neg[q]
 // counts the values with d < 0 and mb[q] keeps the smallest |d|, one
 // accumulator per A pair q so that the steps' dependency chains interleave.
-template <int R, int JU>
-__device__ __forceinline__ void one_edge_step(unsigned bxy_base, unsigned bz_base,
-                                              const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
-                                              const f2_t (&az)[R / 2], const f2_t (&a0)[R / 2],
-                                              int j, unsigned (&neg)[R / 2], float (&mb)[R / 2]) {
+template <int R>
+__device__ __forceinline__ void one_edge_step(unsigned b, const f2_t (&ax)[R / 2],
+                                              const f2_t (&ay)[R / 2], const f2_t (&az)[R / 2],
+                                              const f2_t (&a0)[R / 2], unsigned (&neg)[R / 2],
+                                              float (&mb)[R / 2]) {
+    f2_t bx[2], by[2], bz[2];
+    lds_f2x2(b, bx[0], by[0]);
+    lds_f2x2(b + 16u, bz[0], bx[1]);
+    lds_f2x2(b + 32u, by[1], bz[1]);
 #pragma unroll
-    for (int h = 0; h < JU; ++h) {
-        f2_t bx, by;
-        lds_f2x2(bxy_base + 16u * (unsigned)(j + h), bx, by);
-        const f2_t bz = lds_f2(bz_base + 8u * (unsigned)(j + h));
+    for (int h = 0; h < 2; ++h)
 #pragma unroll
         for (int q = 0; q < R / 2; ++q) {
             float d0, d1;
-            unpack2(fma2(ax[q], bx, fma2(ay[q], by, fma2(az[q], bz, a0[q]))), d0, d1);
+            unpack2(fma2(ax[q], bx[h], fma2(ay[q], by[h], fma2(az[q], bz[h], a0[q]))), d0, d1);
             mb[q] = min3f(mb[q], fabsf(d0), fabsf(d1));
-            neg[q] += (__float_as_uint(d0) >> 31) + (__float_as_uint(d1) >> 31);
+            add_sign(neg[q], d0);
+            add_sign(neg[q], d1);
         }
-    }
 }
 
 // One step against two edges, the second's
 // value from the first's by one more subtraction of half their distance
 // (ndel = -(mid2 - mid1) / 2).
-template <int R, int JU>
-__device__ __forceinline__ void two_edge_step(unsigned bxy_base, unsigned bz_base,
-                                                const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
-                                                const f2_t (&az)[R / 2], const f2_t (&a0)[R / 2],
-                                                int j, f2_t ndel, unsigned& neg1, unsigned& neg2,
-                                                float& mb1, float& mb2) {
+template <int R>
+__device__ __forceinline__ void two_edge_step(unsigned b, const f2_t (&ax)[R / 2],
+                                              const f2_t (&ay)[R / 2], const f2_t (&az)[R / 2],
+                                              const f2_t (&a0)[R / 2], f2_t ndel, unsigned& neg1,
+                                              unsigned& neg2, float& mb1, float& mb2) {
+    f2_t bx[2], by[2], bz[2];
+    lds_f2x2(b, bx[0], by[0]);
+    lds_f2x2(b + 16u, bz[0], bx[1]);
+    lds_f2x2(b + 32u, by[1], bz[1]);
 #pragma unroll
-    for (int h = 0; h < JU; ++h) {
-        f2_t bx, by;
-        lds_f2x2(bxy_base + 16u * (unsigned)(j + h), bx, by);
-        const f2_t bz = lds_f2(bz_base + 8u * (unsigned)(j + h));
+    for (int h = 0; h < 2; ++h)
 #pragma unroll
         for (int q = 0; q < R / 2; ++q) {
-            const f2_t t = fma2(ax[q], bx, fma2(ay[q], by, fma2(az[q], bz, a0[q])));
+            const f2_t t = fma2(ax[q], bx[h], fma2(ay[q], by[h], fma2(az[q], bz[h], a0[q])));
             float d0, d1, e0, e1;
             unpack2(t, d0, d1);
             unpack2(add2(t, ndel), e0, e1);
             mb1 = min3f(mb1, fabsf(d0), fabsf(d1));
             mb2 = min3f(mb2, fabsf(e0), fabsf(e1));
-            neg1 += (__float_as_uint(d0) >> 31) + (__float_as_uint(d1) >> 31);
-            neg2 += (__float_as_uint(e0) >> 31) + (__float_as_uint(e1) >> 31);
+            add_sign(neg1, d0);
+            add_sign(neg1, d1);
+            add_sign(neg2, e0);
+            add_sign(neg2, e1);
         }
-    }
 }
 
 // The pairs of the thread's R A points (tile positions a_first ..) with the
 // B points [j_begin, j_end) of the staged tile.
 template <int NT, int R, int JU, int HM, int DEF, bool DIAG>
-__device__ __forceinline__ void tile_pass(unsigned bxy, unsigned bz, unsigned lut,
-                                          unsigned sC, unsigned hist,
+__device__ __forceinline__ void tile_pass(unsigned tile, unsigned lut, unsigned sC, unsigned hist,
                                           const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
                                           const f2_t (&az)[R / 2], const PairParams& p,
                                           const Segment& S, long long I, long long J, int a_first,
@@ -1240,11 +1328,11 @@ __device__ __forceinline__ void tile_pass(unsigned bxy, unsigned bz, unsigned lu
     const unsigned h_top = p.tab.h_top;
     const float hf = __uint_as_float(h_top);
     const int shift = p.tab.shift, base = p.tab.base, K = p.tab.K, top_idx = p.tab.n_lut - 1;
-    constexpr unsigned row_bytes = PK::ROWB;
+    constexpr unsigned ROWB = PK::ROWB;
     const unsigned col = hist + 4u * (unsigned)PK::column();
     const long long a0 = I * TA + a_first, b0 = J * TB;
 
-    if (DEF) {
+    if (DEF == 1) {
         // Deferred binning: the screening loop only notes, one bit per step,
         // which of 32 consecutive steps hold an in-range value; those steps
         // are then recomputed and binned.  The screening loop stays small.
@@ -1255,7 +1343,8 @@ __device__ __forceinline__ void tile_pass(unsigned bxy, unsigned bz, unsigned lu
 #pragma unroll 1
             for (int st = 0; st < 32; ++st) {
                 float s[NV];
-                chords<NT, R, JU, DIAG>(s, bxy, bz, ax, ay, az, jb + st * JU, a_first);
+                chords<R, JU, DIAG>(s, point_addr(tile, jb + st * JU), ax, ay, az, jb + st * JU,
+                                    a_first);
                 mask |= (min_of(s) <= hf ? 1u : 0u) << st;
             }
             while (mask) {
@@ -1263,11 +1352,10 @@ __device__ __forceinline__ void tile_pass(unsigned bxy, unsigned bz, unsigned lu
                 mask &= mask - 1;
                 const int j = jb + st * JU;
                 StepValues<NV> s;
-                chords<NT, R, JU, DIAG>(s.v, bxy, bz, ax, ay, az, j, a_first);
-                if (bin_values<NV, HM>(s.v, col, lut, shift, base, top_idx))
-                    n_recheck += recount_band_values<NT, R, NV, HM>(s, col, lut, shift, base,
-                                                                    top_idx, row_bytes, K, S, a0,
-                                                                    b0 + j, sC);
+                chords<R, JU, DIAG>(s.v, point_addr(tile, j), ax, ay, az, j, a_first);
+                if (bin_values<NV, HM, ROWB>(s.v, col, lut, shift, base, top_idx))
+                    n_recheck += recount_band_values<NT, R, NV, HM, ROWB>(
+                        s, col, lut, shift, base, top_idx, K, S, a0, b0 + j, sC);
             }
         }
         return;
@@ -1275,18 +1363,18 @@ __device__ __forceinline__ void tile_pass(unsigned bxy, unsigned bz, unsigned lu
 #pragma unroll 1
         for (int j = j_begin; j < j_end; j += JU) {
             float s[NV];
-            chords<NT, R, JU, DIAG>(s, bxy, bz, ax, ay, az, j, a_first);
+            chords<R, JU, DIAG>(s, point_addr(tile, j), ax, ay, az, j, a_first);
             const float m = min_of(s);
             if (!__any_sync(0xffffffffu, m <= hf)) continue;
-            const unsigned trash = (unsigned)(K + 1) * row_bytes;
             unsigned amb_mask = 0;
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
                 const unsigned bits = __float_as_uint(s[v]);
-                const uint4 e = lut_entry(bits, lut, shift, base, top_idx);
-                const bool amb = bits >= e.x && bits <= e.y;
+                const uint2 e = lut_entry(bits, lut, shift, base, top_idx);
+                const bool amb = lut_band(e, bits);
                 amb_mask |= amb ? (1u << v) : 0u;
-                const unsigned off = amb ? trash : (bits < e.x ? e.z : e.w);
+                const unsigned off =
+                    (amb ? (unsigned)K + 1u : lut_slot(e) + (lut_below(e, bits) ? 0u : 1u)) * ROWB;
                 const unsigned peers = __match_any_sync(0xffffffffu, off);
                 if (lane == __ffs(peers) - 1) red_add_shared(col + off, (unsigned)__popc(peers));
             }
@@ -1295,15 +1383,15 @@ __device__ __forceinline__ void tile_pass(unsigned bxy, unsigned bz, unsigned lu
                 amb_mask &= amb_mask - 1;
                 const unsigned slot = recheck_slot(S, a0 + v % R, b0 + j + v / R, sC, K);
                 ++n_recheck;
-                red_add_shared(col + slot * row_bytes, 1u);
+                red_add_shared(col + slot * ROWB, 1u);
             }
         }
         return;
     }
     // pair by pair (diagonal tiles, or span binning off; spans go through
     // span_item's jobs)
-    exact_steps<NT, R, JU, HM, DIAG>(j_begin, j_end, bxy, bz, lut, sC, col, ax, ay, az, hf, shift,
-                                     base, top_idx, row_bytes, K, S, a0, b0, a_first, n_recheck);
+    exact_steps<NT, R, JU, HM, ROWB, DIAG>(j_begin, j_end, tile, lut, sC, col, ax, ay, az, hf,
+                                           shift, base, top_idx, K, S, a0, b0, a_first, n_recheck);
 }
 
 // The thread's R A points, R consecutive points of the spatial order (a
@@ -1397,51 +1485,10 @@ __device__ __forceinline__ unsigned job_word(int lane, int sub, int chunk, unsig
     return (unsigned)lane | ((unsigned)sub << 5) | ((unsigned)chunk << 8) | (slot << 16);
 }
 
-// Chunk c of the B tile starts its steps at point JU c (mod 32): lanes of a
-// round on neighbouring chunks then read points in different banks.
-template <int JU>
-__device__ __forceinline__ int chunk_point(int c0, int t, int rot) {
-    return c0 + ((t + rot) & (kChunk - 1));
-}
-
 __device__ __forceinline__ unsigned atom_add_shared(unsigned a, unsigned v) {
     unsigned old;
     asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(a), "r"(v) : "memory");
     return old;
-}
-
-// A chunk's pairs with the lane's R A points (tile positions a_first ..)
-// binned pair by pair through the table, values inside a guard band settled
-// in FP64: the chunk's points t0, t0 + ts, ... (in its rotated order).  The
-// tile pair (I, J) is read from shared memory (sIJ) only for those values.
-template <int NT, int R, int JU, int HM>
-__device__ __forceinline__ void exact_chunk(int c0, int rot, int t0, int ts, int a_first,
-                                            unsigned sIJ,
-                                            unsigned bxy, unsigned bz, unsigned lut, unsigned sC,
-                                            unsigned col, const f2_t (&ax)[R / 2],
-                                            const f2_t (&ay)[R / 2], const f2_t (&az)[R / 2],
-                                            const PairParams& p, const Segment& S,
-                                            unsigned& n_recheck) {
-    using PK = PairKernel<NT, R, JU, HM, 0>;
-    constexpr int TA = PK::TA, TB = PK::TB;
-    constexpr int NV = R;  // one B point per step: fewer live values
-    const float hf = __uint_as_float(p.tab.h_top);
-    const int shift = p.tab.shift, base = p.tab.base, top_idx = p.tab.n_lut - 1;
-#pragma unroll 1
-    for (int t = t0; t < kChunk; t += ts) {
-        const int j = chunk_point<JU>(c0, t, rot);
-        float s[NV];
-        chords<NT, R, 1, false>(s, bxy, bz, ax, ay, az, j, 0);
-        if (!(min_of(s) <= hf)) continue;
-        if (bin_values<NV, HM>(s, col, lut, shift, base, top_idx)) {
-            StepValues<NV> s2;
-            chords<NT, R, 1, false>(s2.v, bxy, bz, ax, ay, az, j, 0);
-            const long long a0 = lds_s64(sIJ) * TA + a_first;
-            const long long b0 = lds_s64(sIJ + 8u) * TB;
-            n_recheck += recount_band_values<NT, R, NV, HM>(s2, col, lut, shift, base, top_idx,
-                                                            PK::ROWB, p.tab.K, S, a0, b0 + j, sC);
-        }
-    }
 }
 
 // A job's R A points (the owner lane's group), relative to the centre ca of
@@ -1458,19 +1505,37 @@ __device__ __forceinline__ int job_points(unsigned job, unsigned sIJ, const Segm
     return a_first;
 }
 
-// A job of the pair-by-pair kind (the chunk's points t0, t0 + ts, ...).
+// A job of the pair-by-pair kind: the pairs of the lane's R A points with the
+// chunk's points t0, t0 + ts, ... binned through the table, values inside a
+// guard band settled in FP64.  One B point per step: fewer live values.
 template <int NT, int R, int JU, int HM>
-__device__ __forceinline__ void exact_job(unsigned job, int t0, int ts, unsigned sIJ,
-                                          unsigned bxy, unsigned bz, unsigned lut, unsigned caps,
-                                          unsigned sC, unsigned col, const PairParams& p,
-                                          const Segment& S, unsigned& n_recheck) {
+__device__ __forceinline__ void exact_job(unsigned job, int t0, int ts, unsigned sIJ, unsigned tile,
+                                          unsigned lut, unsigned caps, unsigned sC, unsigned col,
+                                          const PairParams& p, const Segment& S,
+                                          unsigned& n_recheck) {
+    using PK = PairKernel<NT, R, JU, HM, 0>;
     f2_t ax[R / 2], ay[R / 2], az[R / 2];
     float4 ca;
     const int a_first = job_points<NT, R, JU, HM>(job, sIJ, S, ca, ax, ay, az);
     const int c = (int)((job >> 8) & 255u);
     recentre<R>(ca, chunk_sphere(caps, c), ax, ay, az, ax, ay, az);
-    exact_chunk<NT, R, JU, HM>(c * kChunk, (JU * c) & (kChunk - 1), t0, ts, a_first, sIJ, bxy,
-                               bz, lut, sC, col, ax, ay, az, p, S, n_recheck);
+    const float hf = __uint_as_float(p.tab.h_top);
+    const int shift = p.tab.shift, base = p.tab.base, top_idx = p.tab.n_lut - 1;
+#pragma unroll 1
+    for (int t = t0; t < kChunk; t += ts) {
+        const unsigned b = tile + (unsigned)c * kChunkB + (unsigned)t * kPointB;
+        float s[R];
+        chords<R, 1, false>(s, b, ax, ay, az, 0, 0);
+        if (!(min_of(s) <= hf)) continue;
+        if (bin_values<R, HM, PK::ROWB>(s, col, lut, shift, base, top_idx)) {
+            StepValues<R> s2;
+            chords<R, 1, false>(s2.v, b, ax, ay, az, 0, 0);
+            const long long a0 = lds_s64(sIJ) * PK::TA + a_first;
+            const long long bj = lds_s64(sIJ + 8u) * PK::TB + c * kChunk + t;
+            n_recheck += recount_band_values<NT, R, R, HM, PK::ROWB>(
+                s2, col, lut, shift, base, top_idx, p.tab.K, S, a0, bj, sC);
+        }
+    }
 }
 
 // The middle of edge k (edge table at shared address band) and half its slack
@@ -1482,12 +1547,12 @@ __device__ __forceinline__ float edge_mid(unsigned band, unsigned k, float& G) {
 }
 
 // A job of kind T (one or two edges) over the chunk's steps t0, t0 + ts, ...
-// (JU points each).  neg1 and neg2 count the values below the first and second
+// (two points each).  neg1 and neg2 count the values below the first and second
 // edge (neg2 = 0 for one), mb1 and mb2 return the smallest |d| less the slack:
 // at most zero if some value may be on either side.
 template <int NT, int R, int JU, int HM>
 __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, unsigned sIJ,
-                                          unsigned bxy, unsigned bz, unsigned caps, unsigned band,
+                                          unsigned tile, unsigned caps, unsigned band,
                                           const Segment& S, unsigned& neg1, unsigned& neg2,
                                           float& mb1, float& mb2) {
     constexpr int CPT = PairKernel<NT, R, JU, HM, 0>::TB / kChunk;
@@ -1496,10 +1561,9 @@ __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, u
     f2_t ax[R / 2], ay[R / 2], az[R / 2], a0[R / 2];
     float4 ca;
     job_points<NT, R, JU, HM>(job, sIJ, S, ca, ax, ay, az);
-    const int c0 = c * kChunk, rot = (JU * c) & (kChunk - 1);
-    const unsigned slot = (job >> 16) & 0x3FFFu;
+    const unsigned edge = (job >> 16) & 0x3FFFu;
     float G, G2 = 0.f;
-    const float mid = edge_mid(band, slot, G);
+    const float mid = edge_mid(band, edge, G);
     {
         f2_t lx[R / 2], ly[R / 2], lz[R / 2];
         recentre<R>(ca, chunk_sphere(caps, c), ax, ay, az, lx, ly, lz);
@@ -1510,6 +1574,9 @@ __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, u
         for (int q = 0; q < R / 2; ++q)
             a0[q] = mul2(half, fma2(lx[q], lx[q], fma2(ly[q], ly[q], fma2(lz[q], lz[q], km2))));
     }
+    unsigned b = tile + (unsigned)c * kChunkB;
+    const unsigned end = b + kChunk * kPointB, step = (unsigned)ts * (2 * kPointB);
+    b += (unsigned)t0 * (2 * kPointB);
     neg1 = neg2 = 0;
     mb1 = mb2 = __int_as_float(0x7f800000);
     if (T == kJobOne) {
@@ -1521,20 +1588,18 @@ __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, u
             mbq[q] = __int_as_float(0x7f800000);
         }
 #pragma unroll 1
-        for (int t = t0; t < kChunk; t += ts)
-            one_edge_step<R, JU>(bxy, bz, ax, ay, az, a0, chunk_point<JU>(c0, t, rot), negq, mbq);
+        for (; b < end; b += step) one_edge_step<R>(b, ax, ay, az, a0, negq, mbq);
 #pragma unroll
         for (int q = 0; q < R / 2; ++q) {
             neg1 += negq[q];
             mb1 = fminf(mb1, mbq[q]);
         }
     } else {
-        const float mid2 = edge_mid(band, slot + 1u, G2);
+        const float mid2 = edge_mid(band, edge + 1u, G2);
         const float ndel = 0.5f * (mid - mid2);
 #pragma unroll 1
-        for (int t = t0; t < kChunk; t += ts)
-            two_edge_step<R, JU>(bxy, bz, ax, ay, az, a0, chunk_point<JU>(c0, t, rot),
-                                   pack2(ndel, ndel), neg1, neg2, mb1, mb2);
+        for (; b < end; b += step)
+            two_edge_step<R>(b, ax, ay, az, a0, pack2(ndel, ndel), neg1, neg2, mb1, mb2);
         mb2 -= G2 + kap.y;
     }
     mb1 -= G + kap.y;
@@ -1589,13 +1654,13 @@ __device__ __forceinline__ void warp_stat(unsigned a, bool flag, unsigned w) {
 }
 
 // One round of jobs of kind T: this lane's share of job `run` (active: the
-// lane has one; steps t0, t0 + ts, ... of the job, its ts lanes adjacent and
-// ts a power of two).  The first lane of each job moves the counts, summed
+// lane has one; ts = 2^lts adjacent lanes share a job, this one taking steps
+// t0, t0 + ts, ...).  The first lane of each job moves the counts, summed
 // over the ts lanes, below the job's edges.
 template <int NT, int R, int JU, int HM, bool ST>
 __device__ __forceinline__ void job_round(int T, unsigned run, bool active, int t0, int ts,
-                                          unsigned sIJ, unsigned bxy, unsigned bz, unsigned lut,
-                                          unsigned caps, unsigned band, unsigned sC, unsigned col,
+                                          unsigned sIJ, unsigned tile, unsigned lut, unsigned caps,
+                                          unsigned band, unsigned sC, unsigned col,
                                           const PairParams& p, const Segment& S, bool stats,
                                           unsigned stat) {
     constexpr unsigned row_bytes = PairKernel<NT, R, JU, HM, 0>::ROWB;
@@ -1603,13 +1668,13 @@ __device__ __forceinline__ void job_round(int T, unsigned run, bool active, int 
     unsigned n_recheck = 0;
     if (T == kJobExact) {
         if (active)
-            exact_job<NT, R, JU, HM>(run, t0, ts, sIJ, bxy, bz, lut, caps, sC, col, p, S, n_recheck);
+            exact_job<NT, R, JU, HM>(run, t0, ts, sIJ, tile, lut, caps, sC, col, p, S, n_recheck);
     } else {
         unsigned neg1 = 0, neg2 = 0;
         float mb1 = __int_as_float(0x7f800000), mb2 = mb1;
         if (active)
-            span_part<NT, R, JU, HM>(T, run, t0 * JU, ts * JU, sIJ, bxy, bz, caps, band, S, neg1,
-                                     neg2, mb1, mb2);
+            span_part<NT, R, JU, HM>(T, run, t0, ts, sIJ, tile, caps, band, S, neg1, neg2, mb1,
+                                     mb2);
 #pragma unroll 1
         for (int o = ts >> 1; o > 0; o >>= 1) {
             neg1 += __shfl_xor_sync(0xffffffffu, neg1, o);
@@ -1653,13 +1718,11 @@ __device__ __forceinline__ void job_round(int T, unsigned run, bool active, int 
     }
 }
 
-// Lanes per job for a round of m < 32 jobs: the largest power of two with
-// m ts <= 32 (span jobs: at most the chunk's steps, kChunk / JU).
-template <int JU>
+// log2 of the lanes per job for a round of m < 32 jobs: the largest power of
+// two with m ts <= 32 (edge jobs: at most the chunk's 16 steps).
 __device__ __forceinline__ int round_share(int T, int m) {
-    int ts = 1 << (31 - __clz(32 / m));
-    if (T != kJobExact) ts = min(ts, kChunk / JU);
-    return ts;
+    const int l = __clz(m - 1) - 27;  // m in (2^(4-l), 2^(5-l)]
+    return m == 1 ? (T == kJobExact ? 5 : 4) : l;
 }
 
 // A warp's share of one item with span binning: units of its own sub-tile
@@ -1681,10 +1744,10 @@ __device__ __forceinline__ int round_share(int T, int m) {
 // calls this once per item (it holds block barriers).
 template <int NT, int R, int JU, int HM, bool ST>
 __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsigned sIJ,
-                                          unsigned bxy, unsigned bz, unsigned lut, unsigned caps,
+                                          unsigned tile, unsigned lut, unsigned caps,
                                           unsigned band, unsigned sC, unsigned hist,
                                           const PairParams& p, const Segment& S, bool diag,
-                                          unsigned stat) {
+                                          int part, int lp, unsigned stat) {
     using PK = PairKernel<NT, R, JU, HM, 0>;
     constexpr int TA = PK::TA, TB = PK::TB;
     constexpr int NW = NT / 32, SA = 32 * R, UPS = 4, UB = TB / UPS, CPU = UB / kChunk;
@@ -1697,42 +1760,50 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned ring = rings + RINGS * (unsigned)warp;
     const unsigned col = hist + 4u * (unsigned)PK::column();
-    const unsigned trash = (unsigned)(p.tab.K + 1) * row_bytes;
     const bool stats = ST && p.stats != nullptr;
+    // the part's chunks
+    const int c_begin = (part * (TB / kChunk)) >> lp, c_end = ((part + 1) * (TB / kChunk)) >> lp;
     unsigned fills = 0;   // jobs waiting per kind, 8 bits each; bit 24 + T: ring T starts at 32
     unsigned word = 0;    // this lane's next job (of the chunk it has classified)
-    int ones = 0, twos = 0, exact = 0;     // and how many of each kind it has to push
-    int k = 0, cap_sub = -1, cn = -1;      // cn: next chunk of the current unit, -1: none
+    int left = 0;         // the edges it still has to push jobs for; kExact: pair by pair
+    constexpr int kExact = 256;
+    int k = 0, sub = 0, own = -1, cn = 0, ce = 0;  // chunks [cn, ce) of the current unit left
+    int cap_sub = -1;
     int pool = -1;                         // kind of the pooled leftovers being run
     float4 ga = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
     for (;;) {
-        int T, m = 32;
+        int T, m = 32, lts = 0;
         unsigned at = 0;  // shared address of this lane's job
-        int ts = 1;
         if (pool < 0 && (fills & FULL) == 0u) {
-            if (!__any_sync(0xffffffffu, (ones | twos | exact) != 0)) {
+            if (!__any_sync(0xffffffffu, left != 0)) {
                 // the next chunk
 #pragma unroll 1
-                while (k < NW && cn < 0) {
-                    const int sub = (warp + k) % NW;
+                while (k < NW && cn >= ce) {
+                    sub = (warp + k) & (NW - 1);
                     unsigned u = 0;
                     if (lane == 0) u = atom_add_shared(units + 4u * (unsigned)sub, 1u);
                     u = __shfl_sync(0xffffffffu, u, 0);
-                    if (u >= (unsigned)UPS) {
+                    // (a one-warp block takes its part of the tile as one unit)
+                    cn = NW == 1 ? c_begin : (int)u * CPU;
+                    ce = NW == 1 ? c_end : cn + CPU;
+                    if (NW == 1 ? u != 0u : cn >= c_end) {
                         ++k;
+                        cn = ce;
                         continue;
                     }
-                    const int ub = (int)u * UB;
-                    if (diag && ub + UB <= sub * SA) continue;  // every pair has i >= j
+                    if (diag && ce * kChunk <= sub * SA) {  // every pair has i >= j
+                        cn = ce;
+                        continue;
+                    }
                     if (sub != cap_sub) {
                         f2_t ax[R / 2], ay[R / 2], az[R / 2];
                         const long long pos = lds_s64(sIJ) * TA + sub * SA + lane * R;
                         load_local<R>(S.al, S.al_stride, pos, ax, ay, az);
                         ga = group_cap<R>(ax, ay, az, __ldg(S.a_caps + pos / kChunk));
+                        own = diag ? (sub * SA + lane * R) / kChunk : -1;
                         cap_sub = sub;
                     }
-                    cn = ub / kChunk;
                 }
                 if (k == NW) {
                     pool = 0;  // every unit taken: the leftovers
@@ -1741,43 +1812,35 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
                     __syncthreads();
                     continue;
                 }
-                const int c = cn, sub = (warp + k) % NW;
-                cn = (c + 1) % CPU == 0 ? -1 : c + 1;
+                const int c = cn++;
                 unsigned rlo = 0, rhi = 0;
-                const int n = span_edges(ga, chunk_sphere(caps, c), lut, p.tab.shift, p.tab.base,
-                                         p.tab.n_lut - 1, row_bytes, rlo, rhi, p.tab.h_top, trash);
-                const int own = diag ? (sub * SA + lane * R) / kChunk : -1;
+                const int n = span_edges(ga, chunk_sphere(caps, c), lut, sC, p.tab.shift,
+                                         p.tab.base, p.tab.n_lut - 1, p.tab.K, p.tab.h_top, rlo,
+                                         rhi);
                 const bool mine = c > own;
-                if (mine) {
-                    if (n >= 0 && rhi != trash) hist_add<HM>(col + rhi, NP);
-                    exact = n < 0 ? 1 : 0;
-                    ones = n > 0 ? n & 1 : 0;
-                    twos = n > 0 ? n >> 1 : 0;
-                    word = job_word(lane, sub, c, rlo / row_bytes);
-                }
+                // (to the trash row if nothing is settled: no branch)
+                hist_add<HM>(col + (mine && n >= 0 ? rhi : (unsigned)p.tab.K + 1u) * row_bytes, NP);
+                left = !mine ? 0 : n < 0 ? kExact : n;
+                word = job_word(lane, sub, c, rlo);
                 if (stats) {
                     warp_stat(stat + 8u, mine && n >= 0, NP);
                     warp_stat(stat + 16u, mine ? n == 0 : c < own, NP);
                 }
             }
-            // push one job of every lane that has some left
-            const unsigned m1 = __ballot_sync(0xffffffffu, ones != 0);
-            const unsigned m2 = __ballot_sync(0xffffffffu, ones == 0 && twos != 0);
-            const unsigned m3 = __ballot_sync(0xffffffffu, exact != 0);
-            if (m1 | m2 | m3) {
-                const int Tp = ones ? kJobOne : twos ? kJobTwo : kJobExact;
-                const unsigned mk = Tp == kJobOne ? m1 : Tp == kJobTwo ? m2 : m3;
-                const unsigned pos = ((fills >> (8 * Tp)) & 255u) + ((fills >> (24 + Tp)) & 1u) * 32u +
-                                     (unsigned)__popc(mk & ((1u << lane) - 1u));
-                if (ones | twos | exact)
-                    sts_u32(ring + RING * (unsigned)Tp + 4u * (pos & (kRing - 1)), word);
-                word += Tp == kJobOne ? 1u << 16 : 2u << 16;
-                if (Tp == kJobOne) ones = 0;
-                else if (Tp == kJobTwo) --twos;
-                else exact = 0;
-                fills += (unsigned)__popc(m1) + ((unsigned)__popc(m2) << 8) +
-                         ((unsigned)__popc(m3) << 16);
-            }
+            // push one job of every lane that has some left: the odd edge alone,
+            // then the others by twos
+            const bool one = (left & 1) != 0;
+            const unsigned m1 = __ballot_sync(0xffffffffu, one);
+            const unsigned m3 = __ballot_sync(0xffffffffu, left == kExact);
+            const unsigned m2 = __ballot_sync(0xffffffffu, left != 0) & ~(m1 | m3);
+            const int Tp = one ? kJobOne : left == kExact ? kJobExact : kJobTwo;
+            const unsigned mk = one ? m1 : left == kExact ? m3 : m2;
+            const unsigned pos = (fills >> (8 * Tp)) + ((fills >> (24 + Tp)) << 5) +
+                                 (unsigned)__popc(mk & ((1u << lane) - 1u));
+            sts_u32_if(left != 0, ring + RING * (unsigned)Tp + ((4u * pos) & (RING - 4u)), word);
+            word += one ? 1u << 16 : 2u << 16;
+            left = left == kExact || left == 0 ? 0 : left - (one ? 1 : 2);
+            fills += (unsigned)__popc(m1) + ((unsigned)__popc(m2) << 8) + ((unsigned)__popc(m3) << 16);
             if ((fills & FULL) == 0u) continue;
         }
         if (pool < 0) {
@@ -1800,9 +1863,9 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
             const int lo = warp * n / NW;
             m = (warp + 1) * n / NW - lo;
             if (m == 0) continue;
-            ts = round_share<JU>(T, m);
+            lts = round_share(T, m);
             // job lo + lane / ts of the pool: position i of warp q's ring
-            int i = lo + min(lane / ts, m - 1), q = 0;
+            int i = lo + min(lane >> lts, m - 1), q = 0;
             unsigned f = lds_u32(units);
 #pragma unroll
             for (int w = 0; w < NW - 1; ++w) {
@@ -1819,11 +1882,12 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
         __syncwarp();
         const unsigned run = lds_u32(at);
         __syncwarp();
-        job_round<NT, R, JU, HM, ST>(T, run, lane / ts < m, lane % ts, ts, sIJ, bxy, bz, lut, caps,
-                                     band, sC, col, p, S, stats, stat);
+        job_round<NT, R, JU, HM, ST>(T, run, (lane >> lts) < m, lane & ((1 << lts) - 1), 1 << lts,
+                                     sIJ, tile, lut, caps, band, sC, col, p, S, stats, stat);
     }
     if (diag) {
-        // every group against its own chunk, pair by pair, i < j
+        // every group against its own chunk (if it is in this part), pair by
+        // pair, i < j
         const int a_first = warp * SA + lane * R, c = a_first / kChunk;
         const long long I = lds_s64(sIJ), J = lds_s64(sIJ + 8u);
         f2_t ax[R / 2], ay[R / 2], az[R / 2];
@@ -1831,7 +1895,7 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
         recentre<R>(__ldg(S.a_caps + (I * TA + a_first) / kChunk), chunk_sphere(caps, c), ax, ay,
                     az, ax, ay, az);
         unsigned long long nr = 0;
-        tile_pass<NT, R, JU, HM, 0, true>(bxy, bz, lut, sC, hist, ax, ay, az, p, S, I, J, a_first,
+        if (c >= c_begin && c < c_end) tile_pass<NT, R, JU, HM, 0, true>(tile, lut, sC, hist, ax, ay, az, p, S, I, J, a_first,
                                           c * kChunk, (c + 1) * kChunk, nr);
         if (stats) {
 #pragma unroll
@@ -1853,13 +1917,11 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
     static_assert(TA == NW * SA && TB % UPS == 0, "units tile the item");
     __shared__ unsigned s_units[NW];
     // span job rings (one per kind and warp) for the shapes that bin spans
-    __shared__ unsigned s_ring[(!DEF && HM != kHistWarp) ? NW * kJobKinds * kRing : 1];
+    __shared__ unsigned s_ring[(DEF == 0 && HM != kHistWarp) ? NW * kJobKinds * kRing : 1];
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = p.tab.K;
-    ulonglong2* sBxy = reinterpret_cast<ulonglong2*>(smem);
-    f2_t* sBz = reinterpret_cast<f2_t*>(sBxy + TB);
-    float4* sCap = reinterpret_cast<float4*>(sBz + TB);
-    uint4* sLut = reinterpret_cast<uint4*>(sCap + TB / 32);
+    float4* sCap = reinterpret_cast<float4*>(smem + TB / 32 * kChunkB);
+    uint2* sLut = reinterpret_cast<uint2*>(sCap + TB / 32);
     double* sC = reinterpret_cast<double*>(sLut + p.tab.n_lut);
     float2* sBand = reinterpret_cast<float2*>(sC + (K + 2));
     unsigned* hist = reinterpret_cast<unsigned*>(sBand + (K + 2));
@@ -1867,13 +1929,12 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
     // block's item count: thread 0 writes the next item's pair while other
     // warps may still read the current one
     __shared__ long long s_item, s_IJ[2][2];
+    __shared__ int s_part[2];
     __shared__ unsigned long long s_stat[3];  // span-path rechecks, span pairs, skipped pairs
 
     const int tid = threadIdx.x;
-    constexpr unsigned row_bytes = PK::ROWB;
     for (int q = tid; q < p.tab.n_lut; q += NT)
-        sLut[q] = make_uint4(p.tab.lut[q][0], p.tab.lut[q][1], p.tab.lut[q][2] * row_bytes,
-                             p.tab.lut[q][3] * row_bytes);
+        sLut[q] = make_uint2(p.tab.lut[q][0], p.tab.lut[q][1]);
     for (int q = tid; q <= K; q += NT) {
         sC[q] = p.tab.c64[q];
         sBand[q] = make_float2(p.tab.edge[q][0], p.tab.edge[q][1]);
@@ -1887,16 +1948,23 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
     __shared__ int s_seg;
     // items of this launch: p.n_items, or fewer when a device-side pass kept
     // only some of them (tile pairs wholly beyond the top edge are skipped)
-    const long long n_launch =
+    // Few items are taken in 2^lp parts of the B tile each: without that a small
+    // count is as long as one tile pair takes one block, on a chip mostly idle.
+    const long long n_tile_pairs =
         p.n_items_dev ? min(p.n_items, (long long)*p.n_items_dev) : p.n_items;
-    unsigned long long n_recheck = 0, n_items = 0;
+    int lp = 0;
+    while (lp < PK::MAXLP && (n_tile_pairs << lp) < (long long)kPartWaves * gridDim.x) ++lp;
+    const long long n_launch = n_tile_pairs << lp, n_end = p.n_items << lp;
+    unsigned long long n_recheck = 0;
+    unsigned n_items = 0, n_tiles = 0;
     int since_flush = 0, cur_seg = -2;
     for (;;) {
         if (tid == 0) {
-            const long long t = (long long)atomicAdd(p.cursor, 1ull);
-            s_item = t < n_launch ? t : p.n_items;
+            const long long tp = (long long)atomicAdd(p.cursor, 1ull), t = tp >> lp;
+            s_item = tp < n_launch ? tp : n_end;
+            s_part[n_items & 1] = (int)(tp & ((1 << lp) - 1));
             int seg = -1;
-            if (t < n_launch && p.n_segs > 0) {
+            if (tp < n_launch && p.n_segs > 0) {
                 const long long g = p.item_begin + t;
                 int lo = 0, hi = p.n_segs - 1;  // last segment with item_begin <= g
                 while (lo < hi) {
@@ -1906,7 +1974,7 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
                 seg = lo;
             }
             s_seg = seg;
-            if (t < n_launch) {
+            if (tp < n_launch) {
                 // tile pair of the item (one thread: FP64 and 64-bit divisions)
                 const Segment* G = seg < 0 ? &p.seg0 : p.segs + seg;
                 long long local = p.item_begin + t - G->item_begin + G->item_offset;
@@ -1918,8 +1986,7 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
             }
         }
         __syncthreads();  // s_item visible; previous item's shared reads finished
-        const long long t = s_item;
-        if (t >= p.n_items) break;
+        if (s_item >= n_end) break;
         const int seg = s_seg;
         if (seg != cur_seg) {
             if (cur_seg != -2 && since_flush > 0) {
@@ -1933,34 +2000,43 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
         }
         const Segment& S = sSeg;
         const long long I = s_IJ[n_items & 1][0], J = s_IJ[n_items & 1][1];
+        // the part of the B tile that this item takes
+        const int part = s_part[n_items & 1], b_len = TB >> lp, b_begin = part * b_len;
+        n_tiles += part == 0 ? 1 : 0;
         // with span binning the tile holds local coordinates (relative to each
         // chunk's centre), otherwise the FP32 copies
         bool spans = false;
-        if constexpr (!DEF && HM != kHistWarp) spans = p.span && S.b_caps;
+        if constexpr (DEF == 0 && HM != kHistWarp) spans = p.span && S.b_caps;
+        const unsigned a_tile = smem_addr(smem);
+        // two points at a time: three 16-byte stores
+        auto stage2 = [&](int j, float x0, float y0, float z0, float x1, float y1, float z1) {
+            const unsigned b = point_addr(a_tile, j);
+            sts_f2x2(b, pack2(-x0, -x0), pack2(-y0, -y0));
+            sts_f2x2(b + 16u, pack2(-z0, -z0), pack2(-x1, -x1));
+            sts_f2x2(b + 32u, pack2(-y1, -y1), pack2(-z1, -z1));
+        };
         if (spans) {
             const float* gL = S.bl + J * TB;
             const long long ls = S.bl_stride;
 #pragma unroll 4
-            for (int q = 0; q < R; ++q) {
-                const int i = q * NT + tid;
-                const float x = -gL[i], y = -gL[ls + i], z = -gL[2 * ls + i];
-                sBxy[i] = make_ulonglong2(pack2(x, x), pack2(y, y));
-                sBz[i] = pack2(z, z);
+            for (int j = b_begin + 2 * tid; j < b_begin + b_len; j += 2 * NT) {
+                const float2 x = *reinterpret_cast<const float2*>(gL + j);
+                const float2 y = *reinterpret_cast<const float2*>(gL + ls + j);
+                const float2 z = *reinterpret_cast<const float2*>(gL + 2 * ls + j);
+                stage2(j, x.x, y.x, z.x, x.y, y.y, z.y);
             }
             for (int q = tid; q < TB / 32; q += NT) sCap[q] = S.b_caps[J * (TB / 32) + q];
         } else {
             const float4* gB = S.b32 + J * TB;
 #pragma unroll 4
-            for (int q = 0; q < R; ++q) {
-                const float4 b = gB[q * NT + tid];
-                sBxy[q * NT + tid] = make_ulonglong2(pack2(-b.x, -b.x), pack2(-b.y, -b.y));
-                sBz[q * NT + tid] = pack2(-b.z, -b.z);
+            for (int j = b_begin + 2 * tid; j < b_begin + b_len; j += 2 * NT) {
+                const float4 a = gB[j], b = gB[j + 1];
+                stage2(j, a.x, a.y, a.z, b.x, b.y, b.z);
             }
         }
-        if (tid < NW) s_units[tid] = 0;
+        if (tid < NW) s_units[tid] = NW == 1 ? 0 : part * UPS >> lp;
         __syncthreads();  // B tile staged, unit counters reset
-        const unsigned a_bxy = smem_addr(sBxy), a_bz = smem_addr(sBz), a_lut = smem_addr(sLut),
-                       a_cap = smem_addr(sCap), a_band = smem_addr(sBand),
+        const unsigned a_lut = smem_addr(sLut), a_cap = smem_addr(sCap), a_band = smem_addr(sBand),
                        a_hist = smem_addr(hist), a_c = smem_addr(sC);
         // The item is split into units of one warp's worth of A points (SA =
         // 32 R consecutive points, a sub-tile) by a quarter of the B tile.  A
@@ -1969,11 +2045,11 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
         // whatever the mix of cheap and costly units.
         const int lane = tid & 31, warp = tid >> 5;
         const bool diag = S.is_auto && I == J;
-        if constexpr (!DEF && HM != kHistWarp) {
+        if constexpr (DEF == 0 && HM != kHistWarp) {
             if (spans)
                 span_item<NT, R, JU, HM, ST>(smem_addr(s_units), smem_addr(s_ring),
-                                         smem_addr(s_IJ[n_items & 1]), a_bxy, a_bz, a_lut, a_cap, a_band, a_c,
-                                         a_hist, p, S, diag, smem_addr(s_stat));
+                                         smem_addr(s_IJ[n_items & 1]), a_tile, a_lut, a_cap, a_band, a_c,
+                                         a_hist, p, S, diag, part, lp, smem_addr(s_stat));
         }
         int cur = -1;
         f2_t ax[R / 2], ay[R / 2], az[R / 2];
@@ -1985,20 +2061,22 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
                 unsigned u = 0;
                 if (lane == 0) u = atomicAdd(&s_units[sub], 1u);
                 u = __shfl_sync(0xffffffffu, u, 0);
-                if (u >= (unsigned)UPS) break;
+                // (one-warp blocks: the part of the tile as one unit)
+                const int jb = NW == 1 ? b_begin : (int)u * UB;
+                const int je = NW == 1 ? b_begin + b_len : jb + UB;
+                if (NW == 1 ? u != 0u : jb >= b_begin + b_len) break;
                 const int a_first = sub * SA + lane * R;
-                const int jb = (int)u * UB, je = jb + UB;
                 if (diag && je <= sub * SA) continue;  // every pair has i >= j
                 if (sub != cur) {
                     load_group<R>(S.a32 + I * TA + a_first, ax, ay, az);
                     cur = sub;
                 }
                 if (diag && jb < (sub + 1) * SA)
-                    tile_pass<NT, R, JU, HM, DEF, true>(a_bxy, a_bz, a_lut, a_c, a_hist, ax, ay,
+                    tile_pass<NT, R, JU, HM, DEF, true>(a_tile, a_lut, a_c, a_hist, ax, ay,
                                                         az, p, S, I, J, a_first, jb, je,
                                                         n_recheck);
                 else
-                    tile_pass<NT, R, JU, HM, DEF, false>(a_bxy, a_bz, a_lut, a_c, a_hist, ax, ay,
+                    tile_pass<NT, R, JU, HM, DEF, false>(a_tile, a_lut, a_c, a_hist, ax, ay,
                                                          az, p, S, I, J, a_first, jb, je,
                                                          n_recheck);
             }
@@ -2026,8 +2104,8 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
             if (s_stat[2]) atomicAdd(p.stats + WTHETA_STAT_PAIRS, 0ull - s_stat[2]);
         }
         if (tid == 0 && n_items) {
-            atomicAdd(p.stats + WTHETA_STAT_TILES, n_items);
-            atomicAdd(p.stats + WTHETA_STAT_PAIRS, n_items * (unsigned long long)TA * TB);
+            if (n_tiles) atomicAdd(p.stats + WTHETA_STAT_TILES, (unsigned long long)n_tiles);
+            atomicAdd(p.stats + WTHETA_STAT_PAIRS, n_items * (unsigned long long)(TA * TB >> lp));
         }
     }
 }
@@ -2068,8 +2146,8 @@ __global__ void k_finalize_segments(const Segment* __restrict__ segs, int n_segs
 // ---------------------------------------------------------------------------
 template <int NT, int R, int JU, int HM, int DEF>
 static Variant make_variant() {
-    constexpr bool spans = !DEF && HM != kHistWarp;  // only the span path has ST code
-    return Variant{NT, R, JU, HM, DEF, &k_pairs<NT, R, JU, HM, DEF, true>,
+    constexpr bool spans = DEF == 0 && HM != kHistWarp;  // only the span path has ST code
+    return Variant{NT, R, JU, HM, DEF, PairKernel<NT, R, JU, HM, DEF>::MAXLP, &k_pairs<NT, R, JU, HM, DEF, true>,
                    spans ? &k_pairs<NT, R, JU, HM, DEF, false> : &k_pairs<NT, R, JU, HM, DEF, true>,
                    &PairKernel<NT, R, JU, HM, DEF>::smem_bytes};
 }
@@ -2090,6 +2168,7 @@ const Variant* variants(int* n) {
         make_variant<256, 8, 2, kHistLaneAtomic, 1>(), make_variant<256, 8, 2, kHistWarp, 0>(),
         make_variant<64, 8, 2, kHistLaneAtomic, 0>(),  make_variant<128, 8, 2, kHistWarpRed, 0>(),
         make_variant<64, 8, 2, kHistWarpRed, 0>(),     make_variant<32, 8, 2, kHistLaneAtomic, 0>(),
+        make_variant<128, 8, 2, kHistLaneAtomic, 2>(),
     };
     *n = (int)(sizeof(v) / sizeof(v[0]));
     return v;
@@ -2146,18 +2225,30 @@ const Variant* pick_variant(const wtheta_tune* tune, int K, int n_lut, int max_s
     auto shape = [&](const Variant& x) {
         return x.nt == want_nt && x.r == want_r && x.ju == want_ju;
     };
+    auto find = [&](int hm, int def) -> const Variant* {
+        for (int i = 0; i < nv; ++i)
+            if (shape(v[i]) && v[i].hm == hm && v[i].def == def && fits(v[i])) return &v[i];
+        return nullptr;
+    };
+    // every pair through the table (span binning off): the build whose threads
+    // have a column each, without span code
+    if (want_hm == 0 && want_def < 0 && tune && tune->span_bins == 2) {
+        const Variant* x = find(kHistLaneAtomic, 2);
+        if (x && x->smem(K, n_lut) <= 100 * 1024) return x;
+    }
     if (want_hm == 0) {
-        // private per-thread histograms while they fit comfortably (measured
-        // 15% faster on the survey workload than per-warp columns, whose shared
-        // reductions contend); per-warp columns updated by shared reductions
-        // otherwise, which keep the span path at large bin counts
-        want_hm = kHistWarp;
+        want_hm = find(kHistWarpRed, 0) ? kHistWarpRed : kHistWarp;
         for (int i = 0; i < nv; ++i)
-            if (shape(v[i]) && v[i].hm == kHistWarpRed && v[i].def == 0 && fits(v[i]))
-                want_hm = kHistWarpRed;
-        for (int i = 0; i < nv; ++i)
-            if (shape(v[i]) && v[i].hm == kHistLaneAtomic && v[i].smem(K, n_lut) <= 100 * 1024)
+            if (shape(v[i]) && v[i].hm == kHistLaneAtomic && v[i].def != 2 &&
+                v[i].smem(K, n_lut) <= 100 * 1024)
                 want_hm = kHistLaneAtomic;
+        // four columns per warp while five blocks of 128 threads fit an SM; one
+        // column per warp beyond (200k + 200k points, 256 bins: 9.2 ms against
+        // 9.9 ms)
+        const Variant* four = find(kHistLaneAtomic, 0);
+        if (want_def != 1 && four && find(kHistWarpRed, 0) &&
+            four->smem(K, n_lut) > (size_t)44 * 1024 * (size_t)want_nt / 128)
+            want_hm = kHistWarpRed;
     }
     if (want_def < 0) want_def = 0;  // inline binning measured faster once in-range pairs matter
     for (int i = 0; i < nv; ++i)
@@ -2194,7 +2285,8 @@ int grid_for(const Variant* v, size_t smem, long long n_items, int sm_count, int
     per_sm = std::max(per_sm, 1);
     if (want_per_sm > 0) per_sm = std::min(per_sm, want_per_sm);
     long long g = (long long)per_sm * sm_count;
-    if (g > n_items) g = n_items;
+    // (a small count's items are taken in up to 2^max_parts parts)
+    g = std::min(g, n_items << v->max_parts);
     *grid = (int)std::max(g, 1LL);
     return WTHETA_OK;
 }
@@ -2442,14 +2534,14 @@ unsigned long long per_item_bound(const Variant* v) {
     // (NT/32 of them): own = NT/32 x R TB pairs of its own groups.  With span
     // jobs it also runs at most one job (R x 32 pairs, counted up or down in a
     // word) per round of its warp; the warp's jobs are at most
-    // (kMaxEdges + 1) / 2 per lane and chunk, so its full rounds add at most
+    // (kMaxEdgesFar + 1) / 2 per lane and chunk, so its full rounds add at most
     // that many times own; after them come at most three pooled rounds and
     // the pairs of its own chunk of a diagonal tile pair.  A per-warp column
     // gains 32 times as much, one shared by eight lanes eight times.
     const unsigned long long own = (unsigned long long)(v->nt / 32) * (unsigned long long)v->r *
                                    (unsigned long long)v->nt * (unsigned long long)v->r;
     return (v->hm == kHistWarp || v->hm == kHistWarpRed ? 32ull : 8ull) *
-           ((1ull + (kMaxEdges + 1) / 2) * own + 4ull * 32ull * (unsigned)v->r);
+           ((1ull + (kMaxEdgesFar + 1) / 2) * own + 4ull * 32ull * (unsigned)v->r);
 }
 
 Segment make_segment(const Prepared& A, const Prepared& B, long long ta, long long tb,
@@ -2549,7 +2641,7 @@ static int count_impl(const double* ca, long long n_a, const double* cb, long lo
     const size_t smem = v->smem(K, tab.n_lut);
     const int want_per_sm = tune && tune->blocks_per_sm ? tune->blocks_per_sm : 0;
     int resident = 0;  // blocks resident at once
-    if ((rc = grid_for(v, smem, 1LL << 40, di.sm_count, want_per_sm, &resident))) return rc;
+    if ((rc = grid_for(v, smem, 1LL << 36, di.sm_count, want_per_sm, &resident))) return rc;
     // skip tile pairs wholly beyond the top edge (their pairs are overflow),
     // unless the items fill at most two waves of the launch: the caps and the
     // culling launches then cost about what they could save
@@ -2685,7 +2777,7 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
     const size_t smem = v->smem(K, tab.n_lut);
     const int want_per_sm = tune && tune->blocks_per_sm ? tune->blocks_per_sm : 0;
     int resident = 0;  // blocks resident at once
-    if ((rc = grid_for(v, smem, 1LL << 40, di.sm_count, want_per_sm, &resident))) return rc;
+    if ((rc = grid_for(v, smem, 1LL << 36, di.sm_count, want_per_sm, &resident))) return rc;
     // skip far tile pairs unless the items fill at most two waves of the
     // launch (the caps and the culling launches then cost about what they
     // could save) or a shard split needs the kept items per row
@@ -3275,6 +3367,7 @@ static int autotune(wtheta_plan* P, const DeviceInfo& di, cudaStream_t st, int* 
     long long cur_T = -1;
     for (int i = 0; i < nv && !rc; ++i) {
         const Variant* v = &vs[i];
+        if (v->def == 2) continue;  // spans are never worth leaving out here
         const size_t smem = v->smem(P->K, P->tab.n_lut);
         if (smem > (size_t)di.max_smem_optin) continue;
         const long long T = (long long)v->nt * v->r;

@@ -1,6 +1,7 @@
 // Host-side parts of libwtheta: bin edges (Sec. 2.1), squared-chord edges
 // (App. A geometry), the FP32 guard band and screening table used by the
 // counting kernels, and the Landy-Szalay estimator (Eq. 2).
+#include <algorithm>
 #include <cmath>
 #include <limits>
 #include <cstring>
@@ -145,9 +146,10 @@ int build_table(const double* edges_deg, int K, BinTable* t) {
     // range (their values go through a band search), the coarsest on ties
     int best_shift = -1;
     long long best_width = -1;
-    for (int shift = 30; shift >= 0; --shift) {
+    for (int shift = kMaxLutShift; shift >= 0; --shift) {
+        // (one entry is kept free for a bucket below the lowest)
         long long n = (long long)(t->h_top >> shift) - (long long)(lo_first >> shift) + 1;
-        if (n > kMaxLut) break;
+        if (n >= kMaxLut) break;
         // count buckets that meet more than one band
         int complex_buckets = 0;
         long long prev_bucket = -1;
@@ -171,16 +173,21 @@ int build_table(const double* edges_deg, int K, BinTable* t) {
         }
         if (complex_buckets == 0) break;
     }
-    if (best_shift < 0) best_shift = 30;
+    if (best_shift < 0) best_shift = kMaxLutShift;
     const int shift = best_shift;
     const long long base = lo_first >> shift;
     const long long top = t->h_top >> shift;
     t->shift = shift;
     t->base = (int32_t)base;
-    t->n_lut = (int32_t)(top - base + 1);
     t->n_complex = 0;
     // slot below the first band: the number of edges with c = 0 (0 or 1)
     const int slot0 = bands[0].k;
+    int n = 0;
+    auto plain = [&](int slot) {
+        t->lut[n][0] = 0xFFFFFFFFu;
+        t->lut[n][1] = (uint32_t)slot;
+        ++n;
+    };
     for (long long q = base; q <= top; ++q) {
         const uint32_t q_lo = (uint32_t)(q << shift);
         const uint32_t q_hi = (uint32_t)(((q + 1) << shift) - 1);
@@ -193,22 +200,29 @@ int build_table(const double* edges_deg, int K, BinTable* t) {
                 if (which < 0) which = (int)i;
             }
         }
-        uint32_t* e = t->lut[q - base];
         if (hits == 0) {
-            e[0] = 0xFFFFFFFFu; e[1] = 0xFFFFFFFFu;
-            e[2] = (uint32_t)slot_before; e[3] = (uint32_t)slot_before;
-        } else if (hits == 1) {
-            e[0] = bands[which].lo; e[1] = bands[which].hi;
-            e[2] = (uint32_t)bands[which].k; e[3] = (uint32_t)(bands[which].k + 1);
-        } else {
-            // every in-range value of the bucket is placed by a search of the
-            // bands (FP64 only inside one); one beyond the top edge (only the
-            // top bucket can hold one) is overflow
-            e[0] = 0u; e[1] = t->h_top;
-            e[2] = (uint32_t)(K + 1); e[3] = (uint32_t)(K + 1);
-            ++t->n_complex;
+            plain(slot_before);
+            continue;
         }
+        // the band (or the run of several) inside the bucket
+        uint32_t lo = q_lo, hi = std::min(q_hi, t->h_top);
+        uint32_t tag = (uint32_t)K | kLutSeveral;
+        if (hits == 1) {
+            lo = std::max(bands[which].lo, q_lo);
+            hi = std::min(bands[which].hi, q_hi);
+            tag = (uint32_t)bands[which].k;
+        } else {
+            ++t->n_complex;
+            if (q == base && base > 0) {
+                plain(slot0);
+                --t->base;
+            }
+        }
+        t->lut[n][0] = lo;
+        t->lut[n][1] = ((hi - lo) << kLutWidthShift) | tag;
+        ++n;
     }
+    t->n_lut = n;
     return WTHETA_OK;
 }
 

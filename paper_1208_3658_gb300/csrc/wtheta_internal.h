@@ -10,23 +10,30 @@
 namespace wtheta {
 
 constexpr int kMaxBins = 256;      // K upper limit (slots 0..K+1)
-constexpr int kMaxLut = 512;       // entries of the FP32 screening table
+constexpr int kMaxLut = 1024;      // entries of the FP32 screening table
 
 // Screening table for one edge set, built on the host, read by every counting
 // kernel.  Non-negative FP32 values order like their bit patterns, so the
 // kernel works on the bits of the FP32 squared chord s:
 //   - bits > h_top: at or above the top edge for certain -> overflow slot,
 //     which is never stored (it is the pair total minus the other slots);
-//   - else idx = max((bits >> shift) - base, 0), e = lut[idx] and
-//       bits < e.x -> slot e.z,  bits > e.y -> slot e.w,
-//       otherwise the pair is inside an edge's guard band (or the bucket holds
-//       more than one band) and is recomputed in FP64 against c64;
+//   - else idx = max((bits >> shift) - base, 0), e = lut[idx], with the slot
+//     s = e.y & kLutSlot and the width w = e.y >> kLutWidthShift of the edge's
+//     guard band inside the bucket: bits < e.x -> slot s, bits > e.x + w ->
+//     slot s + 1, otherwise the pair is inside the band and is recomputed in
+//     FP64 against c64 (a bucket without an edge has e.x = 0xFFFFFFFF);
 //   - slot K+1 (overflow) in the table, and any value beyond h_top, goes to a
 //     trash row that is never added to the counts;
-//   - a bucket holding several bands has {0, h_top, K+1, K+1}: all its
-//     in-range values are rechecked, values beyond h_top are overflow;
+//   - a bucket holding several bands (kLutSeveral) is a band all over, with
+//     s = K: its in-range values are rechecked, values beyond h_top (only the
+//     top bucket can hold one) are overflow; if it is the lowest, a bucket
+//     without an edge goes below it, for the values that idx clamps up;
 //   - every band's upper bound is at most h_top, so a value beyond h_top is
 //     never taken for a band value.
+// 8 bytes an entry: the lookups' lanes go to unrelated entries, so their bank
+// conflicts grow with the entry's size.
+constexpr uint32_t kLutSlot = 511u, kLutSeveral = 512u;
+constexpr int kLutWidthShift = 10, kMaxLutShift = 22;  // a band's width in a bucket < 2^22
 struct BinTable {
     int32_t K;
     uint32_t h_top;        // FP32 bits of the top edge's upper guard bound
@@ -36,7 +43,7 @@ struct BinTable {
     int32_t n_complex;     // buckets holding more than one guard band
     double c64[kMaxBins + 1];            // FP64 squared-chord edges
     float edge[kMaxBins + 1][2];         // {fl32(c_k), half slack of the local form} (local_guard)
-    uint32_t lut[kMaxLut][4];            // {lo_bits, hi_bits, slot_below, slot_above}
+    uint32_t lut[kMaxLut][2];            // {lo_bits, width | several | slot_below}
 };
 
 
@@ -109,6 +116,7 @@ struct PairParams {
 
 struct Variant {
     int nt, r, ju, hm, def;
+    int max_parts;                    // log2 of the most parts an item is taken in
     void (*kernel)(PairParams);       // the build with statistics code
     void (*kernel_fast)(PairParams);  // the build launched without statistics
     size_t (*smem)(int, int);

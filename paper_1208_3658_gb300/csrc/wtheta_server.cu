@@ -348,7 +348,7 @@ bool launch_round(wtheta_server* S, Round& R) {
         rc = check_cuda(cudaMemcpyAsync(R.d_segs, R.h_segs, sizeof(Segment) * n,
                                         cudaMemcpyHostToDevice, R.st));
         if (!rc) rc = check_cuda(cudaMemsetAsync(R.d_cursor, 0, 8, R.st));
-        const int grid = (int)std::min<long long>(S->grid, items);
+        const int grid = (int)std::min<long long>(S->grid, items << S->v->max_parts);
         PairParams prm = make_params(S->v, S->tab, nullptr, R.d_segs, n, 0, items, R.d_cursor,
                                      nullptr);
         prm.span = S->span;
