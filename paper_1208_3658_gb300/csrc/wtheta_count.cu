@@ -506,11 +506,12 @@ __global__ void __launch_bounds__(64) k_joint_keys(const double* __restrict__ a,
 }
 
 // One chunk of 32 consecutive positions of the spatial order, one point per
-// lane (q its FP32 copy, (px, py, pz) its FP64 one): the chunk's bounding
-// sphere and the points' coordinates relative to the sphere's centre c.
-//   - Sphere: centre = the FP32 mean of the chunk's points, radius = the
-//     largest FP32 distance of a point from it, enlarged by a relative 1e-6
-//     for the few roundings of that arithmetic.
+// lane (q its FP32 copy, (px, py, pz) its FP64 one): the bounding spheres of
+// the chunk and of its groups of 8 points, and the points' coordinates relative
+// to the chunk's centre c.
+//   - Spheres (small_sphere): radius = the largest FP32 distance of a point from
+//     the centre, enlarged by a relative 1e-6 for the few roundings of that
+//     arithmetic.
 //   - Local coordinates b' = fl32(b - c), from the FP64 points: the rounding is
 //     relative to |b'|, so a chunk's own geometry is kept to 2^-24 of its size.
 //   - For the pair kernel's local form (one_edge_step) the chunk keeps
@@ -527,27 +528,79 @@ struct LocalChunks {
     float* xyz;       // planar local coordinates, stride apart
     long long stride;
     float4* caps;     // per chunk: centre, radius
+    float4* groups;   // the same per group of 8 points
     float2* kap;      // per chunk: kappa, half the slack
 };
+// Bounding sphere of the points q of W adjacent lanes (8 or 32), nearly the
+// smallest one: from the middle of their bounding box (c), eight steps towards
+// the farthest point by 1/3, 1/4, ... of the distance (Badoiu and Clarkson), the
+// best centre kept.  Against spheres around the mean, radii shrink by 13% (8
+// points) and 8% (32) for uniform points and by a quarter for clustered ones,
+// and with them the number of spans that hold an edge.
+template <int W>
+__device__ __forceinline__ float4 small_sphere(const float4& q, float3 c) {
+    const unsigned lane = threadIdx.x & 31u;
+    auto most = [](unsigned v) {
+        if constexpr (W == 32) {
+            return __reduce_max_sync(0xffffffffu, v);
+        } else {
+#pragma unroll
+            for (int o = 1; o < W; o <<= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+            return v;
+        }
+    };
+    float3 b = c;
+    float best = __int_as_float(0x7f800000);
+#pragma unroll 1
+    for (int it = 0; it < 9; ++it) {
+        const float dx = q.x - c.x, dy = q.y - c.y, dz = q.z - c.z;
+        // the farthest lane, from the squared distance without its last bits
+        const unsigned far =
+            most((__float_as_uint(dx * dx + dy * dy + dz * dz) & ~31u) | lane);
+        const float m = __uint_as_float(far & ~31u);
+        if (m < best) {
+            best = m;
+            b = c;
+        }
+        const float st = 1.f / (float)(it + 3);
+        c.x += st * (__shfl_sync(0xffffffffu, q.x, far & 31u) - c.x);
+        c.y += st * (__shfl_sync(0xffffffffu, q.y, far & 31u) - c.y);
+        c.z += st * (__shfl_sync(0xffffffffu, q.z, far & 31u) - c.z);
+    }
+    const float dx = q.x - b.x, dy = q.y - b.y, dz = q.z - b.z;
+    const float r2 = __uint_as_float(most(__float_as_uint(dx * dx + dy * dy + dz * dz)));
+    return make_float4(b.x, b.y, b.z, sqrtf(r2) * (1.f + 1e-6f));
+}
+
 __device__ __forceinline__ void write_chunk(long long i, const float4& q, double px, double py,
                                             double pz, const LocalChunks& L) {
     const int lane = threadIdx.x & 31;
-    float sx = q.x, sy = q.y, sz = q.z;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        sy += __shfl_xor_sync(0xffffffffu, sy, o);
-        sz += __shfl_xor_sync(0xffffffffu, sz, o);
-    }
-    float cx = sx * (1.f / 32), cy = sy * (1.f / 32), cz = sz * (1.f / 32);
-    const float dx = q.x - cx, dy = q.y - cy, dz = q.z - cz;
-    float m = dx * dx + dy * dy + dz * dz;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    // (a NaN coordinate leaves the sum NaN and the centre with it)
+    float3 lo = make_float3(q.x, q.y, q.z), hi = lo;
+    auto widen = [&](int o) {
+        lo.x = fminf(lo.x, __shfl_xor_sync(0xffffffffu, lo.x, o));
+        lo.y = fminf(lo.y, __shfl_xor_sync(0xffffffffu, lo.y, o));
+        lo.z = fminf(lo.z, __shfl_xor_sync(0xffffffffu, lo.z, o));
+        hi.x = fmaxf(hi.x, __shfl_xor_sync(0xffffffffu, hi.x, o));
+        hi.y = fmaxf(hi.y, __shfl_xor_sync(0xffffffffu, hi.y, o));
+        hi.z = fmaxf(hi.z, __shfl_xor_sync(0xffffffffu, hi.z, o));
+    };
+    auto middle = [&] {
+        return make_float3(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z));
+    };
+    widen(1);
+    widen(2);
+    widen(4);
+    const float4 group = small_sphere<8>(q, middle());
+    if ((lane & 7) == 0) L.groups[i / 8] = group;
+    widen(8);
+    widen(16);
+    const float4 sphere = small_sphere<32>(q, middle());
+    float cx = sphere.x, cy = sphere.y, cz = sphere.z;
+    const float r = sphere.w;
+    // padding; NaN coordinates (which fminf and fmaxf pass over, but not r)
     const bool pad = __any_sync(0xffffffffu, is_sentinel(q));
-    float r = sqrtf(m) * (1.f + 1e-6f);
-    const bool wide = !(r <= 0.5f && cx * cx + cy * cy + cz * cz <= 4.f);
+    const bool nan = __any_sync(0xffffffffu, !(q.x + q.y + q.z == q.x + q.y + q.z));
+    const bool wide = nan || !(r <= 0.5f && cx * cx + cy * cy + cz * cz <= 4.f);
     if (pad || wide) cx = cy = cz = 0.f;
     const double ex = px - (double)cx, ey = py - (double)cy, ez = pz - (double)cz;
     const double kb = ex * (px + (double)cx) + ey * (py + (double)cy) + ez * (pz + (double)cz);
@@ -571,18 +624,17 @@ __device__ __forceinline__ void write_chunk(long long i, const float4& q, double
     }
 }
 
-// FP32 and FP64 copies of both catalogues in the joint order (order: the
-// sorted positions of x, a's points first): FP32 with a's points at [0, na)
+// FP32 copies of both catalogues in the joint order (order: the sorted
+// positions of x, a's points first): a's points at [0, na)
 // and sentinels up to pa, b's at [pa, pa + nb) and sentinels up to pa + pb
 // (tags tag0 and tag0 + 1), each point keeping in w its index within its own
-// catalogue, and the chunks' spheres and local coordinates; FP64 without
-// padding (stride na + nb, b's points from na on).  One warp per chunk (pa and
-// pb are multiples of 32).  L.xyz may lie where the sort kept its keys.
+// catalogue, and the chunks' spheres and local coordinates.  One warp per chunk
+// (pa and pb are multiples of 32).  L.xyz may lie where the sort kept its keys.
 __global__ void __launch_bounds__(256) k_gather_joint(const double* __restrict__ x, long long na,
                                                       long long pa, long long nb, long long pb,
                                                       const unsigned* __restrict__ order, int tag0,
                                                       float4* __restrict__ p32,
-                                                      double* __restrict__ s64, LocalChunks L) {
+                                                      LocalChunks L) {
     const long long N = na + nb, P = pa + pb;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P;
          i += (long long)gridDim.x * blockDim.x) {
@@ -591,15 +643,11 @@ __global__ void __launch_bounds__(256) k_gather_joint(const double* __restrict__
         double px, py, pz;
         float4 q;
         if (j < n) {
-            const long long o = (in_b ? na : 0) + j;
-            const long long k = order[o];
+            const long long k = order[(in_b ? na : 0) + j];
             px = x[k];
             py = x[N + k];
             pz = x[2 * N + k];
             q = point32(px, py, pz, in_b ? k - na : k);
-            s64[o] = px;
-            s64[N + o] = py;
-            s64[2 * N + o] = pz;
         } else {
             q = sentinel32(tag0 + (in_b ? 1 : 0), j - n);
             px = q.x;
@@ -962,14 +1010,11 @@ __device__ __forceinline__ unsigned edges_below(double x, unsigned c64, int K) {
 }
 
 // FP64 recheck: the definition's squared chord and slot for the pair of
-// sorted positions (ia, jb), read from the FP64 copies in the spatial order,
-// or from the caller's FP64 arrays through the original indices kept in the
-// FP32 copies (S.sorted64 says which); c64 is the shared address of
-// the FP64 edges.  hint >= 0: the slot just below the one edge whose guard
+// sorted positions (ia, jb), read from the FP64 arrays through the original
+// indices kept in the FP32 copies; c64 is the shared address of the FP64 edges.  hint >= 0: the slot just below the one edge whose guard
 // band held the FP32 value (checked, else the edges are searched in order).
 __device__ __forceinline__ double pair_chord2(const Segment& S, long long ia, long long jb) {
-    const long long i = (S.sorted64 & 1) ? ia : __float_as_int(S.a32[ia].w);
-    const long long j = (S.sorted64 & 2) ? jb : __float_as_int(S.b32[jb].w);
+    const long long i = __float_as_int(S.a32[ia].w), j = __float_as_int(S.b32[jb].w);
     const double* a = S.a64;
     const double* b = S.b64;
     const long long as = S.a64_stride, bs = S.b64_stride;
@@ -1245,33 +1290,6 @@ __device__ __forceinline__ void exact_steps(int j0, int j1, unsigned tile, unsig
                                                                   top_idx, K, S, a0, b0 + j, sC);
         }
     }
-}
-
-// Bounding sphere of the thread's R A points (FP32), given relative to their
-// chunk's centre c: centre = c + their mean, radius = the largest distance
-// from the mean, enlarged by a relative 1e-6 for the roundings of that
-// arithmetic.  Padding sentinels give a radius far above 2.
-template <int R>
-__device__ __forceinline__ float4 group_cap(const f2_t (&ax)[R / 2], const f2_t (&ay)[R / 2],
-                                            const f2_t (&az)[R / 2], const float4& c) {
-    float x[R], y[R], z[R];
-#pragma unroll
-    for (int q = 0; q < R / 2; ++q) {
-        unpack2(ax[q], x[2 * q], x[2 * q + 1]);
-        unpack2(ay[q], y[2 * q], y[2 * q + 1]);
-        unpack2(az[q], z[2 * q], z[2 * q + 1]);
-    }
-    float cx = 0.f, cy = 0.f, cz = 0.f;
-#pragma unroll
-    for (int r = 0; r < R; ++r) { cx += x[r]; cy += y[r]; cz += z[r]; }
-    cx *= 1.f / R; cy *= 1.f / R; cz *= 1.f / R;
-    float m = 0.f;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const float dx = x[r] - cx, dy = y[r] - cy, dz = z[r] - cz;
-        m = fmaxf(m, dx * dx + dy * dy + dz * dz);
-    }
-    return make_float4(c.x + cx, c.y + cy, c.z + cz, sqrtf(m) * (1.f + 1e-6f));
 }
 
 // How the pairs of a group of A points (sphere ga) with a chunk of B points
@@ -1834,6 +1852,7 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
     constexpr unsigned NP = (unsigned)(R * kChunk);
     constexpr unsigned RING = 4u * kRing, RINGS = RING * kJobKinds;  // bytes: a ring, a warp's
     constexpr unsigned FULL = 0x202020u;  // some fill (8 bits per kind) is 32 or more
+    static_assert(R == 8, "groups of write_chunk");
     static_assert(NW <= 8 && TB / kChunk <= 256 && UB % kChunk == 0 && kChunk % JU == 0,
                   "job fields");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1876,10 +1895,7 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
                         continue;
                     }
                     if (sub != cap_sub) {
-                        f2_t ax[R / 2], ay[R / 2], az[R / 2];
-                        const long long pos = lds_s64(sIJ) * TA + sub * SA + lane * R;
-                        load_local<R>(S.al, S.al_stride, pos, ax, ay, az);
-                        ga = group_cap<R>(ax, ay, az, __ldg(S.a_caps + pos / kChunk));
+                        ga = __ldg(S.a_groups + (lds_s64(sIJ) * TA + sub * SA) / R + lane);
                         own = diag ? (sub * SA + lane * R) / kChunk : -1;
                         cap_sub = sub;
                     }
@@ -2490,17 +2506,17 @@ int spatial_order(const double* x64, long long stride, long long n, int check,
     return check_cuda(cudaGetLastError());
 }
 
-// The FP32 part of a prepared set of P padded positions: points, then chunk
-// spheres; and the part that may lie where the sort kept its buffers: local
+// The FP32 part of a prepared set of P padded positions: points, then the
+// spheres of chunks and groups; and the part that may lie where the sort kept its buffers: local
 // coordinates and the chunks' kappa and slack.
 static size_t a256(size_t b) { return (b + 255) / 256 * 256; }
+static size_t sphere_bytes(long long P) { return a256((size_t)P / 32 * 16) + a256((size_t)P / 8 * 16); }
 static size_t local_bytes(long long P) { return a256((size_t)P * 12) + (size_t)P / 32 * 8; }
 
 size_t prepare_joint_bytes(long long na, long long pa, long long nb, long long pb) {
     const long long N = na + nb, P = pa + pb;
     size_t b = a256((size_t)P * 16);              // FP32 points
-    b += a256((size_t)P / 32 * 16);               // chunk bounding spheres
-    b += a256((size_t)N * 24);                    // FP64, spatial order
+    b += sphere_bytes(P);                         // bounding spheres
     b += a256((size_t)N * 24);                    // FP64, input order
     // the sort; once the order is known its other buffers become the local
     // coordinates
@@ -2518,9 +2534,8 @@ int prepare_joint(const double* a, long long na, long long pa, const double* b, 
     float4* p32 = (float4*)sp;
     sp += a256((size_t)P * 16);
     float4* c32 = (float4*)sp;
-    sp += a256((size_t)P / 32 * 16);
-    double* s64 = (double*)sp;
-    sp += a256((size_t)N * 24);
+    float4* groups = (float4*)(sp + a256((size_t)P / 32 * 16));
+    sp += sphere_bytes(P);
     double* x = (double*)sp;
     sp += a256((size_t)N * 24);
     const SortBufs S = sort_bufs(sp, N, 0);
@@ -2529,6 +2544,7 @@ int prepare_joint(const double* a, long long na, long long pa, const double* b, 
     L.xyz = (float*)sp;
     L.stride = P;
     L.caps = c32;
+    L.groups = groups;
     L.kap = (float2*)(sp + a256((size_t)P * 12));
     if (N > 0) {
         const long long g = std::min<long long>((N + 63) / 64, (long long)sm_count * 32);
@@ -2546,25 +2562,19 @@ int prepare_joint(const double* a, long long na, long long pa, const double* b, 
     }
     if (P > 0) {
         k_gather_joint<<<launch_grid(P, sm_count), 256, 0, st>>>(x, na, pa, nb, pb, S.idx[0], tag0,
-                                                                 p32, s64, L);
+                                                                 p32, L);
         count_launch();
     }
     A->p32 = p32;
     A->c32 = c32;
+    A->groups = groups;
     A->kap = L.kap;
     A->l32 = L.xyz;
     A->l_stride = P;
-    A->x64 = s64;
+    A->x64 = x;
     A->stride = N;
-    A->sorted = 1;
-    B->p32 = p32 + pa;
-    B->c32 = c32 + pa / 32;
-    B->kap = L.kap + pa / 32;
-    B->l32 = L.xyz + pa;
-    B->l_stride = P;
-    B->x64 = s64 + na;
-    B->stride = N;
-    B->sorted = 1;
+    *B = tile_view(*A, pa);
+    B->x64 = x + na;
     return check_cuda(cudaGetLastError());
 }
 
@@ -2592,6 +2602,7 @@ int launch_gather_regions(const double* x64, long long stride, const unsigned* o
     L.xyz = (float*)out.l32;
     L.stride = out.l_stride;
     L.caps = (float4*)out.c32;
+    L.groups = (float4*)out.groups;
     L.kap = (float2*)out.kap;
     k_gather_regions<<<launch_grid(n_pad, sm_count), 256, 0, st>>>(
         x64, stride, order, src, dst, R, n_pad, (float4*)out.p32, tag, L);
@@ -2600,7 +2611,7 @@ int launch_gather_regions(const double* x64, long long stride, const unsigned* o
 }
 
 size_t regions_bytes(long long n_pad) {
-    return a256((size_t)n_pad * 16) + a256((size_t)n_pad / 32 * 16) + a256(local_bytes(n_pad));
+    return a256((size_t)n_pad * 16) + sphere_bytes(n_pad) + a256(local_bytes(n_pad));
 }
 
 Prepared regions_layout(unsigned char* p, long long n_pad) {
@@ -2608,7 +2619,8 @@ Prepared regions_layout(unsigned char* p, long long n_pad) {
     q.p32 = (const float4*)p;
     p += a256((size_t)n_pad * 16);
     q.c32 = (const float4*)p;
-    p += a256((size_t)n_pad / 32 * 16);
+    q.groups = (const float4*)(p + a256((size_t)n_pad / 32 * 16));
+    p += sphere_bytes(n_pad);
     q.l32 = (const float*)p;
     q.l_stride = n_pad;
     q.kap = (const float2*)(p + a256((size_t)n_pad * 12));
@@ -2619,6 +2631,7 @@ Prepared tile_view(const Prepared& A, long long pos) {
     Prepared q = A;
     q.p32 += pos;
     q.c32 += pos / 32;
+    q.groups += pos / 8;
     q.kap += pos / 32;
     q.l32 += pos;
     return q;
@@ -2658,6 +2671,7 @@ Segment make_segment(const Prepared& A, const Prepared& B, long long ta, long lo
     std::memset(&g, 0, sizeof(g));
     g.a32 = A.p32; g.b32 = B.p32; g.a64 = A.x64; g.b64 = B.x64;
     g.a_caps = A.c32;
+    g.a_groups = A.groups;
     g.al = A.l32;
     g.al_stride = A.l_stride;
     g.b_caps = B.c32;
@@ -2665,7 +2679,6 @@ Segment make_segment(const Prepared& A, const Prepared& B, long long ta, long lo
     g.bl = B.l32;
     g.bl_stride = B.l_stride;
     g.a64_stride = A.stride; g.b64_stride = B.stride;
-    g.sorted64 = (A.sorted ? 1 : 0) | (B.sorted ? 2 : 0);
     g.tiles_a = ta; g.tiles_b = tb;
     g.item_begin = item_begin;
     g.n_items = is_auto ? ta * (ta + 1) / 2 : ta * tb;

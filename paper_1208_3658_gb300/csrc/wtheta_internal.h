@@ -59,7 +59,7 @@ enum HistMode { kHistLane = 1, kHistWarp = 2, kHistLaneAtomic = 3, kHistWarpRed 
 struct Segment {
     const float4* a32;       // FP32 points (x, y, z, original index bits), tile-padded
     const float4* b32;
-    const double* a64;       // FP64 SoA, stride a64_stride (order: sorted64)
+    const double* a64;       // FP64 SoA, stride a64_stride, in the original order
     const double* b64;
     long long a64_stride, b64_stride;
     long long tiles_a, tiles_b;
@@ -71,13 +71,13 @@ struct Segment {
     const unsigned* item_list;   // if set: the count's kept items (tile pairs not skipped)
     const float4* b_caps;    // bounding spheres of B's chunks of 32 sorted points, or null
     const float4* a_caps;    // the same of A's chunks
+    const float4* a_groups;  // and of A's groups of 8 sorted points
     const float* al;         // A's local coordinates (planar, al_stride apart)
     long long al_stride;
     const float2* b_kap;     // per chunk of B: kappa and half the slack (with b_caps)
     const float* bl;         // B's local coordinates (planar, bl_stride apart; with b_caps)
     long long bl_stride;
     int is_auto;
-    int sorted64;            // bit 0 (a64), bit 1 (b64): in the spatial order, else original
 };
 
 // Bounding cap of one tile of spatially ordered points: unit centre and an
@@ -96,7 +96,6 @@ struct CullSeg {
     long long ta, tb;
     unsigned* list;
     int is_auto;
-    int sorted64;            // bit 0 (a64), bit 1 (b64): in the spatial order, else original
 };
 
 struct PairParams {
@@ -133,12 +132,12 @@ struct DeviceInfo {
 struct Prepared {
     const float4* p32 = nullptr;
     const float4* c32 = nullptr;   // bounding sphere of each chunk of 32 sorted points
+    const float4* groups = nullptr;  // the same of each group of 8
     const float2* kap = nullptr;   // kappa and half the slack of each chunk
     const float* l32 = nullptr;    // coordinates relative to the chunk's centre (planar, l_stride)
     long long l_stride = 0;
-    const double* x64 = nullptr;   // FP64 SoA (stride), in the spatial order if sorted
+    const double* x64 = nullptr;   // FP64 SoA (stride), in the original order
     long long stride = 0;
-    int sorted = 0;
 };
 
 // Host-side launch plumbing (wtheta_count.cu), shared by the single-count,
