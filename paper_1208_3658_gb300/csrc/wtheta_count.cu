@@ -1074,13 +1074,14 @@ struct PairKernel {
     }
     static constexpr unsigned ROWB = 4u * HSTRIDE;
 
-    // log2 of the most parts an item is taken in: quarters of the B tile (the
-    // units of several warps), or single chunks in a one-warp block
+    // log2 of the most parts an item is taken in: quarters of the B tile (two
+    // units of several warps each), or single chunks in a one-warp block
     static constexpr int MAXLP = NW == 1 ? ilog2(TB / 32) : 2;
 
     static size_t smem_bytes(int K, int n_lut) {
         size_t b = (size_t)TB / 32 * kChunkB;   // B tile
         b += (size_t)TB / 32 * 16;              // bounding spheres of its 32-point chunks
+        b += (size_t)TA / 8 * 16;               // bounding spheres of A's groups of 8
         b += (size_t)n_lut * 8;                 // screening table
         b += (size_t)(K + 2) * 8;               // FP64 edges (+ pad)
         b += (size_t)(K + 2) * 8;               // middle and half slack of every edge
@@ -1328,6 +1329,10 @@ __device__ __forceinline__ int span_edges(float4 ga, float4 gb, unsigned lut, un
     const unsigned bl = __float_as_uint(slo), bh = __float_as_uint(shi);
     // padding (a group's radius far above 2, a chunk's -1), a wide chunk, NaN
     const bool real = (ga.w <= 2.f) & (gb.w >= 0.f) & (gb.w <= 2.f);
+    if (__all_sync(0xffffffffu, real && bl > h_top)) {  // the whole warp beyond the top edge
+        rlo = rhi = (unsigned)K + 1u;
+        return 0;
+    }
     const uint2 el = lut_entry(bl, lut, shift, base, top_idx);
     const uint2 eh = lut_entry(bh, lut, shift, base, top_idx);
     rlo = lut_slot(el) + ((lut_below(el, bl) | lut_band(el, bl)) ? 0u : 1u);
@@ -1554,7 +1559,7 @@ __device__ __forceinline__ void recentre(const float4& a, const float4& b, const
     }
 }
 
-// Sphere of chunk c of the staged tile (caps: shared address).
+// Sphere c of the staged chunks or groups (caps: shared address).
 __device__ __forceinline__ float4 chunk_sphere(unsigned caps, int c) {
     const uint4 g = lds_u4(caps + 16u * (unsigned)c);
     return make_float4(__uint_as_float(g.x), __uint_as_float(g.y), __uint_as_float(g.z),
@@ -1577,7 +1582,10 @@ __device__ __forceinline__ float4 chunk_sphere(unsigned caps, int c) {
 constexpr int kJobOne = 0, kJobTwo = 1, kJobExact = 2, kJobKinds = 3, kChunk = 32;
 constexpr int kRing = 64;  // words of a ring: fewer than 32 waiting, at most 32 pushed at once
 
-// Bits 0-4 lane, 5-7 sub-tile, 8-15 chunk, 16-29 the (first) edge.
+// Bits 0-4 lane, 5-7 sub-tile, 8-15 chunk, 16-24 the (first) edge.  While a
+// lane still has jobs of a span to push, bits 25-30 of its word hold the number
+// of edges left, or kExact for one job pair by pair.
+constexpr unsigned kExact = 32u, kJobBits = (1u << 25) - 1u;
 __device__ __forceinline__ unsigned job_word(int lane, int sub, int chunk, unsigned slot) {
     return (unsigned)lane | ((unsigned)sub << 5) | ((unsigned)chunk << 8) | (slot << 16);
 }
@@ -1658,7 +1666,7 @@ __device__ __forceinline__ void span_part(int T, unsigned job, int t0, int ts, u
     f2_t ax[R / 2], ay[R / 2], az[R / 2], a0[R / 2];
     float4 ca;
     job_points<NT, R, JU, HM>(job, sIJ, S, ca, ax, ay, az);
-    const unsigned edge = (job >> 16) & 0x3FFFu;
+    const unsigned edge = (job >> 16) & 511u;
     float G, G2 = 0.f;
     const float mid = edge_mid(band, edge, G);
     {
@@ -1780,7 +1788,7 @@ __device__ __forceinline__ void job_round(int T, unsigned run, bool active, int 
             mb2 = fminf(mb2, __shfl_xor_sync(0xffffffffu, mb2, o));
         }
         const bool first = active && t0 == 0;
-        const unsigned edge = (run >> 16) & 0x3FFFu;
+        const unsigned edge = (run >> 16) & 511u;
         // jobs with a value within the slack of their first or second edge
         unsigned b1 = __ballot_sync(0xffffffffu, first && !(mb1 > 0.f));
         unsigned b2 = __ballot_sync(0xffffffffu, first && !(mb2 > 0.f));
@@ -1790,7 +1798,7 @@ __device__ __forceinline__ void job_round(int T, unsigned run, bool active, int 
             const int src = __ffs(second ? b2 : b1) - 1;
             if (second) b2 &= b2 - 1u; else b1 &= b1 - 1u;
             const unsigned j = __shfl_sync(0xffffffffu, run, src);
-            const unsigned v = recount_edge<NT, R>(j, ((j >> 16) & 0x3FFFu) + (second ? 1u : 0u),
+            const unsigned v = recount_edge<NT, R>(j, ((j >> 16) & 511u) + (second ? 1u : 0u),
                                                    sIJ, band, sC, S);
             if (lane == src) {
                 if (second) neg2 = v & 0xFFFFu; else neg1 = v & 0xFFFFu;
@@ -1842,12 +1850,12 @@ __device__ __forceinline__ int round_share(int T, int m) {
 template <int NT, int R, int JU, int HM, bool ST>
 __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsigned sIJ,
                                           unsigned tile, unsigned lut, unsigned caps,
-                                          unsigned band, unsigned sC, unsigned hist,
+                                          unsigned groups, unsigned band, unsigned sC, unsigned hist,
                                           const PairParams& p, const Segment& S, bool diag,
                                           int part, int lp, unsigned stat) {
     using PK = PairKernel<NT, R, JU, HM, 0>;
     constexpr int TA = PK::TA, TB = PK::TB;
-    constexpr int NW = NT / 32, SA = 32 * R, UPS = 4, UB = TB / UPS, CPU = UB / kChunk;
+    constexpr int NW = NT / 32, SA = 32 * R, UPS = 8, UB = TB / UPS, CPU = UB / kChunk;
     constexpr unsigned row_bytes = PK::ROWB;
     constexpr unsigned NP = (unsigned)(R * kChunk);
     constexpr unsigned RING = 4u * kRing, RINGS = RING * kJobKinds;  // bytes: a ring, a warp's
@@ -1863,60 +1871,53 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
     const int c_begin = (part * (TB / kChunk)) >> lp, c_end = ((part + 1) * (TB / kChunk)) >> lp;
     unsigned fills = 0;   // jobs waiting per kind, 8 bits each; bit 24 + T: ring T starts at 32
     unsigned word = 0;    // this lane's next job (of the chunk it has classified)
-    int left = 0;         // the edges it still has to push jobs for; kExact: pair by pair
-    constexpr int kExact = 256;
-    int k = 0, sub = 0, own = -1, cn = 0, ce = 0;  // chunks [cn, ce) of the current unit left
-    int cap_sub = -1;
-    int pool = -1;                         // kind of the pooled leftovers being run
-    float4 ga = make_float4(0.f, 0.f, 0.f, 0.f);
+    // chunks left of the current unit (next, end), its sub-tile, sub-tiles done
+    // (bits 0, 8, 16, 20): one register across the rounds
+    unsigned at_unit = 0;
+    int pool = -1;        // kind of the pooled leftovers being run
 #pragma unroll 1
     for (;;) {
         int T, m = 32, lts = 0;
         unsigned at = 0;  // shared address of this lane's job
         if (pool < 0 && (fills & FULL) == 0u) {
-            if (!__any_sync(0xffffffffu, left != 0)) {
+            if (!__any_sync(0xffffffffu, (word >> 25) != 0u)) {
                 // the next chunk
 #pragma unroll 1
-                while (k < NW && cn >= ce) {
-                    sub = (warp + k) & (NW - 1);
+                while ((at_unit & 255u) >= ((at_unit >> 8) & 255u) && (at_unit >> 20) < (unsigned)NW) {
+                    const unsigned k = at_unit >> 20, sub = ((unsigned)warp + k) & (NW - 1);
                     unsigned u = 0;
-                    if (lane == 0) u = atom_add_shared(units + 4u * (unsigned)sub, 1u);
+                    if (lane == 0) u = atom_add_shared(units + 4u * sub, 1u);
                     u = __shfl_sync(0xffffffffu, u, 0);
                     // (a one-warp block takes its part of the tile as one unit)
-                    cn = NW == 1 ? c_begin : (int)u * CPU;
-                    ce = NW == 1 ? c_end : cn + CPU;
+                    const int cn = NW == 1 ? c_begin : (int)u * CPU;
+                    const int ce = NW == 1 ? c_end : cn + CPU;
                     if (NW == 1 ? u != 0u : cn >= c_end) {
-                        ++k;
-                        cn = ce;
+                        at_unit = (k + 1u) << 20;
                         continue;
                     }
-                    if (diag && ce * kChunk <= sub * SA) {  // every pair has i >= j
-                        cn = ce;
-                        continue;
-                    }
-                    if (sub != cap_sub) {
-                        ga = __ldg(S.a_groups + (lds_s64(sIJ) * TA + sub * SA) / R + lane);
-                        own = diag ? (sub * SA + lane * R) / kChunk : -1;
-                        cap_sub = sub;
-                    }
+                    // (in a diagonal tile pair: every pair of the unit has i >= j)
+                    if (diag && ce * kChunk <= (int)sub * SA) continue;
+                    at_unit = (unsigned)cn | ((unsigned)ce << 8) | (sub << 16) | (k << 20);
                 }
-                if (k == NW) {
+                if ((at_unit >> 20) == (unsigned)NW) {
                     pool = 0;  // every unit taken: the leftovers
                     __syncthreads();  // the rings are quiescent
                     if (lane == 0) sts_u32(units + 4u * (unsigned)warp, fills);
                     __syncthreads();
                     continue;
                 }
-                const int c = cn++;
+                const int c = (int)(at_unit & 255u), sub = (int)((at_unit >> 16) & 7u);
+                ++at_unit;
                 unsigned rlo = 0, rhi = 0;
-                const int n = span_edges(ga, chunk_sphere(caps, c), lut, sC, p.tab.shift,
-                                         p.tab.base, p.tab.n_lut - 1, p.tab.K, p.tab.h_top, rlo,
-                                         rhi);
+                const int n = span_edges(chunk_sphere(groups, sub * 32 + lane), chunk_sphere(caps, c),
+                                         lut, sC, p.tab.shift, p.tab.base, p.tab.n_lut - 1, p.tab.K,
+                                         p.tab.h_top, rlo, rhi);
+                const int own = diag ? (sub * SA + lane * R) / kChunk : -1;
                 const bool mine = c > own;
                 // (to the trash row if nothing is settled: no branch)
                 hist_add<HM>(col + (mine && n >= 0 ? rhi : (unsigned)p.tab.K + 1u) * row_bytes, NP);
-                left = !mine ? 0 : n < 0 ? kExact : n;
-                word = job_word(lane, sub, c, rlo);
+                word = job_word(lane, sub, c, rlo) |
+                       ((!mine ? 0u : n < 0 ? kExact : (unsigned)n) << 25);
                 if (stats) {
                     warp_stat(stat + 8u, mine && n >= 0, NP);
                     warp_stat(stat + 16u, mine ? n == 0 : c < own, NP);
@@ -1924,17 +1925,19 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
             }
             // push one job of every lane that has some left: the odd edge alone,
             // then the others by twos
-            const bool one = (left & 1) != 0;
+            const unsigned left = word >> 25;
+            const bool one = (left & 1u) != 0u, exact = left == kExact;
             const unsigned m1 = __ballot_sync(0xffffffffu, one);
-            const unsigned m3 = __ballot_sync(0xffffffffu, left == kExact);
-            const unsigned m2 = __ballot_sync(0xffffffffu, left != 0) & ~(m1 | m3);
-            const int Tp = one ? kJobOne : left == kExact ? kJobExact : kJobTwo;
-            const unsigned mk = one ? m1 : left == kExact ? m3 : m2;
+            const unsigned m3 = __ballot_sync(0xffffffffu, exact);
+            const unsigned m2 = __ballot_sync(0xffffffffu, left != 0u) & ~(m1 | m3);
+            const int Tp = one ? kJobOne : exact ? kJobExact : kJobTwo;
+            const unsigned mk = one ? m1 : exact ? m3 : m2;
             const unsigned pos = (fills >> (8 * Tp)) + ((fills >> (24 + Tp)) << 5) +
                                  (unsigned)__popc(mk & ((1u << lane) - 1u));
-            sts_u32_if(left != 0, ring + RING * (unsigned)Tp + ((4u * pos) & (RING - 4u)), word);
-            word += one ? 1u << 16 : 2u << 16;
-            left = left == kExact || left == 0 ? 0 : left - (one ? 1 : 2);
+            sts_u32_if(left != 0u, ring + RING * (unsigned)Tp + ((4u * pos) & (RING - 4u)),
+                       word & kJobBits);
+            const unsigned by = left == 0u ? 0u : one ? 1u : 2u;
+            word += exact ? 0u - (kExact << 25) : (by << 16) - (by << 25);
             fills += (unsigned)__popc(m1) + ((unsigned)__popc(m2) << 8) + ((unsigned)__popc(m3) << 16);
             if ((fills & FULL) == 0u) continue;
         }
@@ -2002,13 +2005,29 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
     __syncwarp();
 }
 
+// The overflow slots of a launch's counts, total minus the other slots, one warp
+// per count: by the last block to finish, after all others' counts.  Out of
+// line, as its registers would weigh on the kernel's.
+__device__ __noinline__ void fill_overflow(const PairParams& p) {
+    __threadfence();
+    const int K = p.tab.K;
+    for (int q = threadIdx.x >> 5; q < max(p.n_segs, 1); q += blockDim.x >> 5) {
+        const Segment& g = p.n_segs > 0 ? p.segs[q] : p.seg0;
+        unsigned long long sum = 0;
+        for (int k = threadIdx.x & 31; k <= K; k += 32) sum += __ldcg(g.counts + k);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if ((threadIdx.x & 31) == 0) g.counts[K + 1] = g.total - sum;
+    }
+}
+
 // ST: with the span path's statistics code (a launch with p.stats set); the
 // build without it is the one launched when no statistics are asked for.
 template <int NT, int R, int JU, int HM, int DEF, bool ST>
 __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __grid_constant__ PairParams p) {
     using PK = PairKernel<NT, R, JU, HM, DEF>;
     constexpr int TA = PK::TA, TB = PK::TB, HCOLS = PK::HCOLS, HSTRIDE = PK::HSTRIDE;
-    constexpr int NW = NT / 32, SA = 32 * R, UPS = 4, UB = TB / UPS;
+    constexpr int NW = NT / 32, SA = 32 * R, UPS = 8, UB = TB / UPS;
     static_assert(TA == NW * SA && TB % UPS == 0, "units tile the item");
     __shared__ unsigned s_units[NW];
     // span job rings (one per kind and warp) for the shapes that bin spans
@@ -2016,7 +2035,8 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = p.tab.K;
     float4* sCap = reinterpret_cast<float4*>(smem + TB / 32 * kChunkB);
-    uint2* sLut = reinterpret_cast<uint2*>(sCap + TB / 32);
+    float4* sGroup = sCap + TB / 32;  // spheres of A's groups
+    uint2* sLut = reinterpret_cast<uint2*>(sGroup + TA / 8);
     double* sC = reinterpret_cast<double*>(sLut + p.tab.n_lut);
     float2* sBand = reinterpret_cast<float2*>(sC + (K + 2));
     unsigned* hist = reinterpret_cast<unsigned*>(sBand + (K + 2));
@@ -2028,11 +2048,15 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
     __shared__ unsigned long long s_stat[3];  // span-path rechecks, span pairs, skipped pairs
 
     const int tid = threadIdx.x;
+    // the parameter block through its generic address: lanes that index the
+    // constant bank each at their own place are served one by one
+    const PairParams* gp = &p;
+    asm volatile("" : "+l"(gp));
     for (int q = tid; q < p.tab.n_lut; q += NT)
-        sLut[q] = make_uint2(p.tab.lut[q][0], p.tab.lut[q][1]);
+        sLut[q] = make_uint2(gp->tab.lut[q][0], gp->tab.lut[q][1]);
     for (int q = tid; q <= K; q += NT) {
-        sC[q] = p.tab.c64[q];
-        sBand[q] = make_float2(p.tab.edge[q][0], p.tab.edge[q][1]);
+        sC[q] = gp->tab.c64[q];
+        sBand[q] = make_float2(gp->tab.edge[q][0], gp->tab.edge[q][1]);
     }
     for (int q = tid; q < (K + 2) * HSTRIDE; q += NT) hist[q] = 0u;
     if (tid < 3) s_stat[tid] = 0ull;
@@ -2121,6 +2145,7 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
                 stage2(j, x.x, y.x, z.x, x.y, y.y, z.y);
             }
             for (int q = tid; q < TB / 32; q += NT) sCap[q] = S.b_caps[J * (TB / 32) + q];
+            for (int q = tid; q < TA / 8; q += NT) sGroup[q] = S.a_groups[I * (TA / 8) + q];
         } else {
             const float4* gB = S.b32 + J * TB;
 #pragma unroll 4
@@ -2131,10 +2156,12 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
         }
         if (tid < NW) s_units[tid] = NW == 1 ? 0 : part * UPS >> lp;
         __syncthreads();  // B tile staged, unit counters reset
-        const unsigned a_lut = smem_addr(sLut), a_cap = smem_addr(sCap), a_band = smem_addr(sBand),
+        const unsigned a_lut = smem_addr(sLut), a_cap = smem_addr(sCap), a_group = smem_addr(sGroup), a_band = smem_addr(sBand),
                        a_hist = smem_addr(hist), a_c = smem_addr(sC);
         // The item is split into units of one warp's worth of A points (SA =
-        // 32 R consecutive points, a sub-tile) by a quarter of the B tile.  A
+        // 32 R consecutive points, a sub-tile) by an eighth of the B tile (the
+        // warps of a block end an item within less of one another than with
+        // quarters: survey 33.3 -> 32.9 ms).  A
         // warp takes the units of its own sub-tile first, then those left of
         // the others, so the warps of the block finish the item together
         // whatever the mix of cheap and costly units.
@@ -2143,7 +2170,7 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
         if constexpr (DEF == 0 && HM != kHistWarp) {
             if (spans)
                 span_item<NT, R, JU, HM, ST>(smem_addr(s_units), smem_addr(s_ring),
-                                         smem_addr(s_IJ[n_items & 1]), a_tile, a_lut, a_cap, a_band, a_c,
+                                         smem_addr(s_IJ[n_items & 1]), a_tile, a_lut, a_cap, a_group, a_band, a_c,
                                          a_hist, p, S, diag, part, lp, smem_addr(s_stat));
         }
         int cur = -1;
@@ -2186,6 +2213,13 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
     }
     // all threads left the loop after the same barrier
     if (cur_seg != -2) flush_hist<NT, HCOLS, HSTRIDE>(hist, K, sSeg.counts);
+    if (p.done) {
+        __threadfence();  // this block's counts before its mark
+        __syncthreads();
+        if (tid == 0) s_item = atomicAdd(p.done, 1ull) + 1ull == gridDim.x ? 1 : 0;
+        __syncthreads();
+        if (s_item) fill_overflow(p);
+    }
     if (p.stats) {
         unsigned long long v = n_recheck;
 #pragma unroll
@@ -2206,24 +2240,37 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
 }
 
 // The device tables of a w(theta) launch (its counts' segments and culling
-// table), written by one small kernel from its parameters, which also zeroes
-// n0 words at z0 and n1 at z1 (the launch cursor and the kept counters).
+// table), written by one small kernel from its parameters before anything else
+// of the count; it also zeroes what the later kernels add to (counts, launch
+// cursor, kept counters, the digit counts of a small sort), one launch instead
+// of a copy from pageable memory and three memsets.
 struct CountTables {
     Segment segs[3];
     CullSeg cs[3];
     int n_segs;
     int with_cull;
+    unsigned* zero[4];   // words to zero
+    long long n_zero[4];
 };
-__global__ void k_set_tables(const CountTables t, Segment* __restrict__ segs,
-                             CullSeg* __restrict__ cs, unsigned long long* __restrict__ z0, int n0,
-                             unsigned long long* __restrict__ z1, int n1) {
-    const int i = threadIdx.x;
+__global__ void __launch_bounds__(256) k_begin_count(const __grid_constant__ CountTables t,
+                                                     Segment* __restrict__ segs,
+                                                     CullSeg* __restrict__ cs) {
+    const long long i = blockIdx.x * 256LL + threadIdx.x;
     if (i < t.n_segs) {
         segs[i] = t.segs[i];
         if (t.with_cull) cs[i] = t.cs[i];
     }
-    if (i < n0) z0[i] = 0ull;
-    if (i < n1) z1[i] = 0ull;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        for (long long j = i; j < t.n_zero[q]; j += 256LL * gridDim.x) t.zero[q][j] = 0u;
+}
+static int launch_begin_count(const CountTables& t, Segment* segs, CullSeg* cs, cudaStream_t st) {
+    long long n = 1;
+    for (int q = 0; q < 4; ++q) n = std::max(n, t.n_zero[q]);
+    const unsigned g = (unsigned)std::min<long long>((n + 255) / 256, 128);
+    k_begin_count<<<g, 256, 0, st>>>(t, segs, cs);
+    count_launch();
+    return check_cuda(cudaGetLastError());
 }
 
 // counts[K+1] = total - sum(counts[0..K]) for every count of a batch.
@@ -2292,15 +2339,15 @@ int device_info(DeviceInfo* out) {
     return WTHETA_OK;
 }
 
-// The default shape for one call: tiles of 256 points (one warp) when the
-// larger catalogue has at most 16k points and of 512 points (64 threads) up
-// to 64k, so that a small count still has tile pairs for every SM and each
-// CTA's share stays short; the 1024-point shape otherwise.
+// The default shape for one call by the larger catalogue's size: tiles of 256
+// points (one warp) up to 4096, of 512 points (64 threads) up to 32768, else of
+// 1024.  w(theta) with 32, 64, 128 threads: 1k + 1k points 96, 121, 148 us; 10k +
+// 10k 262, 246, 254 us (host copies included); cross 30k x 48k - , 443, 431 us.
 const Variant* pick_for_size(const wtheta_tune* tune, long long n_max, int K, int n_lut,
                              int max_smem) {
-    if (!tune && n_max <= 65536) {
+    if (!tune && n_max <= 32768) {
         wtheta_tune small = {};
-        small.threads = n_max <= 16384 ? 32 : 64;
+        small.threads = n_max <= 4096 ? 32 : 64;
         small.points_per_thread = 8;
         const Variant* v = pick_variant(&small, K, n_lut, max_smem);
         if (v) return v;
@@ -2524,32 +2571,52 @@ size_t prepare_joint_bytes(long long na, long long pa, long long nb, long long p
     return b;
 }
 
+void prepare_layout(long long na, long long pa, long long nb, long long pb, unsigned char* scratch,
+                    Prepared* A, Prepared* B) {
+    const long long N = na + nb, P = pa + pb;
+    unsigned char* sp = scratch;
+    A->p32 = (const float4*)sp;
+    sp += a256((size_t)P * 16);
+    A->c32 = (const float4*)sp;
+    A->groups = (const float4*)(sp + a256((size_t)P / 32 * 16));
+    sp += sphere_bytes(P);
+    A->x64 = (const double*)sp;
+    A->stride = N;
+    sp += a256((size_t)N * 24) + a256((size_t)N * 4);  // and the sorted order
+    A->l32 = (const float*)sp;
+    A->l_stride = P;
+    A->kap = (const float2*)(sp + a256((size_t)P * 12));
+    *B = tile_view(*A, pa);
+    B->x64 = A->x64 + na;
+}
+
+void prepare_zero(long long na, long long pa, long long nb, long long pb, unsigned char* scratch,
+                  unsigned** words, long long* n) {
+    const long long N = na + nb, P = pa + pb;
+    unsigned char* sort = scratch + a256((size_t)P * 16) + sphere_bytes(P) + a256((size_t)N * 24);
+    *words = sort_bufs(sort, N, 0).hist;
+    *n = N <= kSmallSort ? small_blocks(N) * 4 * 256 : 0;
+}
+
 int prepare_joint(const double* a, long long na, long long pa, const double* b, long long nb,
                   long long pb, int is_xyz, int tag0, unsigned char* scratch, int sm_count,
-                  cudaStream_t st, Prepared* A, Prepared* B) {
+                  cudaStream_t st, Prepared* A, Prepared* B, bool zeroed) {
     TraceRange trace("prepare");
     const long long N = na + nb, P = pa + pb;
     if (N >= (1LL << 32) - 1) return WTHETA_EINVAL;  // 32-bit positions in the sort
-    unsigned char* sp = scratch;
-    float4* p32 = (float4*)sp;
-    sp += a256((size_t)P * 16);
-    float4* c32 = (float4*)sp;
-    float4* groups = (float4*)(sp + a256((size_t)P / 32 * 16));
-    sp += sphere_bytes(P);
-    double* x = (double*)sp;
-    sp += a256((size_t)N * 24);
-    const SortBufs S = sort_bufs(sp, N, 0);
-    sp += a256((size_t)N * 4);                    // S.idx[0], the order
+    prepare_layout(na, pa, nb, pb, scratch, A, B);
+    double* x = (double*)A->x64;
+    const SortBufs S = sort_bufs((unsigned char*)x + a256((size_t)N * 24), N, 0);
     LocalChunks L;
-    L.xyz = (float*)sp;
+    L.xyz = (float*)A->l32;
     L.stride = P;
-    L.caps = c32;
-    L.groups = groups;
-    L.kap = (float2*)(sp + a256((size_t)P * 12));
+    L.caps = (float4*)A->c32;
+    L.groups = (float4*)A->groups;
+    L.kap = (float2*)A->kap;
     if (N > 0) {
         const long long g = std::min<long long>((N + 63) / 64, (long long)sm_count * 32);
         const bool small = N <= kSmallSort;
-        if (small) {
+        if (small && !zeroed) {
             const int rc = check_cuda(
                 cudaMemsetAsync(S.hist, 0, (size_t)small_blocks(N) * 4 * 256 * 4, st));
             if (rc) return rc;
@@ -2562,19 +2629,9 @@ int prepare_joint(const double* a, long long na, long long pa, const double* b, 
     }
     if (P > 0) {
         k_gather_joint<<<launch_grid(P, sm_count), 256, 0, st>>>(x, na, pa, nb, pb, S.idx[0], tag0,
-                                                                 p32, L);
+                                                                 (float4*)A->p32, L);
         count_launch();
     }
-    A->p32 = p32;
-    A->c32 = c32;
-    A->groups = groups;
-    A->kap = L.kap;
-    A->l32 = L.xyz;
-    A->l_stride = P;
-    A->x64 = x;
-    A->stride = N;
-    *B = tile_view(*A, pa);
-    B->x64 = x + na;
     return check_cuda(cudaGetLastError());
 }
 
@@ -2739,13 +2796,13 @@ static int count_impl(const double* ca, long long n_a, const double* cb, long lo
     DeviceInfo di;
     if ((rc = device_info(&di))) return rc;
 
-    if ((rc = check_cuda(cudaMemsetAsync(counts, 0, sizeof(unsigned long long) * (K + 2), st))))
-        return rc;
     const unsigned long long total =
         is_auto ? (unsigned long long)n_a * (unsigned long long)(n_a > 0 ? n_a - 1 : 0) / 2ull
                 : (unsigned long long)n_a * (unsigned long long)n_b;
     const bool empty = is_auto ? n_a < 2 : (n_a == 0 || n_b == 0);
     if (empty) {
+        if ((rc = check_cuda(cudaMemsetAsync(counts, 0, sizeof(unsigned long long) * (K + 2), st))))
+            return rc;
         k_finalize<<<1, 1, 0, st>>>(counts, K, total);
         count_launch();
         return check_cuda(cudaGetLastError());
@@ -2778,12 +2835,21 @@ static int count_impl(const double* ca, long long n_a, const double* cb, long lo
     void* scratch = nullptr;
     if ((rc = dev_malloc_async(&scratch, bytes, st))) return rc;
     unsigned char* sp = (unsigned char*)scratch;
-    unsigned long long* cursor = (unsigned long long*)sp;
+    unsigned long long* cursor = (unsigned long long*)sp;  // cursor, kept count, blocks done
     Prepared A, B;
-    rc = prepare_joint(ca, n_a, pa, is_auto ? nullptr : cb, is_auto ? 0 : n_b, is_auto ? 0 : pb,
-                       is_xyz, 0, sp + 256, di.sm_count, st, &A, &B);
+    CountTables begin;
+    std::memset(&begin, 0, sizeof(begin));
+    begin.zero[0] = (unsigned*)counts;
+    begin.n_zero[0] = 2LL * (K + 2);
+    begin.zero[1] = (unsigned*)cursor;
+    begin.n_zero[1] = 2 * 3;
+    prepare_zero(n_a, pa, is_auto ? 0 : n_b, is_auto ? 0 : pb, sp + 256, &begin.zero[2],
+                 &begin.n_zero[2]);
+    rc = launch_begin_count(begin, nullptr, nullptr, st);
+    if (!rc)
+        rc = prepare_joint(ca, n_a, pa, is_auto ? nullptr : cb, is_auto ? 0 : n_b,
+                           is_auto ? 0 : pb, is_xyz, 0, sp + 256, di.sm_count, st, &A, &B, true);
     if (is_auto) B = A;
-    if (!rc) rc = check_cuda(cudaMemsetAsync(cursor, 0, 2 * sizeof(unsigned long long), st));
 
     unsigned* list = nullptr;
     unsigned long long* n_list = nullptr;
@@ -2809,14 +2875,8 @@ static int count_impl(const double* ca, long long n_a, const double* cb, long lo
         PairParams prm = make_params(v, tab, &seg, nullptr, 0, 0, n_items, cursor, stats);
         prm.n_items_dev = n_list;
         prm.span = !(tune && tune->span_bins == 2);
-        pair_kernel(v, prm)<<<grid, v->nt, smem, st>>>(prm);
-        count_launch();
-        rc = check_cuda(cudaGetLastError());
-        if (!rc) {
-            k_finalize<<<1, 1, 0, st>>>(counts, K, total);
-            count_launch();
-            rc = check_cuda(cudaGetLastError());
-        }
+        prm.done = cursor + 2;
+        rc = launch_pairs(v, prm, grid, smem, st);
     }
     const cudaError_t fe = cudaFreeAsync(scratch, st);
     if (!rc) rc = check_cuda(fe);
@@ -2869,7 +2929,6 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
     DeviceInfo di;
     if ((rc = device_info(&di))) return rc;
     const size_t K2 = (size_t)K + 2;
-    if ((rc = check_cuda(cudaMemsetAsync(counts, 0, 3 * K2 * 8, st)))) return rc;
     const Variant* v = pick_for_size(tune, std::max(nd, nr), K, tab.n_lut, di.max_smem_optin);
     if (!v) return WTHETA_EINVAL;
     const long long T = (long long)v->nt * v->r;
@@ -2919,18 +2978,28 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
     if (cull) bytes += (size_t)total_items * 4;
     unsigned char* m = nullptr;
     if ((rc = dev_malloc_async((void**)&m, bytes, st))) return rc;
-    unsigned long long* cursor = (unsigned long long*)m;
+    unsigned long long* cursor = (unsigned long long*)m;  // cursor, kept count, blocks done
     unsigned long long* n_kept = cursor + 1;
     Segment* d_segs = (Segment*)(m + 256);
     CullSeg* d_cull = (CullSeg*)(m + 256 + 1024);
     unsigned long long* d_kept = (unsigned long long*)(m + 256 + 2048);
     static_assert(3 * sizeof(Segment) <= 1024 && 3 * sizeof(CullSeg) <= 1024, "tables fit");
     Prepared D, R;
-    rc = prepare_joint(cd, nd, pd, cr, nr, pr, is_xyz, 0, m + off_prep, di.sm_count, st, &D, &R);
+    CountTables tbl;  // without tables yet if the shard's rows are still to be chosen
+    std::memset(&tbl, 0, sizeof(tbl));
+    tbl.zero[0] = (unsigned*)counts;
+    tbl.n_zero[0] = 6LL * (long long)K2;
+    tbl.zero[1] = (unsigned*)cursor;
+    tbl.n_zero[1] = 2 * 3;
+    prepare_zero(nd, pd, nr, pr, m + off_prep, &tbl.zero[2], &tbl.n_zero[2]);
+    if (cull) {
+        tbl.zero[3] = (unsigned*)d_kept;
+        tbl.n_zero[3] = 2 * 3;
+    }
+    tbl.with_cull = cull ? 1 : 0;
+    prepare_layout(nd, pd, nr, pr, m + off_prep, &D, &R);
     TileCap* caps_d = (TileCap*)(m + off_caps);
     TileCap* caps_r = caps_d + td;  // R's tiles follow D's in the joint copies
-    if (!rc && (cull || n_shards > 1) && td + tr > 0)
-        rc = launch_tile_caps(D.p32, pd + pr, (int)T, td + tr, caps_d, st);
     const double theta_top = edges[K] * (3.14159265358979323846 / 180.0);
     auto cull_seg = [&](int i, long long begin) {
         const int k = cnts[i].kind;
@@ -2946,6 +3015,18 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
         c.cb = k == 0 ? caps_d : caps_r;
         return c;
     };
+    auto prepare_both = [&] {
+        int e = prepare_joint(cd, nd, pd, cr, nr, pr, is_xyz, 0, m + off_prep, di.sm_count, st, &D,
+                              &R, true);
+        if (!e && (cull || n_shards > 1) && td + tr > 0)
+            e = launch_tile_caps(D.p32, pd + pr, (int)T, td + tr, caps_d, st);
+        return e;
+    };
+    if (n_shards > 1) {
+        rc = launch_begin_count(tbl, d_segs, d_cull, st);
+        if (!rc) rc = prepare_both();
+        for (long long& z : tbl.n_zero) z = 0;
+    }
     if (!rc && n_shards > 1 && n_segs > 0) {
         // kept tile pairs per tile row of every count (all tile pairs count when
         // nothing is skipped), then this shard's rows of each count
@@ -3006,20 +3087,14 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
         cs[i].list = (unsigned*)(m + off_lists) + item;
         item += cnts[i].items;
     }
+    for (int i = 0; i < n_segs; ++i) {
+        tbl.segs[i] = segs[i];
+        tbl.cs[i] = cs[i];
+    }
+    tbl.n_segs = n_segs;
+    if (!rc) rc = launch_begin_count(tbl, d_segs, d_cull, st);
+    if (!rc && n_shards == 1) rc = prepare_both();
     if (!rc && n_segs > 0) {
-        // the segments and culling table, cursor and kept counters zeroed: one
-        // small launch instead of copies from pageable memory and memsets
-        CountTables tbl;
-        std::memset(&tbl, 0, sizeof(tbl));
-        for (int i = 0; i < n_segs; ++i) {
-            tbl.segs[i] = segs[i];
-            tbl.cs[i] = cs[i];
-        }
-        tbl.n_segs = n_segs;
-        tbl.with_cull = cull ? 1 : 0;
-        k_set_tables<<<1, 32, 0, st>>>(tbl, d_segs, d_cull, cursor, 2, d_kept, cull ? 3 : 0);
-        count_launch();
-        rc = check_cuda(cudaGetLastError());
         if (!rc && cull)
             rc = launch_cull_batch(d_cull, n_segs, total_items, theta_top, d_kept, d_segs, n_kept,
                                    di.sm_count, st, stats);
@@ -3030,9 +3105,11 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
                                          stats);
             if (cull) prm.n_items_dev = n_kept;
             prm.span = !(tune && tune->span_bins == 2);
+            prm.done = cursor + 2;
             rc = launch_pairs(v, prm, grid, smem, st);
+        } else if (!rc) {
+            rc = launch_finalize_segments(d_segs, n_segs, K, st);
         }
-        if (!rc) rc = launch_finalize_segments(d_segs, n_segs, K, st);
     }
     const cudaError_t fe = cudaFreeAsync(m, st);
     if (!rc) rc = check_cuda(fe);
@@ -3193,7 +3270,8 @@ static int count_xyz_noalloc_impl(const double* ca, long long n_a, const double*
         k_xyz_to_f32<<<cvt_grid(pb), cvt_threads, 0, st>>>(cb, n_b, pb, b32, 1);
         count_launch();
     }
-    if ((rc = check_cuda(cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), st)))) return rc;
+    // (cursor, a word unused here, blocks done)
+    if ((rc = check_cuda(cudaMemsetAsync(cursor, 0, 3 * sizeof(unsigned long long), st)))) return rc;
     const long long ta = pa / T, tb = is_auto ? ta : pb / T;
     const long long n_items = is_auto ? ta * (ta + 1) / 2 : ta * tb;
     const size_t smem = v->smem(K, tab.n_lut);
@@ -3203,13 +3281,9 @@ static int count_xyz_noalloc_impl(const double* ca, long long n_a, const double*
     A.p32 = a32; A.x64 = ca; A.stride = n_a;
     B.p32 = b32; B.x64 = cb; B.stride = n_b;
     const Segment seg = make_segment(A, B, ta, tb, is_auto, 0, counts, total);
-    const PairParams prm = make_params(v, tab, &seg, nullptr, 0, 0, n_items, cursor, nullptr);
-    pair_kernel(v, prm)<<<grid, v->nt, smem, st>>>(prm);
-    count_launch();
-    if ((rc = check_cuda(cudaGetLastError()))) return rc;
-    k_finalize<<<1, 1, 0, st>>>(counts, K, total);
-    count_launch();
-    return check_cuda(cudaGetLastError());
+    PairParams prm = make_params(v, tab, &seg, nullptr, 0, 0, n_items, cursor, nullptr);
+    prm.done = cursor + 2;
+    return launch_pairs(v, prm, grid, smem, st);
 }
 
 }  // namespace wtheta

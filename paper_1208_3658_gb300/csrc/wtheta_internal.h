@@ -107,6 +107,7 @@ struct PairParams {
     long long n_items;
     const unsigned long long* n_items_dev;  // if set: at most this many items (device count)
     unsigned long long* cursor;
+    unsigned long long* done;     // if set (zeroed): the last block to finish fills the overflow slots
     unsigned long long* stats;    // WTHETA_NSTATS or null
     int span;                // settle (A group, B chunk) spans without a lookup per pair
     int pad_;
@@ -162,7 +163,13 @@ int check_cuda(cudaError_t e);
 size_t prepare_joint_bytes(long long na, long long pa, long long nb, long long pb);
 int prepare_joint(const double* a, long long na, long long pa, const double* b, long long nb,
                   long long pb, int is_xyz, int tag0, unsigned char* scratch, int sm_count,
-                  cudaStream_t st, Prepared* A, Prepared* B);
+                  cudaStream_t st, Prepared* A, Prepared* B, bool zeroed = false);
+// Where prepare_joint puts the copies in scratch, and the words it needs zeroed
+// before (zeroed: the caller has done that).
+void prepare_layout(long long na, long long pa, long long nb, long long pb, unsigned char* scratch,
+                    Prepared* A, Prepared* B);
+void prepare_zero(long long na, long long pa, long long nb, long long pb, unsigned char* scratch,
+                  unsigned** words, long long* n);
 unsigned long long per_item_bound(const Variant* v);
 Segment make_segment(const Prepared& A, const Prepared& B, long long ta, long long tb,
                      int is_auto, long long item_begin, unsigned long long* counts,
