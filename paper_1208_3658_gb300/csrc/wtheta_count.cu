@@ -1870,10 +1870,59 @@ __device__ __forceinline__ int round_share(int T, int m) {
     return m == 1 ? (T == kJobExact ? 5 : 4) : l;
 }
 
+// Before an item's units: every sub-tile of A (32 R = 256 points, the sphere
+// around its 8 chunks' spheres) against every chunk of B, one pair per lane.
+// Where all 8192 pairs are in one slot, or beyond the top edge, they are
+// counted here and the chunk drops out of the sub-tile's list (a word of chunk
+// bits at todo + 4 sub), instead of 32 lanes finding that out one group each.
+// Not in a diagonal tile pair.
+template <int NT, int R, int JU, int HM, bool ST>
+__device__ __forceinline__ void settle_chunks(unsigned todo, unsigned lut, unsigned sC, unsigned hist,
+                                              const PairParams& p, const Segment& S, long long I,
+                                              long long J, bool diag, int part, int lp,
+                                              unsigned stat) {
+    using PK = PairKernel<NT, R, JU, HM, 0>;
+    constexpr int CPT = PK::TB / kChunk, SA = 32 * R;
+    static_assert(SA / kChunk == 8 && CPT <= 32, "8 chunks a sub-tile, a word of chunk bits");
+    const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
+    const float4 own = __ldg(S.a_caps + (I * PK::TA + sub * SA) / kChunk + (lane & 7));
+    const float4 gb = __ldg(S.b_caps + J * CPT + min(lane, CPT - 1));
+    float4 ga = own;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        ga.x += __shfl_xor_sync(0xffffffffu, ga.x, o);
+        ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o);
+        ga.z += __shfl_xor_sync(0xffffffffu, ga.z, o);
+    }
+    ga.x *= 0.125f; ga.y *= 0.125f; ga.z *= 0.125f;
+    const float dx = own.x - ga.x, dy = own.y - ga.y, dz = own.z - ga.z;
+    // (the factor and the term cover the roundings of this arithmetic; a chunk
+    // with padding or too wide a one leaves the sub-tile to its groups)
+    ga.w = own.w >= 0.f && own.w <= 0.5f
+               ? (sqrt_approx(dx * dx + dy * dy + dz * dz) + own.w) * (1.f + 4e-6f) + 2e-7f
+               : 3.f;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) ga.w = fmaxf(ga.w, __shfl_xor_sync(0xffffffffu, ga.w, o));
+    unsigned rlo = 0, rhi = 0;
+    const int n = span_edges(ga, gb, lut, sC, p.tab.shift, p.tab.base, p.tab.n_lut - 1, p.tab.K,
+                             p.tab.h_top, rlo, rhi);
+    const bool here = lane < CPT && lane >= (part * CPT) >> lp && lane < ((part + 1) * CPT) >> lp;
+    const bool settled = here && !diag && n == 0;
+    hist_add<HM>(hist + 4u * (unsigned)PK::column() +
+                     (settled ? rhi : (unsigned)p.tab.K + 1u) * PK::ROWB,
+                 (unsigned)(SA * kChunk));
+    const unsigned left = __ballot_sync(0xffffffffu, here && !settled);
+    if (lane == 0) sts_u32(todo + 4u * (unsigned)sub, left);
+    if (ST && p.stats != nullptr) {
+        warp_stat(stat + 8u, settled, (unsigned)(SA * kChunk));
+        warp_stat(stat + 16u, settled, (unsigned)(SA * kChunk));
+    }
+}
+
 // A warp's share of one item with span binning: units of its own sub-tile
 // first, then those left of the others (shared counters at address units, one
 // per sub-tile).  Each lane classifies its group against every chunk of a
-// unit; a chunk in one slot is counted at once, the others become jobs (the
+// unit that settle_chunks left; a chunk in one slot is counted at once, the others become jobs (the
 // warp's rings in the block's ring array at shared address rings, kRing words
 // per kind) and 32 jobs of a kind run as one round.  When every unit is taken,
 // the jobs left in all the warps' rings are pooled and shared out evenly (a
@@ -1901,8 +1950,9 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
     constexpr unsigned RING = 4u * kRing, RINGS = RING * kJobKinds;  // bytes: a ring, a warp's
     constexpr unsigned FULL = 0x202020u;  // some fill (8 bits per kind) is 32 or more
     static_assert(R == 8, "groups of write_chunk");
-    static_assert(NW <= 8 && TB / kChunk <= 256 && UB % kChunk == 0 && kChunk % JU == 0,
-                  "job fields");
+    static_assert(NW <= 8 && TB / kChunk <= 32 && UB % kChunk == 0 && CPU <= 8 && kChunk % JU == 0 &&
+                      (NW > 1 || TB / kChunk <= 8),
+                  "job fields, a unit's chunk bits");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned ring = rings + RINGS * (unsigned)warp;
     const unsigned col = hist + 4u * (unsigned)PK::column();
@@ -1911,8 +1961,8 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
     const int c_begin = (part * (TB / kChunk)) >> lp, c_end = ((part + 1) * (TB / kChunk)) >> lp;
     unsigned fills = 0;   // jobs waiting per kind, 8 bits each; bit 24 + T: ring T starts at 32
     unsigned word = 0;    // this lane's next job (of the chunk it has classified)
-    // chunks left of the current unit (next, end), its sub-tile, sub-tiles done
-    // (bits 0, 8, 16, 20): one register across the rounds
+    // the current unit: its first chunk, bits of the chunks left, its sub-tile,
+    // sub-tiles done (from bits 0, 8, 16, 20): one register across the rounds
     unsigned at_unit = 0;
     int pool = -1;        // kind of the pooled leftovers being run
 #pragma unroll 1
@@ -1923,7 +1973,7 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
             if (!__any_sync(0xffffffffu, (word >> 25) != 0u)) {
                 // the next chunk
 #pragma unroll 1
-                while ((at_unit & 255u) >= ((at_unit >> 8) & 255u) && (at_unit >> 20) < (unsigned)NW) {
+                while ((at_unit & 0xFF00u) == 0u && (at_unit >> 20) < (unsigned)NW) {
                     const unsigned k = at_unit >> 20, sub = ((unsigned)warp + k) & (NW - 1);
                     unsigned u = 0;
                     if (lane == 0) u = atom_add_shared(units + 4u * sub, 1u);
@@ -1937,7 +1987,9 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
                     }
                     // (in a diagonal tile pair: every pair of the unit has i >= j)
                     if (diag && ce * kChunk <= (int)sub * SA) continue;
-                    at_unit = (unsigned)cn | ((unsigned)ce << 8) | (sub << 16) | (k << 20);
+                    const unsigned bits = (lds_u32(units + 4u * (unsigned)NW + 4u * sub) >> cn) &
+                                          ((1u << (ce - cn)) - 1u);
+                    at_unit = (unsigned)cn | (bits << 8) | (sub << 16) | (k << 20);
                 }
                 if ((at_unit >> 20) == (unsigned)NW) {
                     pool = 0;  // every unit taken: the leftovers
@@ -1946,8 +1998,9 @@ __device__ __forceinline__ void span_item(unsigned units, unsigned rings, unsign
                     __syncthreads();
                     continue;
                 }
-                const int c = (int)(at_unit & 255u), sub = (int)((at_unit >> 16) & 7u);
-                ++at_unit;
+                const unsigned bit = at_unit & 0xFF00u & (0u - (at_unit & 0xFF00u));
+                const int c = (int)(at_unit & 255u) + 23 - __clz(bit), sub = (int)((at_unit >> 16) & 7u);
+                at_unit ^= bit;
                 unsigned rlo = 0, rhi = 0;
                 const int n = span_edges(chunk_sphere(groups, sub * 32 + lane), chunk_sphere(caps, c),
                                          lut, sC, p.tab.shift, p.tab.base, p.tab.n_lut - 1, p.tab.K,
@@ -2077,7 +2130,7 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
     constexpr int TA = PK::TA, TB = PK::TB, HCOLS = PK::HCOLS, HSTRIDE = PK::HSTRIDE;
     constexpr int NW = NT / 32, SA = 32 * R, UPS = 8, UB = TB / UPS;
     static_assert(TA == NW * SA && TB % UPS == 0, "units tile the item");
-    __shared__ unsigned s_units[NW];
+    __shared__ unsigned s_units[2 * NW];  // units taken; chunks left per sub-tile (spans)
     // span job rings (one per kind and warp) for the shapes that bin spans
     __shared__ unsigned s_ring[(DEF == 0 && HM != kHistWarp) ? NW * kJobKinds * kRing : 1];
     extern __shared__ __align__(16) unsigned char smem[];
@@ -2205,7 +2258,13 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
                 stage2(j, a.x, a.y, a.z, b.x, b.y, b.z);
             }
         }
-        if (tid < NW) s_units[tid] = NW == 1 ? 0 : part * UPS >> lp;
+        if (tid < NW) s_units[tid] = NW == 1 ? 0 : (part * UPS) >> lp;
+        if constexpr (DEF == 0 && HM != kHistWarp) {
+            if (spans)
+                settle_chunks<NT, R, JU, HM, ST>(smem_addr(s_units + NW), smem_addr(sLut),
+                                                 smem_addr(sC), smem_addr(hist), p, S, I, J,
+                                                 S.is_auto && I == J, part, lp, smem_addr(s_stat));
+        }
         __syncthreads();  // B tile staged, unit counters reset
         const unsigned a_lut = smem_addr(sLut), a_cap = smem_addr(sCap), a_group = smem_addr(sGroup), a_band = smem_addr(sBand),
                        a_hist = smem_addr(hist), a_c = smem_addr(sC);
@@ -2763,13 +2822,14 @@ unsigned long long per_item_bound(const Variant* v) {
     // jobs it also runs at most one job (R x 32 pairs, counted up or down in a
     // word) per round of its warp; the warp's jobs are at most
     // (kMaxEdgesFar + 1) / 2 per lane and chunk, so its full rounds add at most
-    // that many times own; after them come at most three pooled rounds and
-    // the pairs of its own chunk of a diagonal tile pair.  A per-warp column
+    // that many times own; before them come its chunk's pairs with a whole
+    // sub-tile (at most own), after them at most three pooled rounds and the
+    // pairs of its own chunk of a diagonal tile pair.  A per-warp column
     // gains 32 times as much, one shared by eight lanes eight times.
     const unsigned long long own = (unsigned long long)(v->nt / 32) * (unsigned long long)v->r *
                                    (unsigned long long)v->nt * (unsigned long long)v->r;
     return (v->hm == kHistWarp || v->hm == kHistWarpRed ? 32ull : 8ull) *
-           ((1ull + (kMaxEdgesFar + 1) / 2) * own + 4ull * 32ull * (unsigned)v->r);
+           ((2ull + (kMaxEdgesFar + 1) / 2) * own + 4ull * 32ull * (unsigned)v->r);
 }
 
 Segment make_segment(const Prepared& A, const Prepared& B, long long ta, long long tb,
