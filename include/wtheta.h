@@ -173,7 +173,8 @@ typedef struct wtheta_tune {
     int32_t points_per_thread; /* A points held in registers per thread: 8 or 16 */
     int32_t hist_mode;         /* 1: private per-thread histograms, plain add;
                                   2: per-warp histograms, warp-aggregated atomics;
-                                  3: private per-thread histograms, shared atomic add;
+                                  3: shared atomic add, to a column per thread or, where
+                                     span binning applies, to four columns per warp;
                                   4: per-warp histograms, shared atomic add (lanes on
                                      one word merged by the hardware)              */
     int32_t j_per_screen;      /* B points per screening test: 1 or 2          */
@@ -186,10 +187,10 @@ typedef struct wtheta_tune {
                                   when the tile pairs fill more than two waves of
                                   the launch                                      */
     int32_t span_bins;         /* 1: settle a thread's A points against a chunk of
-                                  32 B points in one slot, or by one compare per pair
-                                  against a single edge, when the bounding spheres
-                                  of the two groups allow it (exact); 2: bin every
-                                  pair through the table                          */
+                                  32 B points in one slot, or by counting the pairs
+                                  below each of a few edges, when the bounding
+                                  spheres of the two groups allow it (exact); 2: bin
+                                  every pair through the table                    */
 } wtheta_tune;
 
 /* statistics slots accumulated by wtheta_count_ex (uint64 each) */

@@ -13,24 +13,26 @@
 //     points is a compact patch of sky and a warp's pairs mostly share one
 //     fate (all beyond the top edge, or all in range);
 //   - tile pairs whose bounding caps lie wholly beyond the top edge are
-//     skipped (their pairs are overflow); inside a tile pair, a thread's group
-//     of R consecutive A points and a chunk of 32 B points are settled in one
-//     slot, or by one FP32 comparison per pair against a single edge, when
-//     their bounding spheres allow it;
+//     skipped (their pairs are overflow); inside a tile pair, a sub-tile of 256
+//     A points or a group of 8 and a chunk of 32 B points are settled in one
+//     slot, or by counting the pairs below each edge between them, when their
+//     bounding spheres allow it;
 //   - FP32 float4 copies (x, y, z, original index) padded to whole tiles with
-//     far-away sentinel points that never land in a bin;
+//     far-away sentinel points that never land in a bin, and planar FP32
+//     coordinates relative to the centre of each point's chunk;
 //   - a CTA stages the B tile in shared memory, negated and duplicated for
-//     packed FP32x2 arithmetic, and keeps R A points per thread in registers;
-//     the squared chord of two pairs costs 3 add.f32x2 + 1 mul.f32x2 +
-//     2 fma.f32x2, i.e. the 6 FP32 operations per pair in half the issue slots;
+//     packed FP32x2 arithmetic, and a lane keeps R A points in registers; against
+//     an edge two pairs cost 3 fma.f32x2 in those local coordinates, and a squared
+//     chord 3 add.f32x2 + 1 mul.f32x2 + 2 fma.f32x2;
 //   - s is screened against the top edge: pairs beyond it are overflow and
 //     cost nothing more (Sec. 2.2: separations outside the bin range can be
 //     skipped); the overflow slot is filled at the end as total minus the rest;
 //   - in-range pairs are binned by a table lookup on the bits of s, the FP32
 //     comparison being final outside a rigorous guard band around each edge;
 //     inside it the pair is recomputed in FP64 exactly as the definition says;
-//   - counts go to private per-thread (or per-warp, warp-aggregated) uint32
-//     shared histograms, flushed into uint64 global counts before any can wrap.
+//   - counts go to 32-bit shared histogram columns, a few per warp (or private
+//     to a thread or a warp), flushed into uint64 global counts before any can
+//     wrap.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -3872,7 +3874,7 @@ static int batch_plan_impl(const wtheta_catalog_pair* cats, int n_cats, int is_x
         P->tune.points_per_thread = P->v->r;
         P->tune.j_per_screen = P->v->ju;
         P->tune.hist_mode = P->v->hm;
-        P->tune.deferred = P->v->def + 1;
+        P->tune.deferred = P->v->def == 1 ? 2 : 1;
         P->tune.skip_far = P->cull ? 1 : 2;
         P->tune.span_bins = tune && tune->span_bins == 2 ? 2 : 1;
         P->smem = P->v->smem(K, P->tab.n_lut);

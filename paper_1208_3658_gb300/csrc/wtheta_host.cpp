@@ -66,7 +66,7 @@ double guard_half_width(double c) {
 }
 
 // Slack of the local form's s - mid around an edge c (the part that does not
-// depend on the chunk; see two_slot_step and write_chunk).
+// depend on the chunk; see one_edge_step and write_chunk).
 //
 // With a the FP64 point, c0 the chunk's centre (an FP32 vector, exact), r its
 // radius, q = |a32 - c0| <= sqrt(s) + r + u and mid = fl32(c), the kernel's
@@ -81,7 +81,7 @@ double guard_half_width(double c) {
 // and the chunk's deviation of kappa.  q^2 <= 1.1 c + 11 r^2 near the edge, so
 // the sum is u (2 sqrt(c) + 7.5 c + 10 r + 55 r^2 + 5 |kappa|) + deviation:
 // the first two terms here, the others per chunk.  The second edge of a
-// three-slot job adds 5 u c for its subtraction.  The terms 3 u |s - c| and
+// two-edge job adds 5 u c for its subtraction.  The terms 3 u |s - c| and
 // the growth of the bound with s are less than |s - c| itself by a factor 10
 // for c >= 1e-10 and lie within the 5% margin; smaller edges are never settled
 // in this form (infinite slack).  The FP64 predicate's own error (8 u64 s) and

@@ -49,7 +49,7 @@ struct BinTable {
 
 // Private histogram columns of the pair kernel: per thread, plain
 // read-modify-write (1); per warp, lanes merged by __match_any_sync (2); per
-// thread, shared reduction (3); per warp, shared reduction (4: the shared
+// thread, or four per warp with span jobs, shared reduction (3); per warp, shared reduction (4: the shared
 // atomic unit merges lanes that hit one word at full rate, and the rows of a
 // warp's column sit an odd number of words apart so that different rows hit
 // different banks).
