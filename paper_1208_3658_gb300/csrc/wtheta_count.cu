@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(64) k_joint_keys(const double* __restrict__ a,
 //     kappa = |b|^2 - |c|^2 (for unit vectors the same for every point of the
 //     chunk; the middle of its range here) and half the slack that the form
 //     adds to an edge's guard band for this chunk: the deviation of kappa from
-//     that middle, and u (10 r + 55 r^2 + 5 |kappa|) for the roundings that
+//     that middle, and u (12 r + 80 r^2 + 5 |kappa|) for the roundings that
 //     grow with the chunk's radius r (u = 2^-24; derived at local_guard in the
 //     host sources), times 1.05.
 // A chunk holding a padding sentinel gets radius -1 and one wider than 0.5 gets
@@ -619,7 +619,7 @@ __device__ __forceinline__ void write_chunk(long long i, const float4& q, double
         const float kappa = (float)(0.5 * (k0 + k1));
         const float dev = (float)fmax(k1 - (double)kappa, (double)kappa - k0);
         const float rr = r + 2.4e-7f;
-        const float slack = 1.05f * (dev + 5.9604645e-8f * (10.f * rr + 55.f * rr * rr +
+        const float slack = 1.05f * (dev + 5.9604645e-8f * (12.f * rr + 80.f * rr * rr +
                                                             5.f * fabsf(kappa)));
         L.caps[i / 32] = make_float4(cx, cy, cz, pad ? -1.f : wide ? 3.f : r);
         L.kap[i / 32] = make_float2(kappa, 0.5f * slack);
@@ -1594,7 +1594,9 @@ __device__ __forceinline__ void load_local(const float* __restrict__ p, long lon
 // the points themselves).  b - a is rounded relative to itself and the sum
 // relative to itself, so a coordinate difference against a point b' of b's
 // chunk errs by about 2 u |a - b| + u (ra + rb) instead of the 2 u of
-// differences of the FP32 copies: inside every guard band derived for those.
+// differences of the FP32 copies.  A squared chord of such differences errs by
+// at most u (10 s + sqrt(s) (6 r + 4 ra)), r and ra <= 0.5 (write_chunk): inside the
+// guard band derived for the FP32 copies, u (11.3 sqrt(c) + 22 c).
 template <int R>
 __device__ __forceinline__ void recentre(const float4& a, const float4& b, const f2_t (&ax)[R / 2],
                                          const f2_t (&ay)[R / 2], const f2_t (&az)[R / 2],

@@ -68,28 +68,34 @@ double guard_half_width(double c) {
 // Slack of the local form's s - mid around an edge c (the part that does not
 // depend on the chunk; see one_edge_step and write_chunk).
 //
-// With a the FP64 point, c0 the chunk's centre (an FP32 vector, exact), r its
-// radius, q = |a32 - c0| <= sqrt(s) + r + u and mid = fl32(c), the kernel's
-// value differs from s - c by at most, with u = 2^-24 and first order in u,
-//   2 u q + 2 u r        a32 = fl32(a) in |a - c0|^2 and in 2 a.b'
-//   2 u q^2              a' = fl32(a32 - c0), rounded relative to itself
-//   u |kappa - mid| + u c  kappa - mid and mid rounded
-//   3 u (max(c, q^2) + |kappa|)  the three roundings of |a'|^2 + (kappa - mid)
-//   4 u r + 3 u |s - c|  the three fmas: every partial sum is the result plus
-//                        products that add up to at most 2 r
-//   2 u r                b' rounded relative to itself
-// and the chunk's deviation of kappa.  q^2 <= 1.1 c + 11 r^2 near the edge, so
-// the sum is u (2 sqrt(c) + 7.5 c + 10 r + 55 r^2 + 5 |kappa|) + deviation:
-// the first two terms here, the others per chunk.  The second edge of a
-// two-edge job adds 5 u c for its subtraction.  The terms 3 u |s - c| and
-// the growth of the bound with s are less than |s - c| itself by a factor 10
-// for c >= 1e-10 and lie within the 5% margin; smaller edges are never settled
-// in this form (infinite slack).  The FP64 predicate's own error (8 u64 s) and
-// the second-order terms are inside 1e-13 + the margin.
+// With u = 2^-24 and first order in u: a is kept as a_l = fl32(a - ca) relative
+// to its own chunk's centre ca (radius ra <= 0.5), b as b' = fl32(b - cb) (radius
+// r); centres are FP32 vectors, so exact.  With q = |a - cb| <= sqrt(s) + r and
+// mid = fl32(c), the kernel's value differs from s - c by at most u times
+//   4 q^2 + 4 q ra     a' = fl(a_l + fl(ca - cb)): a_l, the centres' difference and
+//                      the sum are each rounded relative to themselves, at most
+//                      2 q + 2 ra in all, twice that times q in |a'|^2
+//   3 r                fl(a_l + ca) for a in 2 a.b'
+//   |kappa - mid| + c  kappa - mid and mid rounded
+//   3 (max(c, q^2) + |kappa|)  the three roundings of |a'|^2 + (kappa - mid)
+//   4 r + 3 |s - c|    the three fmas: every partial sum is the result plus
+//                      products that add up to at most 2 r
+//   2 r                b' rounded relative to itself
+// (a group whose chunk keeps the origin as its centre has a_l = fl32(a) and an
+// exact difference of centres: 2 q + 2 q^2 in the first line, within the same
+// bound) and by the chunk's deviation of kappa.  With 4 q ra <= 2 q <= 2 sqrt(c) + 2 r and
+// q^2 <= 1.1 c + 11 r^2 near the edge the sum is at most
+// 2 sqrt(c) + 10 c + 11 r + 77 r^2 + 4 |kappa|: the first two terms here, the
+// others (rounded up) per chunk.  The second edge of a two-edge job adds 5 c for
+// its subtraction.  The terms 3 |s - c| and the growth of the bound with s are
+// less than |s - c| itself by a factor 10 for c >= 1e-10 and lie within the 5%
+// margin; smaller edges are never settled in this form (infinite slack).  The
+// FP64 predicate's own error (8 u64 s) and the second-order terms are inside
+// 1e-13 + the margin.
 double local_guard(double c) {
     const double u = 5.9604644775390625e-08;  // 2^-24
     if (!(c >= 1e-10)) return std::numeric_limits<double>::infinity();
-    return 1.05 * u * (2.0 * std::sqrt(c) + 12.5 * c) + 1e-13;
+    return 1.05 * u * (2.0 * std::sqrt(c) + 16.0 * c) + 1e-13;
 }
 
 static float round_down_f(double x) {

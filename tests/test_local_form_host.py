@@ -22,8 +22,8 @@ def _fma(a, b, c):
 
 
 def _edge_slack(c):
-    """local_guard: 1.05 u (2 sqrt(c) + 12.5 c) + 1e-13, halved and rounded up."""
-    g = 0.5 * (1.05 * U * (2.0 * np.sqrt(c) + 12.5 * c) + 1e-13)
+    """local_guard: 1.05 u (2 sqrt(c) + 16 c) + 1e-13, halved and rounded up."""
+    g = 0.5 * (1.05 * U * (2.0 * np.sqrt(c) + 16.0 * c) + 1e-13)
     return np.nextafter(F(g), F(np.inf))
 
 
@@ -38,7 +38,7 @@ def _chunk(p):
     kappa = F(0.5 * (kb.min() + kb.max()))
     dev = max(kb.max() - float(kappa), float(kappa) - kb.min())
     rr = float(r) + 2.4e-7
-    slack = 1.05 * (dev + U * (10 * rr + 55 * rr * rr + 5 * abs(float(kappa))))
+    slack = 1.05 * (dev + U * (12 * rr + 80 * rr * rr + 5 * abs(float(kappa))))
     return c, loc, r, kappa, F(0.5 * slack)
 
 
