@@ -3036,6 +3036,31 @@ static long long row_item(long long I, long long ta, long long tb, int is_auto) 
     return is_auto ? I * ta - I * (I - 1) / 2 : I * tb;
 }
 
+// A w(theta)'s device scratch: cursor, kept total and blocks done, segments,
+// culling table and kept counts, both catalogues prepared together, tile caps
+// (n_caps of them: for the skipping, and for a shard split's kept items per row,
+// which reads them whether far tile pairs are skipped or not), kept items per
+// row with the first row of every count, kept lists.
+WthetaLayout wtheta_layout(long long nd, long long pd, long long nr, long long pr, long long T,
+                           bool cull, int n_shards, long long total_items) {
+    const long long td = pd / T, tr = pr / T;
+    WthetaLayout Y;
+    size_t b = 256 + 1024 + 1024 + 256;
+    Y.prep = b;
+    b += a256(prepare_joint_bytes(nd, pd, nr, pr));
+    Y.caps = b;
+    Y.n_caps = cull || n_shards > 1 ? td + tr : 0;
+    b += a256((size_t)Y.n_caps * sizeof(TileCap));
+    Y.rows = b;
+    if (n_shards > 1) b += a256((size_t)(2 * td + tr) * 8);
+    Y.row0 = b;
+    if (n_shards > 1) b += 256;
+    Y.lists = b;
+    if (cull) b += (size_t)total_items * 4;
+    Y.bytes = b;
+    return Y;
+}
+
 // The three counts of one w(theta) (DD, DR, RR) in one persistent launch:
 // each catalogue is prepared once, far tile pairs of each count are skipped
 // on the device, and the counts are three segments of one work table, so
@@ -3102,21 +3127,9 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
     const bool cull = (!tune || tune->skip_far != 2) && edges[K] < 180.0 && td * td < (1LL << 32) &&
                       td * tr < (1LL << 32) && tr * tr < (1LL << 32) &&
                       (total_items > 2LL * resident || n_shards > 1 || (tune && tune->skip_far == 1));
-    // scratch: cursor and kept total, segments, culling table, kept counts,
-    // both catalogues prepared together, tile caps, kept lists (and kept
-    // items per row)
-    const size_t bp = prepare_joint_bytes(nd, pd, nr, pr);
-    size_t bytes = 256 + 1024 + 1024 + 256;
-    const size_t off_prep = bytes;
-    bytes += (bp + 255) / 256 * 256;
-    const size_t off_caps = bytes;
-    if (cull) bytes += ((size_t)(td + tr) * sizeof(TileCap) + 255) / 256 * 256;
-    const size_t off_rows = bytes;
-    if (n_shards > 1) bytes += ((size_t)(2 * td + tr) * 8 + 255) / 256 * 256 + 256;
-    const size_t off_lists = bytes;
-    if (cull) bytes += (size_t)total_items * 4;
+    const WthetaLayout Y = wtheta_layout(nd, pd, nr, pr, T, cull, n_shards, total_items);
     unsigned char* m = nullptr;
-    if ((rc = dev_malloc_async((void**)&m, bytes, st))) return rc;
+    if ((rc = dev_malloc_async((void**)&m, Y.bytes, st))) return rc;
     unsigned long long* cursor = (unsigned long long*)m;  // cursor, kept count, blocks done
     unsigned long long* n_kept = cursor + 1;
     Segment* d_segs = (Segment*)(m + 256);
@@ -3130,14 +3143,14 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
     tbl.n_zero[0] = 6LL * (long long)K2;
     tbl.zero[1] = (unsigned*)cursor;
     tbl.n_zero[1] = 2 * 3;
-    prepare_zero(nd, pd, nr, pr, m + off_prep, &tbl.zero[2], &tbl.n_zero[2]);
+    prepare_zero(nd, pd, nr, pr, m + Y.prep, &tbl.zero[2], &tbl.n_zero[2]);
     if (cull) {
         tbl.zero[3] = (unsigned*)d_kept;
         tbl.n_zero[3] = 2 * 3;
     }
     tbl.with_cull = cull ? 1 : 0;
-    prepare_layout(nd, pd, nr, pr, m + off_prep, &D, &R);
-    TileCap* caps_d = (TileCap*)(m + off_caps);
+    prepare_layout(nd, pd, nr, pr, m + Y.prep, &D, &R);
+    TileCap* caps_d = (TileCap*)(m + Y.caps);
     TileCap* caps_r = caps_d + td;  // R's tiles follow D's in the joint copies
     const double theta_top = edges[K] * (3.14159265358979323846 / 180.0);
     auto cull_seg = [&](int i, long long begin) {
@@ -3155,9 +3168,9 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
         return c;
     };
     auto prepare_both = [&] {
-        int e = prepare_joint(cd, nd, pd, cr, nr, pr, is_xyz, 0, m + off_prep, di.sm_count, st, &D,
+        int e = prepare_joint(cd, nd, pd, cr, nr, pr, is_xyz, 0, m + Y.prep, di.sm_count, st, &D,
                               &R, true);
-        if (!e && (cull || n_shards > 1) && td + tr > 0)
+        if (!e && Y.n_caps > 0)
             e = launch_tile_caps(D.p32, pd + pr, (int)T, td + tr, caps_d, st);
         return e;
     };
@@ -3177,8 +3190,8 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
             row0[i] = i == 0 ? 0 : row0[i - 1] + nrow[i - 1];
             nrow[i] = cnts[i].kind == 2 ? tr : td;
         }
-        unsigned long long* d_rows = (unsigned long long*)(m + off_rows);
-        long long* d_row0 = (long long*)(m + off_rows + ((size_t)(2 * td + tr) * 8 + 255) / 256 * 256);
+        unsigned long long* d_rows = (unsigned long long*)(m + Y.rows);
+        long long* d_row0 = (long long*)(m + Y.row0);
         const long long n_rows = row0[n_segs - 1] + nrow[n_segs - 1];
         std::vector<unsigned long long> rows(n_rows);
         rc = check_cuda(cudaMemsetAsync(d_rows, 0, (size_t)n_rows * 8, st));
@@ -3223,7 +3236,7 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
         segs[i].n_items = cnts[i].items;
         segs[i].item_offset = cnts[i].offset;
         cs[i] = cull_seg(i, item);
-        cs[i].list = (unsigned*)(m + off_lists) + item;
+        cs[i].list = (unsigned*)(m + Y.lists) + item;
         item += cnts[i].items;
     }
     for (int i = 0; i < n_segs; ++i) {

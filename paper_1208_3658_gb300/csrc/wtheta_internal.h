@@ -170,6 +170,14 @@ void prepare_layout(long long na, long long pa, long long nb, long long pb, unsi
                     Prepared* A, Prepared* B);
 void prepare_zero(long long na, long long pa, long long nb, long long pb, unsigned char* scratch,
                   unsigned** words, long long* n);
+// Offsets into the scratch of a w(theta) count, its size, and the tile caps it
+// holds (0: none are computed).
+struct WthetaLayout {
+    size_t prep, caps, rows, row0, lists, bytes;
+    long long n_caps;
+};
+WthetaLayout wtheta_layout(long long nd, long long pd, long long nr, long long pr, long long T,
+                           bool cull, int n_shards, long long total_items);
 unsigned long long per_item_bound(const Variant* v);
 Segment make_segment(const Prepared& A, const Prepared& B, long long ta, long long tb,
                      int is_auto, long long item_begin, unsigned long long* counts,
