@@ -1227,7 +1227,11 @@ struct StepValues {
 // again, take back their provisional counts and add each to the row its FP64
 // recheck gives (one copy of the recheck code, in a loop over a bitmask);
 // returns the number of values rechecked.  Kept out of line: its FP64
-// registers then do not weigh on the loops that call it.
+// registers then do not weigh on the loops that call it.  Where the first value
+// lies in one edge's band, so does nearly always every other one, and FP64
+// settles them without a search in FP32 before (10k + 10k points in 36 arcsec, 16
+// bins 0.1 - 10 arcsec, 1.8e7 rechecks: 4.38 ms with it, 3.74 without; with a hint
+// for each value 3.85, and 0.5% on every other workload, in spilled registers).
 template <int NT, int R, int NV, int HM, unsigned ROWB>
 __device__ __noinline__ unsigned recount_band_values(const StepValues<NV> sv, unsigned col,
                                                      unsigned lut, int shift, int base,
@@ -1255,8 +1259,8 @@ __device__ __noinline__ unsigned recount_band_values(const StepValues<NV> sv, un
         mask &= mask - 1;
         unsigned slot = 0;
         bool sure = false;
-        if (v != hint_v || hint < 0) {
-            // perhaps a bucket with several edges: the edges searched in FP32
+        if (hint < 0) {
+            // the step met a bucket with several edges: the edges searched in FP32
             // first, and FP64 only within a guard band of the edges next to it
             slot = edges_below(s[v], sC, K);
             sure = (slot == 0u || outside_guard(s[v], sC, slot - 1u)) &&
