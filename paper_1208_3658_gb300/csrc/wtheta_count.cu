@@ -2441,6 +2441,8 @@ static void (*pair_kernel(const Variant* v, const PairParams& prm))(PairParams) 
     return prm.stats ? v->kernel : v->kernel_fast;
 }
 
+constexpr int kMaxVariants = 32;
+
 // Instantiated shapes (tile = threads x points_per_thread).  Per-warp
 // histograms (mode 2) need the whole warp in step, so they bin inline.
 const Variant* variants(int* n) {
@@ -2454,6 +2456,7 @@ const Variant* variants(int* n) {
         make_variant<64, 8, 2, kHistWarpRed, 0>(),     make_variant<32, 8, 2, kHistLaneAtomic, 0>(),
         make_variant<128, 8, 2, kHistLaneAtomic, 2>(),
     };
+    static_assert(sizeof(v) / sizeof(v[0]) <= kMaxVariants, "grid_for's table");
     *n = (int)(sizeof(v) / sizeof(v[0]));
     return v;
 }
@@ -2548,15 +2551,23 @@ const Variant* pick_variant(const wtheta_tune* tune, int K, int n_lut, int max_s
 
 int grid_for(const Variant* v, size_t smem, long long n_items, int sm_count, int want_per_sm,
                     int* grid) {
+    // The limit of a kernel's dynamic shared memory only rises: a server, a plan or
+    // another thread may launch the same kernel with the size it asked for before.
     static std::mutex mu;
+    static size_t most[64][kMaxVariants];
+    int dev = 0, nv = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return WTHETA_ECUDA;
     {
         std::lock_guard<std::mutex> g(mu);
+        size_t& kept = most[dev][v - variants(&nv)];
+        const size_t limit = std::max(kept, smem);
         if (cudaFuncSetAttribute((const void*)v->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem) != cudaSuccess ||
+                                 (int)limit) != cudaSuccess ||
             cudaFuncSetAttribute((const void*)v->kernel_fast,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem) != cudaSuccess)
+                                 (int)limit) != cudaSuccess)
             return WTHETA_ECUDA;
+        kept = limit;
     }
     int per_sm = 0;
     int per_sm_fast = 0;
