@@ -1078,10 +1078,13 @@ __device__ __forceinline__ unsigned recheck_slot(const Segment& S, long long ia,
 
 // The staged B tile: per point its three coordinates, negated and duplicated
 // for the packed FP32 arithmetic (24 B), so that two consecutive points are
-// three 16-byte loads; a chunk of 32 points takes 16 B more, so that lanes on
-// different chunks read different banks.
+// three 16-byte loads.  For span jobs a chunk of 32 points takes 16 B more, so
+// that lanes on different chunks read different banks (PAD); without them all
+// lanes read the same point, and a step's address is one addition.
 constexpr unsigned kPointB = 24, kChunkB = 32 * kPointB + 16;
+template <bool PAD>
 __device__ __forceinline__ unsigned point_addr(unsigned tile, int j) {
+    if (!PAD) return tile + (unsigned)j * kPointB;
     return tile + (unsigned)(j >> 5) * kChunkB + (unsigned)(j & 31) * kPointB;
 }
 
@@ -1110,6 +1113,10 @@ struct PairKernel {
         return (int)(threadIdx.x >> 5) * CPW + (int)(threadIdx.x & (CPW - 1));
     }
     static constexpr unsigned ROWB = 4u * HSTRIDE;
+    static constexpr bool SPANS = DEF == 0 && HM != kHistWarp;  // has span jobs
+    // Bytes of a screening-table entry in shared memory (lut_entry).
+    static constexpr unsigned LUTB = SPANS ? 8 : 16;
+    static constexpr unsigned TILEB = SPANS ? TB / 32 * kChunkB : TB * kPointB;
 
     // log2 of the most parts an item is taken in: eighths of the B tile (one unit
     // per sub-tile), or single chunks in a one-warp block.  With quarters at most,
@@ -1118,12 +1125,14 @@ struct PairKernel {
     static constexpr int MAXLP = NW == 1 ? ilog2(TB / 32) : 3;
 
     static size_t smem_bytes(int K, int n_lut) {
-        size_t b = (size_t)TB / 32 * kChunkB;   // B tile
-        b += (size_t)TB / 32 * 16;              // bounding spheres of its 32-point chunks
-        b += (size_t)TA / 8 * 16;               // bounding spheres of A's groups of 8
-        b += (size_t)n_lut * 8;                 // screening table
+        size_t b = TILEB;                       // B tile
+        b += (size_t)n_lut * LUTB;              // screening table
         b += (size_t)(K + 2) * 8;               // FP64 edges (+ pad)
-        b += (size_t)(K + 2) * 8;               // middle and half slack of every edge
+        if (SPANS) {
+            b += (size_t)TB / 32 * 16;          // bounding spheres of its 32-point chunks
+            b += (size_t)TA / 8 * 16;           // bounding spheres of A's groups of 8
+            b += (size_t)(K + 2) * 8;           // middle and half slack of every edge
+        }
         b += (size_t)(K + 2) * ROWB;            // histograms, row K+1 a trash row
         return b;
     }
@@ -1171,17 +1180,61 @@ __device__ __forceinline__ void hist_add(unsigned cell, unsigned v) {
 }
 
 // Table entry of an FP32 squared chord's bucket (bits >= 0: non-negative).
-__device__ __forceinline__ uint2 lut_entry(unsigned bits, unsigned lut, int shift, int base,
-                                           int top_idx) {
+// Builds with span jobs keep the 8 bytes of BinTable (LUTB = 8): their pairs are
+// mostly told apart by edges, and the table leaves the L1 its room.  Builds that
+// bin every pair through the table keep 16 bytes: the band's bounds and the byte
+// offsets of the rows below and above it (both the trash row in a bucket with
+// several edges, whose values are a band all over), four operations fewer per pair.
+// 200k + 200k survey points without span binning: 10.6 ms with 8 bytes and a step's
+// address by chunk, 9.2 in an earlier kernel, 9.0 with 16 bytes and point_addr<false>.
+template <unsigned LUTB>
+__device__ __forceinline__ auto lut_entry(unsigned bits, unsigned lut, int shift, int base,
+                                          int top_idx) {
     const int idx = min(max((int)(bits >> shift) - base, 0), top_idx);
-    return lds_u2(lut + 8u * (unsigned)idx);
+    if constexpr (LUTB == 8) return lds_u2(lut + 8u * (unsigned)idx);
+    else return lds_u4(lut + 16u * (unsigned)idx);
 }
-// The entry's parts: the slot below its edge, and whether bits lie below the
-// edge's band, or inside it (BinTable).
-__device__ __forceinline__ unsigned lut_slot(uint2 e) { return e.y & kLutSlot; }
+// The entry's parts: whether bits lie below the edge's band, or inside it, the
+// row they go to if not inside (provisionally, if inside, the row above), and the
+// slot below the edge (-1: several edges).
 __device__ __forceinline__ bool lut_below(uint2 e, unsigned bits) { return bits < e.x; }
-__device__ __forceinline__ bool lut_band(uint2 e, unsigned bits) {
+__device__ __forceinline__ bool lut_band(uint2 e, unsigned bits, bool) {
     return bits - e.x <= e.y >> kLutWidthShift;  // below: the difference wraps
+}
+__device__ __forceinline__ unsigned lut_slot(uint2 e) { return e.y & kLutSlot; }
+template <unsigned ROWB>
+__device__ __forceinline__ unsigned lut_row(uint2 e, bool below) {
+    return (lut_slot(e) + (below ? 0u : 1u)) * ROWB;
+}
+template <unsigned ROWB>
+__device__ __forceinline__ int lut_hint(uint2 e) {
+    return (e.y & kLutSeveral) ? -1 : (int)lut_slot(e);
+}
+__device__ __forceinline__ bool lut_below(uint4 e, unsigned bits) { return bits < e.x; }
+// (from the comparison that is made anyway: with both made here, the compiler kept
+// the entries of all of a step's values to the end, 254 registers against 174 at
+// 16 A points a thread)
+__device__ __forceinline__ bool lut_band(uint4 e, unsigned bits, bool below) {
+    return !below && bits <= e.y;
+}
+template <unsigned ROWB>
+__device__ __forceinline__ unsigned lut_row(uint4 e, bool below) {
+    return below ? e.z : e.w;
+}
+template <unsigned ROWB>
+__device__ __forceinline__ int lut_hint(uint4 e) {
+    return e.w == e.z ? -1 : (int)(e.z / ROWB);
+}
+// The 16-byte entry of BinTable's entry (x, y).
+template <unsigned ROWB>
+__device__ __forceinline__ uint4 lut_wide(unsigned x, unsigned y, int K) {
+    const unsigned slot = y & kLutSlot, row = slot * ROWB;
+    if (x == 0xFFFFFFFFu) return make_uint4(x, x, row, row + ROWB);  // no edge: all below
+    if (y & kLutSeveral) {
+        const unsigned trash = ((unsigned)K + 1u) * ROWB;
+        return make_uint4(x, x + (y >> kLutWidthShift), trash, trash);
+    }
+    return make_uint4(x, x + (y >> kLutWidthShift), row, row + ROWB);
 }
 
 // Bins NV screened values s[h R + r] (pairs of A point r and B point j + h)
@@ -1191,17 +1244,17 @@ __device__ __forceinline__ bool lut_band(uint2 e, unsigned bits) {
 // inside a band is counted, for now, in the row above it; the function returns
 // true if the step held any such value, and the caller then settles them
 // (recount_band_values).  No branch.
-template <int NV, int HM, unsigned ROWB>
+template <int NV, int HM, unsigned ROWB, unsigned LUTB>
 __device__ __forceinline__ bool bin_values(const float (&s)[NV], unsigned col, unsigned lut,
                                            int shift, int base, int top_idx) {
     bool any_band = false;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         const unsigned bits = __float_as_uint(s[v]);
-        const uint2 e = lut_entry(bits, lut, shift, base, top_idx);
+        const auto e = lut_entry<LUTB>(bits, lut, shift, base, top_idx);
         const bool below = lut_below(e, bits);
-        any_band |= lut_band(e, bits);
-        hist_add<HM>(col + (lut_slot(e) + (below ? 0u : 1u)) * ROWB, 1u);
+        any_band |= lut_band(e, bits, below);
+        hist_add<HM>(col + lut_row<ROWB>(e, below), 1u);
     }
     return any_band;
 }
@@ -1232,7 +1285,7 @@ struct StepValues {
 // settles them without a search in FP32 before (10k + 10k points in 36 arcsec, 16
 // bins 0.1 - 10 arcsec, 1.8e7 rechecks: 4.38 ms with it, 3.74 without; with a hint
 // for each value 3.85, and 0.5% on every other workload, in spilled registers).
-template <int NT, int R, int NV, int HM, unsigned ROWB>
+template <int NT, int R, int NV, int HM, unsigned ROWB, unsigned LUTB>
 __device__ __noinline__ unsigned recount_band_values(const StepValues<NV> sv, unsigned col,
                                                      unsigned lut, int shift, int base,
                                                      int top_idx, int K, const Segment& S,
@@ -1244,13 +1297,13 @@ __device__ __noinline__ unsigned recount_band_values(const StepValues<NV> sv, un
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         const unsigned bits = __float_as_uint(s[v]);
-        const uint2 e = lut_entry(bits, lut, shift, base, top_idx);
-        if (lut_band(e, bits)) {
+        const auto e = lut_entry<LUTB>(bits, lut, shift, base, top_idx);
+        if (lut_band(e, bits, lut_below(e, bits))) {
             mask |= 1u << v;
-            hist_add<HM>(col + (lut_slot(e) + 1u) * ROWB, 0xFFFFFFFFu);  // -1
+            hist_add<HM>(col + lut_row<ROWB>(e, false), 0xFFFFFFFFu);  // -1
             if (hint_v < 0) {
                 hint_v = v;
-                hint = (e.y & kLutSeveral) ? -1 : (int)lut_slot(e);
+                hint = lut_hint<ROWB>(e);
             }
         }
     }
@@ -1262,9 +1315,17 @@ __device__ __noinline__ unsigned recount_band_values(const StepValues<NV> sv, un
         if (hint < 0) {
             // the step met a bucket with several edges: the edges searched in FP32
             // first, and FP64 only within a guard band of the edges next to it
-            slot = edges_below(s[v], sC, K);
-            sure = (slot == 0u || outside_guard(s[v], sC, slot - 1u)) &&
-                   (slot > (unsigned)K || outside_guard(s[v], sC, slot));
+            float x;
+            if constexpr (LUTB == 8) {
+                x = s[v];
+            } else {
+                x = s[0];  // s[v] without an index: s stays in registers
+#pragma unroll
+                for (int w = 1; w < NV; ++w) x = v == w ? s[w] : x;
+            }
+            slot = edges_below(x, sC, K);
+            sure = (slot == 0u || outside_guard(x, sC, slot - 1u)) &&
+                   (slot > (unsigned)K || outside_guard(x, sC, slot));
         }
         if (!sure) {
             slot = recheck_slot(S, a0 + v % R, bj + v / R, sC, K, v == hint_v ? hint : -1);
@@ -1325,7 +1386,7 @@ __device__ __forceinline__ float min_of(const float (&s)[NV]) {
 
 // The FP32 steps [j0, j1) of a B tile for the thread's R A points, each pair
 // binned through the table (values inside a guard band settled in FP64).
-template <int NT, int R, int JU, int HM, unsigned ROWB, bool DIAG>
+template <int NT, int R, int JU, int HM, unsigned ROWB, bool SPANS, bool DIAG>
 __device__ __forceinline__ void exact_steps(int j0, int j1, unsigned tile, unsigned lut,
                                             unsigned sC, unsigned col, const f2_t (&ax)[R / 2],
                                             const f2_t (&ay)[R / 2], const f2_t (&az)[R / 2],
@@ -1333,18 +1394,20 @@ __device__ __forceinline__ void exact_steps(int j0, int j1, unsigned tile, unsig
                                             const Segment& S, long long a0, long long b0,
                                             int a_first, unsigned long long& n_recheck) {
     constexpr int NV = JU * R;
-    unsigned b = point_addr(tile, j0);
+    constexpr unsigned LUTB = SPANS ? 8 : 16;
+    unsigned b = point_addr<SPANS>(tile, j0);
 #pragma unroll 1
-    for (int j = j0; j < j1; b += JU * kPointB + ((j & 31) == 32 - JU ? 16u : 0u), j += JU) {
+    for (int j = j0; j < j1;
+         b += JU * kPointB + (SPANS && (j & 31) == 32 - JU ? 16u : 0u), j += JU) {
         float s[NV];
         chords<R, JU, DIAG>(s, b, ax, ay, az, j, a_first);
         const float m = min_of(s);
         if (!(m <= hf)) continue;
-        if (bin_values<NV, HM, ROWB>(s, col, lut, shift, base, top_idx)) {
+        if (bin_values<NV, HM, ROWB, LUTB>(s, col, lut, shift, base, top_idx)) {
             StepValues<NV> s2;
             chords<R, JU, DIAG>(s2.v, b, ax, ay, az, j, a_first);
-            n_recheck += recount_band_values<NT, R, NV, HM, ROWB>(s2, col, lut, shift, base,
-                                                                  top_idx, K, S, a0, b0 + j, sC);
+            n_recheck += recount_band_values<NT, R, NV, HM, ROWB, LUTB>(
+                s2, col, lut, shift, base, top_idx, K, S, a0, b0 + j, sC);
         }
     }
 }
@@ -1389,9 +1452,9 @@ __device__ __forceinline__ int span_edges(float4 ga, float4 gb, unsigned lut, un
         rlo = rhi = (unsigned)K + 1u;
         return 0;
     }
-    const uint2 el = lut_entry(bl, lut, shift, base, top_idx);
-    const uint2 eh = lut_entry(bh, lut, shift, base, top_idx);
-    rlo = lut_slot(el) + ((lut_below(el, bl) | lut_band(el, bl)) ? 0u : 1u);
+    const uint2 el = lut_entry<8>(bl, lut, shift, base, top_idx);
+    const uint2 eh = lut_entry<8>(bh, lut, shift, base, top_idx);
+    rlo = lut_slot(el) + ((lut_below(el, bl) | lut_band(el, bl, false)) ? 0u : 1u);
     rhi = lut_slot(eh) + (lut_below(eh, bh) ? 0u : 1u);
     if ((el.y | eh.y) & kLutSeveral) {
         rlo = edges_below(slo, c64, K);
@@ -1486,7 +1549,7 @@ __device__ __forceinline__ void tile_pass(unsigned tile, unsigned lut, unsigned 
     const unsigned h_top = p.tab.h_top;
     const float hf = __uint_as_float(h_top);
     const int shift = p.tab.shift, base = p.tab.base, K = p.tab.K, top_idx = p.tab.n_lut - 1;
-    constexpr unsigned ROWB = PK::ROWB;
+    constexpr unsigned ROWB = PK::ROWB, LUTB = PK::LUTB;
     const unsigned col = hist + 4u * (unsigned)PK::column();
     const long long a0 = I * TA + a_first, b0 = J * TB;
 
@@ -1494,15 +1557,15 @@ __device__ __forceinline__ void tile_pass(unsigned tile, unsigned lut, unsigned 
         // Deferred binning: the screening loop only notes, one bit per step,
         // which of 32 consecutive steps hold an in-range value; those steps
         // are then recomputed and binned.  The screening loop stays small.
-        static_assert(TB % (4 * 32 * JU) == 0, "units must hold whole 32-step blocks");
+        static_assert(DEF != 1 || TB % (8 * 32 * JU) == 0, "an eighth holds whole 32-step blocks");
 #pragma unroll 1
         for (int jb = j_begin; jb < j_end; jb += 32 * JU) {
             unsigned mask = 0;
 #pragma unroll 1
             for (int st = 0; st < 32; ++st) {
                 float s[NV];
-                chords<R, JU, DIAG>(s, point_addr(tile, jb + st * JU), ax, ay, az, jb + st * JU,
-                                    a_first);
+                chords<R, JU, DIAG>(s, point_addr<false>(tile, jb + st * JU), ax, ay, az,
+                                    jb + st * JU, a_first);
                 mask |= (min_of(s) <= hf ? 1u : 0u) << st;
             }
             while (mask) {
@@ -1510,9 +1573,9 @@ __device__ __forceinline__ void tile_pass(unsigned tile, unsigned lut, unsigned 
                 mask &= mask - 1;
                 const int j = jb + st * JU;
                 StepValues<NV> s;
-                chords<R, JU, DIAG>(s.v, point_addr(tile, j), ax, ay, az, j, a_first);
-                if (bin_values<NV, HM, ROWB>(s.v, col, lut, shift, base, top_idx))
-                    n_recheck += recount_band_values<NT, R, NV, HM, ROWB>(
+                chords<R, JU, DIAG>(s.v, point_addr<false>(tile, j), ax, ay, az, j, a_first);
+                if (bin_values<NV, HM, ROWB, LUTB>(s.v, col, lut, shift, base, top_idx))
+                    n_recheck += recount_band_values<NT, R, NV, HM, ROWB, LUTB>(
                         s, col, lut, shift, base, top_idx, K, S, a0, b0 + j, sC);
             }
         }
@@ -1521,18 +1584,18 @@ __device__ __forceinline__ void tile_pass(unsigned tile, unsigned lut, unsigned 
 #pragma unroll 1
         for (int j = j_begin; j < j_end; j += JU) {
             float s[NV];
-            chords<R, JU, DIAG>(s, point_addr(tile, j), ax, ay, az, j, a_first);
+            chords<R, JU, DIAG>(s, point_addr<false>(tile, j), ax, ay, az, j, a_first);
             const float m = min_of(s);
             if (!__any_sync(0xffffffffu, m <= hf)) continue;
             unsigned amb_mask = 0;
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
                 const unsigned bits = __float_as_uint(s[v]);
-                const uint2 e = lut_entry(bits, lut, shift, base, top_idx);
-                const bool amb = lut_band(e, bits);
+                const auto e = lut_entry<LUTB>(bits, lut, shift, base, top_idx);
+                const bool below = lut_below(e, bits), amb = lut_band(e, bits, below);
                 amb_mask |= amb ? (1u << v) : 0u;
                 const unsigned off =
-                    (amb ? (unsigned)K + 1u : lut_slot(e) + (lut_below(e, bits) ? 0u : 1u)) * ROWB;
+                    amb ? ((unsigned)K + 1u) * ROWB : lut_row<ROWB>(e, below);
                 const unsigned peers = __match_any_sync(0xffffffffu, off);
                 if (lane == __ffs(peers) - 1) red_add_shared(col + off, (unsigned)__popc(peers));
             }
@@ -1548,8 +1611,9 @@ __device__ __forceinline__ void tile_pass(unsigned tile, unsigned lut, unsigned 
     }
     // pair by pair (diagonal tiles, or span binning off; spans go through
     // span_item's jobs)
-    exact_steps<NT, R, JU, HM, ROWB, DIAG>(j_begin, j_end, tile, lut, sC, col, ax, ay, az, hf,
-                                           shift, base, top_idx, K, S, a0, b0, a_first, n_recheck);
+    exact_steps<NT, R, JU, HM, ROWB, PK::SPANS, DIAG>(j_begin, j_end, tile, lut, sC, col, ax, ay, az,
+                                                      hf, shift, base, top_idx, K, S, a0, b0,
+                                                      a_first, n_recheck);
 }
 
 // The thread's R A points, R consecutive points of the spatial order (a
@@ -1688,10 +1752,10 @@ __device__ __forceinline__ void exact_chunk(unsigned tile, int c, int t0, int ts
         float s[R];
         chords<R, 1, DIAG>(s, b, ax, ay, az, j, a_first);
         if (!(min_of(s) <= hf)) continue;
-        if (bin_values<R, HM, ROWB>(s, col, lut, shift, base, top_idx)) {
+        if (bin_values<R, HM, ROWB, 8>(s, col, lut, shift, base, top_idx)) {
             StepValues<R> s2;
             chords<R, 1, DIAG>(s2.v, b, ax, ay, az, j, a_first);
-            n_recheck += recount_band_values<NT, R, R, HM, ROWB>(
+            n_recheck += recount_band_values<NT, R, R, HM, ROWB, 8>(
                 s2, col, lut, shift, base, top_idx, p.tab.K, S, a0, b0 + t, sC);
         }
     }
@@ -2156,23 +2220,27 @@ __device__ __noinline__ void fill_overflow(const PairParams& p) {
 
 // ST: with the span path's statistics code (a launch with p.stats set); the
 // build without it is the one launched when no statistics are asked for.
+// Registers: 96 at 8 A points a thread (20 warps an SM), 168 at 16 (12 warps; left to
+// itself the compiler took 174, one block less: 16 points, deferred, 200k + 200k
+// survey points 17.9 ms against 14.7).
 template <int NT, int R, int JU, int HM, int DEF, bool ST>
-__global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __grid_constant__ PairParams p) {
+__global__ void __launch_bounds__(NT, (R == 8 ? 640 : 384) / NT) k_pairs(const __grid_constant__ PairParams p) {
     using PK = PairKernel<NT, R, JU, HM, DEF>;
     constexpr int TA = PK::TA, TB = PK::TB, HCOLS = PK::HCOLS, HSTRIDE = PK::HSTRIDE;
     constexpr int NW = NT / 32, SA = 32 * R, UPS = 8, UB = TB / UPS;
     static_assert(TA == NW * SA && TB % UPS == 0, "units tile the item");
     __shared__ unsigned s_units[2 * NW];  // units taken; chunks left per sub-tile (spans)
     // span job rings (one per kind and warp) for the shapes that bin spans
-    __shared__ unsigned s_ring[(DEF == 0 && HM != kHistWarp) ? NW * kJobKinds * kRing : 1];
+    __shared__ unsigned s_ring[PK::SPANS ? NW * kJobKinds * kRing : 1];
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = p.tab.K;
-    float4* sCap = reinterpret_cast<float4*>(smem + TB / 32 * kChunkB);
-    float4* sGroup = sCap + TB / 32;  // spheres of A's groups
-    uint2* sLut = reinterpret_cast<uint2*>(sGroup + TA / 8);
-    double* sC = reinterpret_cast<double*>(sLut + p.tab.n_lut);
+    // (the spheres and edge middles only where there are span jobs)
+    float4* sCap = reinterpret_cast<float4*>(smem + PK::TILEB);
+    float4* sGroup = sCap + (PK::SPANS ? TB / 32 : 0);  // spheres of A's groups
+    unsigned char* sLut = reinterpret_cast<unsigned char*>(sGroup + (PK::SPANS ? TA / 8 : 0));
+    double* sC = reinterpret_cast<double*>(sLut + PK::LUTB * (unsigned)p.tab.n_lut);
     float2* sBand = reinterpret_cast<float2*>(sC + (K + 2));
-    unsigned* hist = reinterpret_cast<unsigned*>(sBand + (K + 2));
+    unsigned* hist = reinterpret_cast<unsigned*>(sBand + (PK::SPANS ? K + 2 : 0));
     // the item and its tile pair (I, J), in two buffers by the parity of the
     // block's item count: thread 0 writes the next item's while other warps may
     // still be in the current one
@@ -2185,11 +2253,14 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
     // constant bank each at their own place are served one by one
     const PairParams* gp = &p;
     asm volatile("" : "+l"(gp));
-    for (int q = tid; q < p.tab.n_lut; q += NT)
-        sLut[q] = make_uint2(gp->tab.lut[q][0], gp->tab.lut[q][1]);
+    for (int q = tid; q < p.tab.n_lut; q += NT) {
+        const unsigned x = gp->tab.lut[q][0], y = gp->tab.lut[q][1];
+        if constexpr (PK::LUTB == 8) reinterpret_cast<uint2*>(sLut)[q] = make_uint2(x, y);
+        else reinterpret_cast<uint4*>(sLut)[q] = lut_wide<PK::ROWB>(x, y, K);
+    }
     for (int q = tid; q <= K; q += NT) {
         sC[q] = gp->tab.c64[q];
-        sBand[q] = make_float2(gp->tab.edge[q][0], gp->tab.edge[q][1]);
+        if constexpr (PK::SPANS) sBand[q] = make_float2(gp->tab.edge[q][0], gp->tab.edge[q][1]);
     }
     for (int q = tid; q < (K + 2) * HSTRIDE; q += NT) hist[q] = 0u;
     if (tid < 3) s_stat[tid] = 0ull;
@@ -2261,11 +2332,11 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
         // with span binning the tile holds local coordinates (relative to each
         // chunk's centre), otherwise the FP32 copies
         bool spans = false;
-        if constexpr (DEF == 0 && HM != kHistWarp) spans = p.span && S.b_caps;
+        if constexpr (PK::SPANS) spans = p.span && S.b_caps;
         const unsigned a_tile = smem_addr(smem);
         // two points at a time: three 16-byte stores
         auto stage2 = [&](int j, float x0, float y0, float z0, float x1, float y1, float z1) {
-            const unsigned b = point_addr(a_tile, j);
+            const unsigned b = point_addr<PK::SPANS>(a_tile, j);
             sts_f2x2(b, pack2(-x0, -x0), pack2(-y0, -y0));
             sts_f2x2(b + 16u, pack2(-z0, -z0), pack2(-x1, -x1));
             sts_f2x2(b + 32u, pack2(-y1, -y1), pack2(-z1, -z1));
@@ -2291,7 +2362,7 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
             }
         }
         if (tid < NW) s_units[tid] = NW == 1 ? 0 : (part * UPS) >> lp;
-        if constexpr (DEF == 0 && HM != kHistWarp) {
+        if constexpr (PK::SPANS) {
             if (spans)
                 settle_chunks<NT, R, JU, HM, ST>(smem_addr(s_units + NW), smem_addr(sLut),
                                                  smem_addr(sC), smem_addr(hist), p, S, I, J,
@@ -2303,13 +2374,13 @@ __global__ void __launch_bounds__(NT, R == 8 ? 640 / NT : 1) k_pairs(const __gri
         // The item is split into units of one warp's worth of A points (SA =
         // 32 R consecutive points, a sub-tile) by an eighth of the B tile (the
         // warps of a block end an item within less of one another than with
-        // quarters: survey 33.3 -> 32.9 ms).  A
-        // warp takes the units of its own sub-tile first, then those left of
-        // the others, so the warps of the block finish the item together
-        // whatever the mix of cheap and costly units.
+        // quarters: survey 33.3 -> 32.9 ms, 200k + 200k binned after screening
+        // 15.3 -> 12.3 ms).  A warp takes the units of its own sub-tile first, then
+        // those left of the others, so the warps of the block finish the item
+        // together whatever the mix of cheap and costly units.
         const int lane = tid & 31, warp = tid >> 5;
         const bool diag = S.is_auto && I == J;
-        if constexpr (DEF == 0 && HM != kHistWarp) {
+        if constexpr (PK::SPANS) {
             if (spans)
                 span_item<NT, R, JU, HM, ST>(smem_addr(s_units), smem_addr(s_ring),
                                          smem_addr(s_IJ[n_items & 1]), a_tile, a_lut, a_cap, a_group, a_band, a_c,
@@ -2430,7 +2501,7 @@ __global__ void k_finalize_segments(const Segment* __restrict__ segs, int n_segs
 // ---------------------------------------------------------------------------
 template <int NT, int R, int JU, int HM, int DEF>
 static Variant make_variant() {
-    constexpr bool spans = DEF == 0 && HM != kHistWarp;  // only the span path has ST code
+    constexpr bool spans = PairKernel<NT, R, JU, HM, DEF>::SPANS;  // only the span path has ST code
     return Variant{NT, R, JU, HM, DEF, PairKernel<NT, R, JU, HM, DEF>::MAXLP, &k_pairs<NT, R, JU, HM, DEF, true>,
                    spans ? &k_pairs<NT, R, JU, HM, DEF, false> : &k_pairs<NT, R, JU, HM, DEF, true>,
                    &PairKernel<NT, R, JU, HM, DEF>::smem_bytes};
@@ -2455,7 +2526,8 @@ const Variant* variants(int* n) {
         make_variant<64, 8, 2, kHistLaneAtomic, 0>(),  make_variant<128, 8, 2, kHistWarpRed, 0>(),
         make_variant<64, 8, 2, kHistWarpRed, 0>(),     make_variant<32, 8, 2, kHistLaneAtomic, 0>(),
         make_variant<128, 8, 2, kHistLaneAtomic, 2>(), make_variant<64, 8, 2, kHistLaneAtomic, 2>(),
-        make_variant<32, 8, 2, kHistLaneAtomic, 2>(),
+        make_variant<32, 8, 2, kHistLaneAtomic, 2>(), make_variant<128, 8, 2, kHistWarpRed, 2>(),
+        make_variant<64, 8, 2, kHistWarpRed, 2>(),
     };
     static_assert(sizeof(v) / sizeof(v[0]) <= kMaxVariants, "grid_for's table");
     *n = (int)(sizeof(v) / sizeof(v[0]));
@@ -2518,13 +2590,15 @@ const Variant* pick_variant(const wtheta_tune* tune, int K, int n_lut, int max_s
             if (shape(v[i]) && v[i].hm == hm && v[i].def == def && fits(v[i])) return &v[i];
         return nullptr;
     };
-    // every pair through the table (span binning off): the build whose threads
-    // have a column each, without span code (four columns per warp contend: 100k x
-    // 100k points, 16 bins, hist_mode 3: 4.53 ms against 4.46)
-    if ((want_hm == 0 || want_hm == kHistLaneAtomic) && want_def != 1 && tune &&
-        tune->span_bins == 2) {
-        const Variant* x = find(kHistLaneAtomic, 2);
+    // every pair through the table (span binning off): the builds without span
+    // code, with a column per thread (four per warp contend: 100k x 100k points, 16
+    // bins, hist_mode 3: 4.53 ms against 4.46) or per warp
+    const bool no_spans = tune && tune->span_bins == 2 && want_def != 1;
+    if (no_spans) {
+        const Variant* x = find(want_hm == 0 ? (int)kHistLaneAtomic : want_hm, 2);
         if (x && (want_hm != 0 || x->smem(K, n_lut) <= 100 * 1024)) return x;
+        x = want_hm == 0 ? find(kHistWarpRed, 2) : nullptr;
+        if (x) return x;
     }
     if (want_hm == 0) {
         want_hm = find(kHistWarpRed, 0) ? kHistWarpRed : kHistWarp;

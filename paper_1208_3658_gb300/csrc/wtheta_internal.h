@@ -31,9 +31,10 @@ constexpr int kMaxLut = 1024;      // entries of the FP32 screening table
 //   - every band's upper bound is at most h_top, so a value beyond h_top is
 //     never taken for a band value.
 // 8 bytes an entry: the lookups' lanes go to unrelated entries, so their bank
-// conflicts grow with the entry's size.
+// conflicts grow with the entry's size (builds that bin every pair through the
+// table widen the entries to 16 bytes, lut_wide).
 constexpr uint32_t kLutSlot = 511u, kLutSeveral = 512u;
-constexpr int kLutWidthShift = 10, kMaxLutShift = 22;  // a band's width in a bucket < 2^22
+constexpr int kLutWidthShift = 10, kMaxLutShift = 22;  // a width is < 2^22
 struct BinTable {
     int32_t K;
     uint32_t h_top;        // FP32 bits of the top edge's upper guard bound
