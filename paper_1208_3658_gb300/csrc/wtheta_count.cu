@@ -2898,20 +2898,43 @@ int launch_gather_regions(const double* x64, long long stride, const unsigned* o
 }
 
 size_t regions_bytes(long long n_pad) {
-    return a256((size_t)n_pad * 16) + sphere_bytes(n_pad) + a256(local_bytes(n_pad));
+    return a256((size_t)n_pad * 16) + a256((size_t)n_pad / 32 * 16);
+}
+size_t regions_group_bytes(long long n_pad) { return a256((size_t)n_pad / 8 * 16); }
+size_t regions_sort_bytes(long long n, long long n_pad) {
+    return std::max(a256(order_bytes(n, 1)), 2 * a256((size_t)n * 4) + a256(local_bytes(n_pad)));
 }
 
-Prepared regions_layout(unsigned char* p, long long n_pad) {
+Prepared regions_layout(unsigned char* p, unsigned char* groups, unsigned char* sort, long long n,
+                        long long n_pad) {
     Prepared q;
     q.p32 = (const float4*)p;
-    p += a256((size_t)n_pad * 16);
-    q.c32 = (const float4*)p;
-    q.groups = (const float4*)(p + a256((size_t)n_pad / 32 * 16));
-    p += sphere_bytes(n_pad);
-    q.l32 = (const float*)p;
+    q.c32 = (const float4*)(p + a256((size_t)n_pad * 16));
+    q.groups = (const float4*)groups;
+    unsigned char* local = sort + 2 * a256((size_t)n * 4);  // past both index buffers
+    q.l32 = (const float*)local;
     q.l_stride = n_pad;
-    q.kap = (const float2*)(p + a256((size_t)n_pad * 12));
+    q.kap = (const float2*)(local + a256((size_t)n_pad * 12));
     return q;
+}
+
+PlanLayout plan_scratch(int n_cats2, long long n, long long n_pad) {
+    PlanLayout Y;
+    size_t b = 256;  // the cursor
+    Y.cats = b;
+    b += a256((size_t)n_cats2 * sizeof(BatchCat));
+    Y.offs = b;
+    b += a256((size_t)2 * (n_cats2 + 1) * 8);
+    Y.x = b;
+    b += a256((size_t)n * 24);
+    Y.lab = b;  // the labels; once sorted, the groups' spheres
+    b += std::max(a256((size_t)n * 4), regions_group_bytes(n_pad));
+    Y.sort = b;
+    b += regions_sort_bytes(n, n_pad);
+    Y.all = b;
+    b += regions_bytes(n_pad);
+    Y.bytes = b;
+    return Y;
 }
 
 Prepared tile_view(const Prepared& A, long long pos) {
@@ -3654,34 +3677,19 @@ static int plan_layout(wtheta_plan* P, const Variant* v, int sm_count, cudaStrea
     P->n_all = P->src_off[nc2];
     P->n_all_pad = P->dst_off[nc2];
     const long long N = P->n_all, NP = P->n_all_pad;
-    // scratch: the cursor head, the catalogue table and offsets, the FP64
-    // array and labels, the sort, the FP32 copies, chunk spheres and local
-    // coordinates
-    size_t bytes = 256;
-    const size_t off_cats = bytes;
-    bytes += a256((size_t)nc2 * sizeof(BatchCat));
-    const size_t off_offs = bytes;
-    bytes += a256((size_t)2 * (nc2 + 1) * 8);
-    const size_t off_x = bytes;
-    bytes += a256((size_t)N * 24);
-    const size_t off_lab = bytes;
-    bytes += a256((size_t)N * 4);
-    const size_t off_sort = bytes;
-    bytes += a256(order_bytes(N, 1));
-    const size_t off_all = bytes;
-    bytes += regions_bytes(NP);
+    const PlanLayout Y = plan_scratch(nc2, N, NP);
     if (P->scratch) cudaFree(P->scratch);
     P->scratch = nullptr;
-    int rc = dev_malloc(&P->scratch, bytes);
+    int rc = dev_malloc(&P->scratch, Y.bytes);
     if (rc) return rc;
     unsigned char* base = (unsigned char*)P->scratch;
     P->d_cursor = (unsigned long long*)base;
-    P->d_cats = (BatchCat*)(base + off_cats);
-    P->d_src_off = (long long*)(base + off_offs);
-    P->x_all = (double*)(base + off_x);
-    P->lab_all = (int*)(base + off_lab);
-    P->sort_scratch = base + off_sort;
-    P->all = regions_layout(base + off_all, NP);
+    P->d_cats = (BatchCat*)(base + Y.cats);
+    P->d_src_off = (long long*)(base + Y.offs);
+    P->x_all = (double*)(base + Y.x);
+    P->lab_all = (int*)(base + Y.lab);
+    P->sort_scratch = base + Y.sort;
+    P->all = regions_layout(base + Y.all, base + Y.lab, base + Y.sort, N, NP);
     P->all.x64 = P->x_all;
     P->all.stride = N;
     std::vector<long long> offs(P->src_off);

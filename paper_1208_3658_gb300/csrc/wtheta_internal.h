@@ -208,11 +208,25 @@ int launch_count_labels(const unsigned* lab, long long n, int n_labels,
 int launch_gather_regions(const double* x64, long long stride, const unsigned* order,
                           const long long* src, const long long* dst, int R, long long n_pad,
                           int tag, int sm_count, cudaStream_t st, const Prepared& out);
-// The memory those copies take and their layout in it; the copies from
-// position pos (a multiple of the tile) on.
+// The memory those copies take: FP32 points and chunk spheres (regions_bytes, at
+// p), groups' spheres (regions_group_bytes, at groups), and the local coordinates
+// with kappa and slack in the sort's scratch, whose keys, labels and digit counts
+// are no longer read once the order is known (regions_sort_bytes, at sort: the sort's
+// own scratch and the room for them).  Then the copies from position pos (a multiple
+// of the tile) on.
 size_t regions_bytes(long long n_pad);
-Prepared regions_layout(unsigned char* p, long long n_pad);
+size_t regions_group_bytes(long long n_pad);
+size_t regions_sort_bytes(long long n, long long n_pad);
+Prepared regions_layout(unsigned char* p, unsigned char* groups, unsigned char* sort, long long n,
+                        long long n_pad);
 Prepared tile_view(const Prepared& A, long long pos);
+// Offsets into a batch plan's scratch (n_cats2 catalogues of n points in all, n_pad
+// padded) and its size: catalogue table, offsets, FP64 points, labels (later the
+// groups' spheres), the sort (later the local coordinates), FP32 copies.
+struct PlanLayout {
+    size_t cats, offs, x, lab, sort, all, bytes;
+};
+PlanLayout plan_scratch(int n_cats2, long long n, long long n_pad);
 // Skipping over a table of counts: kept items per count, then each count's
 // kept range and list written into segs, their number into *n_kept.
 int launch_cull_batch(const CullSeg* cs, int n_segs, long long total, double theta_top,

@@ -78,7 +78,9 @@ int count_regions_impl(const double* cd, long long nd, const int* ld, const doub
         off_x[c] = b1;
         if (!is_xyz) b1 += ((size_t)n_of[c] * 24 + 255) / 256 * 256;
         off_sort[c] = b1;
-        b1 += order_bytes(n_of[c], 1);
+        // (the local coordinates follow the sort there; every region's last tile may
+        // hold padding)
+        b1 += regions_sort_bytes(n_of[c], round_up(n_of[c] + R * T, T));
     }
     unsigned char* m1 = nullptr;
     if ((rc = dev_malloc_async((void**)&m1, b1, st))) return rc;
@@ -151,7 +153,7 @@ int count_regions_impl(const double* cd, long long nd, const int* ld, const doub
     for (int c = 0; c < 2; ++c) {
         const long long np = L[c].dst[R];
         off_copies[c] = b2;
-        b2 += regions_bytes(np);
+        b2 += regions_bytes(np) + regions_group_bytes(np);
         off_tc[c] = b2;
         b2 += ((size_t)(np / T) * sizeof(TileCap) + 255) / 256 * 256;
     }
@@ -179,7 +181,8 @@ int count_regions_impl(const double* cd, long long nd, const int* ld, const doub
     TileCap* tcaps[2];
     for (int c = 0; c < 2 && !rc; ++c) {
         const long long np = L[c].dst[R];
-        P[c] = regions_layout(m2 + off_copies[c], np);
+        unsigned char* copies = m2 + off_copies[c];
+        P[c] = regions_layout(copies, copies + regions_bytes(np), m1 + off_sort[c], n_of[c], np);
         P[c].x64 = x64[c];
         P[c].stride = n_of[c];
         tcaps[c] = (TileCap*)(m2 + off_tc[c]);
