@@ -1,13 +1,13 @@
 // Shared-memory atomic throughput of this GPU, for the second roofline of the
 // pair kernel: its histogram updates are `red.shared.add.u32`, one per pair
-// binned through the table (to the thread's own column) and a few per chunk
+// binned through the table and a few per chunk
 // settled by span.  One block of 1024 threads per SM (its shared memory
 // request keeps a second block off the SM) issues a fixed number of
 // reductions, either each thread to its own word (distinct banks within a
 // warp) or every thread to one word; the SM clock counter times the block.
 #include <cuda_runtime.h>
 
-#include <cmath>
+#include <algorithm>
 
 #include "wtheta_internal.h"
 
@@ -16,6 +16,10 @@ namespace {
 constexpr int kThreads = 1024;
 constexpr int kIters = 4096;
 constexpr int kSmem = 160 * 1024;  // more than half an SM's shared memory
+// Launches, of which the fastest counts: a launch's mean takes one of a few values
+// some 10^-6 apart, at random; the fastest of 32 is the same every time (and the
+// same for both address patterns).
+constexpr int kLaunches = 32;
 
 __global__ void __launch_bounds__(kThreads) k_shared_atomics(int same_address,
                                                              unsigned long long* cycles,
@@ -48,23 +52,22 @@ extern "C" int wtheta_probe_shared_atomics(int32_t same_address, double* per_sm_
              k_shared_atomics, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem))))
         return rc;
     if ((rc = wtheta::check_cuda(cudaMalloc(&d, 16)))) return rc;
-    rc = wtheta::check_cuda(cudaMemset(d, 0, 16));
-    for (int rep = 0; rep < 2 && !rc; ++rep) {  // the first launch warms up
-        if (!rc) rc = wtheta::check_cuda(cudaMemset(d, 0, 16));
+    unsigned long long best = ~0ull;
+    for (int rep = 0; rep < kLaunches && !rc; ++rep) {
+        if ((rc = wtheta::check_cuda(cudaMemset(d, 0, 16)))) break;
         k_shared_atomics<<<di.sm_count, kThreads, kSmem>>>(same_address, d, (unsigned*)(d + 1));
         wtheta::add_launches(1);
         if (!rc) rc = wtheta::check_cuda(cudaGetLastError());
         if (!rc) rc = wtheta::check_cuda(cudaDeviceSynchronize());
+        unsigned long long cyc = 0;
+        if (!rc) rc = wtheta::check_cuda(cudaMemcpy(&cyc, d, 8, cudaMemcpyDeviceToHost));
+        best = std::min(best, cyc);
     }
-    unsigned long long cyc = 0;
-    if (!rc) rc = wtheta::check_cuda(cudaMemcpy(&cyc, d, 8, cudaMemcpyDeviceToHost));
     cudaFree(d);
     if (rc) return rc;
     // warp-wide reductions per SM per clock, averaged over the blocks (one per SM)
     const double warps = kThreads / 32.0;
-    const double mean_cycles = (double)cyc / (double)di.sm_count;
-    // to three decimals: the block's start and end cost some 10^-5 of its cycles,
-    // differently from launch to launch
-    *per_sm_per_clock = std::round(1000.0 * warps * kIters / mean_cycles) / 1000.0;
+    const double mean_cycles = (double)best / (double)di.sm_count;
+    *per_sm_per_clock = warps * kIters / mean_cycles;
     return WTHETA_OK;
 }
