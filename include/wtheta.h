@@ -169,7 +169,7 @@ int wtheta_shard_weights(const uint64_t* weights, int64_t n_rows, int32_t shard,
 
 /* Tuning knobs of the counting kernel; zero fields mean "choose". */
 typedef struct wtheta_tune {
-    int32_t threads;           /* threads per block: 64, 128 or 256           */
+    int32_t threads;           /* threads per block: 32, 64, 128 or 256       */
     int32_t points_per_thread; /* A points held in registers per thread: 8 or 16 */
     int32_t hist_mode;         /* 1: private per-thread histograms, plain add;
                                   2: per-warp histograms, warp-aggregated atomics;

@@ -149,11 +149,6 @@ __device__ __forceinline__ void sts_u32_if(bool p, unsigned a, unsigned v) {
 __device__ __forceinline__ void red_add_shared(unsigned a, unsigned v) {
     asm volatile("red.shared.add.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
 }
-__device__ __forceinline__ void inc_shared(unsigned a) {
-    unsigned c;
-    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(c) : "r"(a) : "memory");
-    asm volatile("st.shared.b32 [%0], %1;" :: "r"(a), "r"(c + 1u) : "memory");
-}
 
 // ---------------------------------------------------------------------------
 // conversion kernels
@@ -403,8 +398,9 @@ __global__ void __launch_bounds__(kSortThreads) k_digit_scatter(
 // a block, warps in order and lanes in order.
 //
 // Bound by the latency of a launch and of about six dependent memory accesses:
-// a w(theta) of 1k + 1k points takes 96 us instead of 117 with three launches a
-// pass, one of 10k + 10k 271 us instead of 300 (with the host copies).
+// a w(theta) of 1k + 1k points took 96 us instead of 117 with three launches a
+// pass, one of 10k + 10k 271 us instead of 300 (with the host copies), in the build
+// that it came with (77 and 227 us now).
 constexpr int kSmallThreads = 1024;
 constexpr long long kSmallSort = 65536;
 __global__ void __launch_bounds__(kSmallThreads) k_small_pass(
@@ -786,9 +782,10 @@ __global__ void k_finalize(unsigned long long* counts, int K, unsigned long long
 // kHistLane: one private uint32 column per thread, plain read-modify-write;
 // kHistWarp: one column per warp, lanes with equal slots merged by
 //            __match_any_sync and added by one shared atomic;
-// kHistLaneAtomic: one private column per thread, updated by a shared atomic
-//            add (one instruction instead of load, add, store).
-
+// kHistLaneAtomic: updated by a shared atomic add (one instruction instead of
+//            load, add, store): four columns per warp in builds with span jobs,
+//            one per thread in those without;
+// kHistWarpRed: one column per warp, shared atomic add.
 
 // Tile-pair index -> (I, J).  Auto: upper triangle I <= J, row-major.
 __device__ __forceinline__ void item_to_tiles(long long t, long long T_a, long long T_b,
@@ -1046,10 +1043,8 @@ __device__ __forceinline__ unsigned edges_below(double x, unsigned c64, int K) {
     return lo;
 }
 
-// FP64 recheck: the definition's squared chord and slot for the pair of
-// sorted positions (ia, jb), read from the FP64 arrays through the original
-// indices kept in the FP32 copies; c64 is the shared address of the FP64 edges.  hint >= 0: the slot just below the one edge whose guard
-// band held the FP32 value (checked, else the edges are searched in order).
+// The definition's squared chord, in FP64, of the pair of sorted positions (ia, jb),
+// read from the FP64 arrays through the original indices kept in the FP32 copies.
 __device__ __forceinline__ double pair_chord2(const Segment& S, long long ia, long long jb) {
     const long long i = __float_as_int(S.a32[ia].w), j = __float_as_int(S.b32[jb].w);
     const double* a = S.a64;
@@ -1061,6 +1056,9 @@ __device__ __forceinline__ double pair_chord2(const Segment& S, long long ia, lo
     return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
+// FP64 recheck: the slot of that squared chord; c64 is the shared address of the
+// FP64 edges.  hint >= 0: the slot just below the one edge whose guard band held the
+// FP32 value (checked, else the edges are searched).
 __device__ __forceinline__ unsigned recheck_slot(const Segment& S, long long ia, long long jb,
                                                  unsigned c64, int K, int hint = -1) {
     const double s = pair_chord2(S, ia, jb);
@@ -1425,16 +1423,22 @@ __device__ __forceinline__ void exact_steps(int j0, int j1, unsigned tile, unsig
 //   0        every pair is in slot rlo (a span wholly above h_top, the top
 //            edge's band, is the overflow slot K + 1 at once);
 //   1 .. kMaxEdges  the counts of the slots follow from the number of pairs
-//            below each of those edges;
-//            (up to kMaxEdgesFar beyond 60 degrees, where guard bands are
-//            widest and the table's buckets hold several edges, whose pairs
-//            would be searched one by one);
+//            below each of those edges (up to kMaxEdgesFar if the span reaches
+//            beyond 60 degrees);
 //   -1       more edges, or padding: bin pair by pair.
 // Two edges cost a job about a quarter of the table's lookups and shared
-// atomics for its 256 pairs.  The lines, one build, kMaxEdges 4, 6, 8: 256 bins
-// (200k + 200k points) 8.70, 8.91, 9.39 ms; 24 bins (30k x 48k) 513, 509, 517
-// us; 32 bins (1M + 1M) 36.67, 36.72, 36.81 ms; 36 linear bins to 180 deg (100k +
-// 100k) 14.3, 13.6, 10.0 ms, and 10.0 with 6 and the line for far spans.
+// atomics for its 256 pairs.  kMaxEdges 4, 6, 8 in the build that it came with: 256
+// log bins to 20 deg (200k + 200k points) 8.70, 8.91, 9.39 ms; 24 bins (30k x 48k)
+// 513, 509, 517 us; 32 bins (1M + 1M) 36.67, 36.72, 36.81 ms.
+// Beyond 60 degrees the line is 16, because values in a bucket with several edges
+// are recounted out of line, one by one, and linear bins have such buckets there
+// (the table's buckets are steps of the logarithm).  The span's ends do not tell:
+// 36 linear bins have only one, just below 180 deg, and the spans across it end in
+// the next.  Now, 6 everywhere / a line of 16 where an end meets such a bucket / this
+// / 16 everywhere, full sky: 36 bins (100k + 100k) 12.8, 12.7, 8.7, 8.7 ms (4.7e7
+// values recounted with 6, 1.1e6 with this), 256 bins (100k + 100k) 203, 166, 134,
+// 135, 90 bins (300k + 300k) 182, 162, 113, 113, 20 bins from 60 deg 6.4, 6.4, 6.6,
+// 6.6; the 256 log bins to 20 deg 8.3, 8.3, 8.3, 9.9.
 constexpr int kMaxEdges = 6, kMaxEdgesFar = 16;
 __device__ __forceinline__ int span_edges(float4 ga, float4 gb, unsigned lut, unsigned c64,
                                           int shift, int base, int top_idx, int K, unsigned h_top,
@@ -1617,7 +1621,7 @@ __device__ __forceinline__ void tile_pass(unsigned tile, unsigned lut, unsigned 
 }
 
 // The thread's R A points, R consecutive points of the spatial order (a
-// compact group: see span_class), packed two by two for the FP32x2
+// compact group: see write_chunk), packed two by two for the FP32x2
 // instructions.  Each value goes through an explicit add of +0 (exact; it
 // only turns -0 into +0, which leaves every squared chord unchanged): the
 // packed operands then get registers of their own instead of being formed in
@@ -2559,8 +2563,20 @@ int device_info(DeviceInfo* out) {
 
 // The default shape for one call by the larger catalogue's size: tiles of 256
 // points (one warp) up to 4096, of 512 points (64 threads) up to 32768, else of
-// 1024.  w(theta) with 32, 64, 128 threads: 1k + 1k points 96, 121, 148 us; 10k +
-// 10k 262, 246, 254 us (host copies included); cross 30k x 48k - , 443, 431 us.
+// 1024.  w(theta) of n + n points on a 10 deg patch (16 bins) / a 15 deg patch (24) /
+// a 60 deg cap (32), with 32, 64, 128 threads, us per call on the device:
+//    1k  106 113 135 / 111 118 133 / 104 110 128
+//    4k  118 125 145 / 125 125 147 / 116 125 138
+//    6k  138 138 144 / 152 147 152 / 135 133 142
+//    8k  163 152 155 / 181 162 174 / 151 143 150
+//   16k  262 246 249 / 300 279 288 / 221 213 218
+//   32k  455 461 486 / 578 569 609 / 340 345 379
+//   48k  751 724 728 / 996 935 940 / 489 496 517
+//   64k 1090 1015 1024 / 1476 1357 1368 / 657 636 669
+// and cross counts n x n: 4k 104 117 138 / 109 115 138 / 105 110 134, 32k 318 327 327 /
+// 388 381 374 / 237 240 264, 48k 491 508 505 / 617 628 615 / 340 347 362.  So 32
+// threads up to about 5k; from there 64, clearly up to 32k; at 48k and 64k the last
+// two lie within 2% on the patches (64 ahead by 4% on the cap).
 const Variant* pick_for_size(const wtheta_tune* tune, long long n_max, int K, int n_lut,
                              int max_smem) {
     if (!tune && n_max <= 32768) {

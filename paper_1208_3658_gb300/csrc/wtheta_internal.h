@@ -50,10 +50,10 @@ struct BinTable {
 
 // Private histogram columns of the pair kernel: per thread, plain
 // read-modify-write (1); per warp, lanes merged by __match_any_sync (2); per
-// thread, or four per warp with span jobs, shared reduction (3); per warp, shared reduction (4: the shared
-// atomic unit merges lanes that hit one word at full rate, and the rows of a
-// warp's column sit an odd number of words apart so that different rows hit
-// different banks).
+// thread, or four per warp with span jobs, shared reduction (3); per warp, shared
+// reduction (4: the shared atomic unit merges lanes that hit one word at full
+// rate, and the rows of a warp's column sit an odd number of words apart so that
+// different rows hit different banks).
 enum HistMode { kHistLane = 1, kHistWarp = 2, kHistLaneAtomic = 3, kHistWarpRed = 4 };
 
 // One count: catalogue a against catalogue b (auto: a = b, pairs i < j).
@@ -155,10 +155,10 @@ long long round_up(long long x, long long m);
 int check_cuda(cudaError_t e);
 // The one or two catalogues of a count prepared together (b absent: nb = pb
 // = 0): one conversion and key launch, one sort of the na + nb points, one
-// gather into FP32 and FP64 copies, chunk spheres and local coordinates with
-// a's points at [0, pa) and b's at [pa, pa + pb) (each catalogue tile-padded
-// with sentinels of tags tag0 and tag0 + 1: catalogues that a count may pair
-// need different tags).  scratch: prepare_joint_bytes(na, pa, nb, pb); a and b
+// gather into FP32 copies, spheres and local coordinates (the FP64 points stay in
+// input order) with a's points at [0, pa) and b's at [pa, pa + pb) (each catalogue
+// tile-padded with sentinels of tags tag0 and tag0 + 1: catalogues that a count may
+// pair need different tags).  scratch: prepare_joint_bytes(na, pa, nb, pb); a and b
 // may lie in its first 16 (na + nb) bytes (the FP32 copies, written after both
 // are read).
 size_t prepare_joint_bytes(long long na, long long pa, long long nb, long long pb);
