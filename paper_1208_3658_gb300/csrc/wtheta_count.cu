@@ -2633,11 +2633,11 @@ const Variant* pick_variant(const wtheta_tune* tune, int K, int n_lut, int max_s
     if (want_def < 0) want_def = 0;  // inline binning measured faster once in-range pairs matter
     for (int i = 0; i < nv; ++i)
         if (shape(v[i]) && v[i].hm == want_hm && v[i].def == want_def && fits(v[i])) return &v[i];
-    // fall back: same tile size, per-warp histograms (with span jobs first)
+    // fall back: same tile size, per-warp histograms (shared atomics first)
     for (int hm : {(int)kHistWarpRed, (int)kHistWarp})
         for (int i = 0; i < nv; ++i)
-            if (v[i].nt * v[i].r == want_nt * want_r && v[i].hm == hm && v[i].def == 0 &&
-                fits(v[i]))
+            if (v[i].nt * v[i].r == want_nt * want_r && v[i].hm == hm &&
+                v[i].def == (no_spans && hm == kHistWarpRed ? 2 : 0) && fits(v[i]))
                 return &v[i];
     return nullptr;
 }

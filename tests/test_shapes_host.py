@@ -30,11 +30,12 @@ def test_no_spans_means_a_column_per_thread(tmp_path, threads, hist_mode, deferr
 
 
 def test_other_requests_without_spans(tmp_path):
-    deferred, warp, red = (run(tmp_path, BODY, [128, h, d, 2, 24])[0]
-                           for h, d in ((3, 2), (2, 0), (4, 0)))
+    deferred, warp, red, plain = (run(tmp_path, BODY, [128, h, d, 2, 24])[0]
+                                  for h, d in ((3, 2), (2, 0), (4, 0), (1, 0)))
     assert deferred[:4] == ["128", "8", "3", "1"]
     assert warp[:4] == ["128", "8", "2", "0"]
     assert red[:4] == ["128", "8", "4", "2"]
+    assert plain[:4] == ["128", "8", "4", "2"]   # (mode 1 is built deferred only)
     # 256 bins: a column per thread only if it is asked for
     (chosen,), (asked,) = (run(tmp_path, BODY, [128, h, 0, 2, 256]) for h in (0, 3))
     assert chosen[2:4] == ["4", "2"] and asked[2:4] == ["3", "2"]
