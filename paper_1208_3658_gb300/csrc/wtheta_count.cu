@@ -2609,8 +2609,8 @@ const Variant* pick_variant(const wtheta_tune* tune, int K, int n_lut, int max_s
     // every pair through the table (span binning off): the builds without span
     // code, with a column per thread (four per warp contend: 100k x 100k points, 16
     // bins, hist_mode 3: 4.53 ms against 4.46) or per warp
-    const bool no_spans = tune && tune->span_bins == 2 && want_def != 1;
-    if (no_spans) {
+    const bool no_spans = tune && tune->span_bins == 2;
+    if (no_spans && want_def != 1) {
         const Variant* x = find(want_hm == 0 ? (int)kHistLaneAtomic : want_hm, 2);
         if (x && (want_hm != 0 || x->smem(K, n_lut) <= 100 * 1024)) return x;
         x = want_hm == 0 ? find(kHistWarpRed, 2) : nullptr;

@@ -29,6 +29,29 @@ def test_no_spans_means_a_column_per_thread(tmp_path, threads, hist_mode, deferr
     assert again == no
 
 
+def test_no_request_without_spans_gets_span_code(tmp_path):
+    """Every combination of the tuning's fields: what is refused is refused with and
+    without spans alike, and without them the build has no span jobs (deferred 0
+    with hist_mode 3 or 4 is a span build)."""
+    out = run(tmp_path, """
+    for (int K : {1, 24, 100, 256}) for (int n_lut : {20, 1000}) for (int t : {0, 32, 64, 128, 256, 512})
+    for (int r : {0, 8, 16}) for (int h = 0; h <= 4; ++h) for (int j = 0; j <= 2; ++j)
+    for (int d = 0; d <= 2; ++d) {
+        wtheta_tune u = {};
+        u.threads = t; u.points_per_thread = r; u.hist_mode = h; u.j_per_screen = j; u.deferred = d;
+        u.span_bins = 2;
+        const Variant* no = pick_variant(&u, K, n_lut, 232448);
+        u.span_bins = 1;
+        const Variant* yes = pick_variant(&u, K, n_lut, 232448);
+        const bool spans = no && no->def == 0 && no->hm != kHistWarp;
+        printf("%d %d %d %d %d\\n", !no == !yes, spans, no ? no->nt * no->r : 0,
+               yes ? yes->nt * yes->r : 0, no && no->smem(K, n_lut) > 232448);
+    }""")
+    assert len(out) == 4 * 2 * 6 * 3 * 5 * 3 * 3
+    for same, spans, tile, tile_yes, too_big in out:
+        assert same == "1" and spans == "0" and tile == tile_yes and too_big == "0"
+
+
 def test_other_requests_without_spans(tmp_path):
     deferred, warp, red, plain = (run(tmp_path, BODY, [128, h, d, 2, 24])[0]
                                   for h, d in ((3, 2), (2, 0), (4, 0), (1, 0)))
