@@ -1384,7 +1384,7 @@ __device__ __forceinline__ float min_of(const float (&s)[NV]) {
 
 // The FP32 steps [j0, j1) of a B tile for the thread's R A points, each pair
 // binned through the table (values inside a guard band settled in FP64).
-template <int NT, int R, int JU, int HM, unsigned ROWB, bool SPANS, bool DIAG>
+template <int NT, int R, int JU, int HM, unsigned ROWB, bool DIAG>
 __device__ __forceinline__ void exact_steps(int j0, int j1, unsigned tile, unsigned lut,
                                             unsigned sC, unsigned col, const f2_t (&ax)[R / 2],
                                             const f2_t (&ay)[R / 2], const f2_t (&az)[R / 2],
@@ -1392,11 +1392,10 @@ __device__ __forceinline__ void exact_steps(int j0, int j1, unsigned tile, unsig
                                             const Segment& S, long long a0, long long b0,
                                             int a_first, unsigned long long& n_recheck) {
     constexpr int NV = JU * R;
-    constexpr unsigned LUTB = SPANS ? 8 : 16;
-    unsigned b = point_addr<SPANS>(tile, j0);
+    constexpr unsigned LUTB = 16;  // (builds without span jobs)
+    unsigned b = point_addr<false>(tile, j0);
 #pragma unroll 1
-    for (int j = j0; j < j1;
-         b += JU * kPointB + (SPANS && (j & 31) == 32 - JU ? 16u : 0u), j += JU) {
+    for (int j = j0; j < j1; b += JU * kPointB, j += JU) {
         float s[NV];
         chords<R, JU, DIAG>(s, b, ax, ay, az, j, a_first);
         const float m = min_of(s);
@@ -1613,11 +1612,9 @@ __device__ __forceinline__ void tile_pass(unsigned tile, unsigned lut, unsigned 
         }
         return;
     }
-    // pair by pair (diagonal tiles, or span binning off; spans go through
-    // span_item's jobs)
-    exact_steps<NT, R, JU, HM, ROWB, PK::SPANS, DIAG>(j_begin, j_end, tile, lut, sC, col, ax, ay, az,
-                                                      hf, shift, base, top_idx, K, S, a0, b0,
-                                                      a_first, n_recheck);
+    // pair by pair as screened
+    exact_steps<NT, R, JU, HM, ROWB, DIAG>(j_begin, j_end, tile, lut, sC, col, ax, ay, az, hf, shift,
+                                           base, top_idx, K, S, a0, b0, a_first, n_recheck);
 }
 
 // The thread's R A points, R consecutive points of the spatial order (a
@@ -2333,10 +2330,8 @@ __global__ void __launch_bounds__(NT, (R == 8 ? 640 : 384) / NT) k_pairs(const _
         // the part of the B tile that this item takes
         const int part = s_part[n_items & 1], b_len = TB >> lp, b_begin = part * b_len;
         n_tiles += part == 0 ? 1 : 0;
-        // with span binning the tile holds local coordinates (relative to each
-        // chunk's centre), otherwise the FP32 copies
-        bool spans = false;
-        if constexpr (PK::SPANS) spans = p.span && S.b_caps;
+        // with span jobs the tile holds local coordinates (relative to each chunk's
+        // centre), otherwise the FP32 copies
         const unsigned a_tile = smem_addr(smem);
         // two points at a time: three 16-byte stores
         auto stage2 = [&](int j, float x0, float y0, float z0, float x1, float y1, float z1) {
@@ -2345,7 +2340,7 @@ __global__ void __launch_bounds__(NT, (R == 8 ? 640 : 384) / NT) k_pairs(const _
             sts_f2x2(b + 16u, pack2(-z0, -z0), pack2(-x1, -x1));
             sts_f2x2(b + 32u, pack2(-y1, -y1), pack2(-z1, -z1));
         };
-        if (spans) {
+        if constexpr (PK::SPANS) {
             const float* gL = S.bl + J * TB;
             const long long ls = S.bl_stride;
 #pragma unroll 4
@@ -2366,12 +2361,10 @@ __global__ void __launch_bounds__(NT, (R == 8 ? 640 : 384) / NT) k_pairs(const _
             }
         }
         if (tid < NW) s_units[tid] = NW == 1 ? 0 : (part * UPS) >> lp;
-        if constexpr (PK::SPANS) {
-            if (spans)
-                settle_chunks<NT, R, JU, HM, ST>(smem_addr(s_units + NW), smem_addr(sLut),
-                                                 smem_addr(sC), smem_addr(hist), p, S, I, J,
-                                                 S.is_auto && I == J, part, lp, smem_addr(s_stat));
-        }
+        if constexpr (PK::SPANS)
+            settle_chunks<NT, R, JU, HM, ST>(smem_addr(s_units + NW), smem_addr(sLut), smem_addr(sC),
+                                             smem_addr(hist), p, S, I, J, S.is_auto && I == J, part,
+                                             lp, smem_addr(s_stat));
         __syncthreads();  // B tile staged, unit counters reset
         const unsigned a_lut = smem_addr(sLut), a_cap = smem_addr(sCap), a_group = smem_addr(sGroup), a_band = smem_addr(sBand),
                        a_hist = smem_addr(hist), a_c = smem_addr(sC);
@@ -2382,42 +2375,40 @@ __global__ void __launch_bounds__(NT, (R == 8 ? 640 : 384) / NT) k_pairs(const _
         // 15.3 -> 12.3 ms).  A warp takes the units of its own sub-tile first, then
         // those left of the others, so the warps of the block finish the item
         // together whatever the mix of cheap and costly units.
-        const int lane = tid & 31, warp = tid >> 5;
         const bool diag = S.is_auto && I == J;
         if constexpr (PK::SPANS) {
-            if (spans)
-                span_item<NT, R, JU, HM, ST>(smem_addr(s_units), smem_addr(s_ring),
-                                         smem_addr(s_IJ[n_items & 1]), a_tile, a_lut, a_cap, a_group, a_band, a_c,
-                                         a_hist, p, S, diag, part, lp, smem_addr(s_stat));
-        }
-        int cur = -1;
-        f2_t ax[R / 2], ay[R / 2], az[R / 2];
+            span_item<NT, R, JU, HM, ST>(smem_addr(s_units), smem_addr(s_ring),
+                                         smem_addr(s_IJ[n_items & 1]), a_tile, a_lut, a_cap, a_group,
+                                         a_band, a_c, a_hist, p, S, diag, part, lp, smem_addr(s_stat));
+        } else {
+            const int lane = tid & 31, warp = tid >> 5;
+            int cur = -1;
+            f2_t ax[R / 2], ay[R / 2], az[R / 2];
 #pragma unroll 1
-        for (int k = 0; k < NW && !spans; ++k) {
-            const int sub = (warp + k) % NW;
+            for (int k = 0; k < NW; ++k) {
+                const int sub = (warp + k) % NW;
 #pragma unroll 1
-            for (;;) {
-                unsigned u = 0;
-                if (lane == 0) u = atomicAdd(&s_units[sub], 1u);
-                u = __shfl_sync(0xffffffffu, u, 0);
-                // (one-warp blocks: the part of the tile as one unit)
-                const int jb = NW == 1 ? b_begin : (int)u * UB;
-                const int je = NW == 1 ? b_begin + b_len : jb + UB;
-                if (NW == 1 ? u != 0u : jb >= b_begin + b_len) break;
-                const int a_first = sub * SA + lane * R;
-                if (diag && je <= sub * SA) continue;  // every pair has i >= j
-                if (sub != cur) {
-                    load_group<R>(S.a32 + I * TA + a_first, ax, ay, az);
-                    cur = sub;
+                for (;;) {
+                    unsigned u = 0;
+                    if (lane == 0) u = atomicAdd(&s_units[sub], 1u);
+                    u = __shfl_sync(0xffffffffu, u, 0);
+                    // (one-warp blocks: the part of the tile as one unit)
+                    const int jb = NW == 1 ? b_begin : (int)u * UB;
+                    const int je = NW == 1 ? b_begin + b_len : jb + UB;
+                    if (NW == 1 ? u != 0u : jb >= b_begin + b_len) break;
+                    const int a_first = sub * SA + lane * R;
+                    if (diag && je <= sub * SA) continue;  // every pair has i >= j
+                    if (sub != cur) {
+                        load_group<R>(S.a32 + I * TA + a_first, ax, ay, az);
+                        cur = sub;
+                    }
+                    if (diag && jb < (sub + 1) * SA)
+                        tile_pass<NT, R, JU, HM, DEF, true>(a_tile, a_lut, a_c, a_hist, ax, ay, az, p,
+                                                            S, I, J, a_first, jb, je, n_recheck);
+                    else
+                        tile_pass<NT, R, JU, HM, DEF, false>(a_tile, a_lut, a_c, a_hist, ax, ay, az, p,
+                                                             S, I, J, a_first, jb, je, n_recheck);
                 }
-                if (diag && jb < (sub + 1) * SA)
-                    tile_pass<NT, R, JU, HM, DEF, true>(a_tile, a_lut, a_c, a_hist, ax, ay,
-                                                        az, p, S, I, J, a_first, jb, je,
-                                                        n_recheck);
-                else
-                    tile_pass<NT, R, JU, HM, DEF, false>(a_tile, a_lut, a_c, a_hist, ax, ay,
-                                                         az, p, S, I, J, a_first, jb, je,
-                                                         n_recheck);
             }
         }
         ++n_items;
@@ -3031,7 +3022,6 @@ PairParams make_params(const Variant* v, const BinTable& tab, const Segment* seg
                                                             1ull << 30);
     prm.cursor = cursor;
     prm.stats = stats;
-    prm.span = 1;
     std::memcpy(&prm.tab, &tab, sizeof(tab));
     return prm;
 }
@@ -3144,7 +3134,6 @@ static int count_impl(const double* ca, long long n_a, const double* cb, long lo
         seg.item_list = list;
         PairParams prm = make_params(v, tab, &seg, nullptr, 0, 0, n_items, cursor, stats);
         prm.n_items_dev = n_list;
-        prm.span = !(tune && tune->span_bins == 2);
         prm.done = cursor + 2;
         rc = launch_pairs(v, prm, grid, smem, st);
     }
@@ -3387,7 +3376,6 @@ static int count_wtheta_impl(const double* cd, long long nd, const double* cr, l
             PairParams prm = make_params(v, tab, nullptr, d_segs, n_segs, 0, total_items, cursor,
                                          stats);
             if (cull) prm.n_items_dev = n_kept;
-            prm.span = !(tune && tune->span_bins == 2);
             prm.done = cursor + 2;
             rc = launch_pairs(v, prm, grid, smem, st);
         } else if (!rc) {
@@ -3536,7 +3524,8 @@ static int count_xyz_noalloc_impl(const double* ca, long long n_a, const double*
     }
     wtheta_tune fixed = {128, 8, 0, 0, 0, 0, 2, 2};  // the tile of WTHETA_NOALLOC_TILE points
     const Variant* v = pick_variant(&fixed, K, tab.n_lut, di.max_smem_optin);
-    if (!v || (long long)v->nt * v->r != T) return WTHETA_EINVAL;
+    // (without spheres: only a build without span jobs)
+    if (!v || (long long)v->nt * v->r != T || has_spans(v)) return WTHETA_EINVAL;
 
     unsigned long long* cursor = (unsigned long long*)base;
     float4* a32 = (float4*)(base + 256);
@@ -3808,7 +3797,6 @@ static int launch_batch_pairs(wtheta_plan* P, const Variant* v, long long item_b
                               unsigned long long* stats = nullptr) {
     PairParams prm = make_params(v, P->tab, nullptr, P->d_segs, P->n_segs, item_begin,
                                  n_items, P->d_cursor, stats);
-    prm.span = P->tune.span_bins != 2;
     prm.n_items_dev = n_items_dev;
     pair_kernel(v, prm)<<<grid, v->nt, smem, st>>>(prm);
     count_launch();

@@ -110,8 +110,6 @@ struct PairParams {
     unsigned long long* cursor;
     unsigned long long* done;     // if set (zeroed): the last block to finish fills the overflow slots
     unsigned long long* stats;    // WTHETA_NSTATS or null
-    int span;                // settle (A group, B chunk) spans without a lookup per pair
-    int pad_;
     BinTable tab;
 };
 
@@ -122,6 +120,10 @@ struct Variant {
     void (*kernel_fast)(PairParams);  // the build launched without statistics
     size_t (*smem)(int, int);
 };
+// def: 0 in-range pairs binned as they are screened, 1 deferred, 2 as 0 without span
+// code.  A build with span jobs takes every count by spans and needs the spheres and
+// local coordinates of both catalogues.
+inline bool has_spans(const Variant* v) { return v->def == 0 && v->hm != kHistWarp; }
 
 struct DeviceInfo {
     int sm_count = 0;

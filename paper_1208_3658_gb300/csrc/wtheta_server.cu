@@ -89,7 +89,6 @@ struct wtheta_server {
     const Variant* v = nullptr;
     size_t smem = 0;
     int grid = 0;
-    int span = 1;              // settle (A group, B chunk) spans without a lookup per pair
     int cull = 1;              // skip tile pairs wholly beyond the top edge
     double theta_top = 0.0;    // top edge, radians
     int sm_count = 0;
@@ -351,7 +350,6 @@ bool launch_round(wtheta_server* S, Round& R) {
         const int grid = (int)std::min<long long>(S->grid, items << S->v->max_parts);
         PairParams prm = make_params(S->v, S->tab, nullptr, R.d_segs, n, 0, items, R.d_cursor,
                                      nullptr);
-        prm.span = S->span;
         if (!rc) rc = launch_pairs(S->v, prm, grid, S->smem, R.st);
         ++S->kernels;
     }
@@ -465,7 +463,6 @@ int server_create(const double* edges, int K, size_t budget, int max_active,
         S->max_active = max_active ? max_active : 1024;
         S->sm_count = di.sm_count;
         S->v = pick_variant(tune, K, S->tab.n_lut, di.max_smem_optin);
-        S->span = !(tune && tune->span_bins == 2);
         S->cull = !(tune && tune->skip_far == 2) && edges[K] < 180.0;
         S->theta_top = edges[K] * (3.14159265358979323846 / 180.0);
         if (!S->v) rc = WTHETA_EINVAL;
