@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(kSortThreads) k_digit_scatter(
 // Bound by the latency of a launch and of about six dependent memory accesses:
 // a w(theta) of 1k + 1k points took 96 us instead of 117 with three launches a
 // pass, one of 10k + 10k 271 us instead of 300 (with the host copies), in the build
-// that it came with (77 and 227 us now).
+// that it came with (75 and 217 us now).
 constexpr int kSmallThreads = 1024;
 constexpr long long kSmallSort = 65536;
 __global__ void __launch_bounds__(kSmallThreads) k_small_pass(
@@ -1426,18 +1426,19 @@ __device__ __forceinline__ void exact_steps(int j0, int j1, unsigned tile, unsig
 //            beyond 60 degrees);
 //   -1       more edges, or padding: bin pair by pair.
 // Two edges cost a job about a quarter of the table's lookups and shared
-// atomics for its 256 pairs.  kMaxEdges 4, 6, 8 in the build that it came with: 256
-// log bins to 20 deg (200k + 200k points) 8.70, 8.91, 9.39 ms; 24 bins (30k x 48k)
-// 513, 509, 517 us; 32 bins (1M + 1M) 36.67, 36.72, 36.81 ms.
+// atomics for its 256 pairs.  kMaxEdges 4, 6, 8: 256 log bins to 20 deg (200k + 200k
+// points) 7.80, 7.67, 7.87 ms; 24 bins (30k x 48k) 446, 444, 444 us with the host's
+// part; 32 bins (1M + 1M) 29.26, 29.26, 29.29 ms; 60 linear bins to 60 deg (100k +
+// 100k) 7.14, 7.26, 7.32 ms.
 // Beyond 60 degrees the line is 16, because values in a bucket with several edges
 // are recounted out of line, one by one, and linear bins have such buckets there
 // (the table's buckets are steps of the logarithm).  The span's ends do not tell:
 // 36 linear bins have only one, just below 180 deg, and the spans across it end in
-// the next.  Now, 6 everywhere / a line of 16 where an end meets such a bucket / this
-// / 16 everywhere, full sky: 36 bins (100k + 100k) 12.8, 12.7, 8.7, 8.7 ms (4.7e7
-// values recounted with 6, 1.1e6 with this), 256 bins (100k + 100k) 203, 166, 134,
-// 135, 90 bins (300k + 300k) 182, 162, 113, 113, 20 bins from 60 deg 6.4, 6.4, 6.6,
-// 6.6; the 256 log bins to 20 deg 8.3, 8.3, 8.3, 9.9.
+// the next.  6 everywhere / a line of 16 where an end meets such a bucket / this / 16
+// everywhere, full sky: 36 bins (100k + 100k) 12.3, 12.5, 8.2, 8.2 ms (4.7e7 values
+// recounted with 6, 1.1e6 with this), 256 bins (100k + 100k) 203, 166, 134, 134, 90
+// bins (300k + 300k) 175, 154, 104, 104, 20 bins from 60 deg 6.0, 6.0, 6.2, 6.2; the
+// 256 log bins to 20 deg 7.6, 7.7, 7.7, 9.0.
 constexpr int kMaxEdges = 6, kMaxEdgesFar = 16;
 __device__ __forceinline__ int span_edges(float4 ga, float4 gb, unsigned lut, unsigned c64,
                                           int shift, int base, int top_idx, int K, unsigned h_top,
@@ -2556,18 +2557,18 @@ int device_info(DeviceInfo* out) {
 // points (one warp) up to 4096, of 512 points (64 threads) up to 32768, else of
 // 1024.  w(theta) of n + n points on a 10 deg patch (16 bins) / a 15 deg patch (24) /
 // a 60 deg cap (32), with 32, 64, 128 threads, us per call on the device:
-//    1k  106 113 135 / 111 118 133 / 104 110 128
-//    4k  118 125 145 / 125 125 147 / 116 125 138
-//    6k  138 138 144 / 152 147 152 / 135 133 142
-//    8k  163 152 155 / 181 162 174 / 151 143 150
-//   16k  262 246 249 / 300 279 288 / 221 213 218
-//   32k  455 461 486 / 578 569 609 / 340 345 379
-//   48k  751 724 728 / 996 935 940 / 489 496 517
-//   64k 1090 1015 1024 / 1476 1357 1368 / 657 636 669
-// and cross counts n x n: 4k 104 117 138 / 109 115 138 / 105 110 134, 32k 318 327 327 /
-// 388 381 374 / 237 240 264, 48k 491 508 505 / 617 628 615 / 340 347 362.  So 32
-// threads up to about 5k; from there 64, clearly up to 32k; at 48k and 64k the last
-// two lie within 2% on the patches (64 ahead by 4% on the cap).
+//    1k  101 107 125 / 106 111 125 /  99 105 122
+//    4k  112 118 136 / 118 119 136 / 109 121 129
+//    8k  143 142 146 / 158 151 164 / 135 133 140
+//   16k  241 230 234 / 272 265 271 / 200 198 204
+//   32k  421 441 457 / 531 541 575 / 304 326 357
+//   48k  686 694 700 / 899 892 898 / 454 473 492
+//   64k  979 970 981 / 1319 1288 1300 / 603 605 641
+// and cross counts n x n: 4k 99 112 129 / 104 109 129 / 98 103 125, 32k 284 306 305 /
+// 355 359 350 / 213 226 244, 48k 460 483 474 / 571 597 577 / 315 330 343.  The lines
+// were drawn with 32 and 64 threads level from 5k on and 64 ahead of 128 up to 32k
+// (32k 455 461 486 on the 10 deg patch); since the span builds spill nothing, 32
+// threads are ahead by up to 7% at 32k and level or ahead to 64k.
 const Variant* pick_for_size(const wtheta_tune* tune, long long n_max, int K, int n_lut,
                              int max_smem) {
     if (!tune && n_max <= 32768) {
